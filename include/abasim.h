@@ -304,8 +304,8 @@ int sim_set_tape_space(sim_handle* h, int32_t space);
  * state and input streams on chip, 2 tape on chip, 3 the pipelined two-warp
  * kernels, 4 the world-aligned kernels with the tape on chip, 5 the world-aligned
  * kernels with the tape in global memory, 6 / 7 the pipelined world-aligned adjoint
- * with its tapes on chip / in global memory.  Either pointer may be NULL.  No
- * device work. */
+ * with its tapes on chip / in global memory, 8 - 11 the modes 4 - 7 for a model with
+ * a free joint (AUTO only).  Either pointer may be NULL.  No device work. */
 int sim_last_storage(const sim_handle* h, int32_t* rollout_mode, int32_t* backward_mode);
 
 /* Prefetch distance of the world-aligned kernels when their tape is in global

@@ -211,12 +211,14 @@ class Simulator:
         self._check(lib.sim_set_tape_space(self._h, code), "sim_set_tape_space")
 
     STORAGE = ("global", "hybrid", "shared", "pipelined", "aligned_shared", "aligned_global",
-               "aligned_pipelined_shared", "aligned_pipelined_global")
+               "aligned_pipelined_shared", "aligned_pipelined_global", "floating_shared", "floating_global",
+               "floating_pipelined_shared", "floating_pipelined_global")
 
     def last_storage(self):
         """(rollout, backward) storage modes of the last launches: 'global', 'hybrid',
-        'shared', 'pipelined', or the world-aligned kernels' 'aligned_shared' /
-        'aligned_global'."""
+        'shared', 'pipelined', the world-aligned kernels' 'aligned_shared' /
+        'aligned_global' and 'aligned_pipelined_shared' / 'aligned_pipelined_global',
+        or 'floating_...' where they run a model with a floating base."""
         f, b = ctypes.c_int32(), ctypes.c_int32()
         self._check(lib.sim_last_storage(self._h, ctypes.byref(f), ctypes.byref(b)), "sim_last_storage")
         return self.STORAGE[f.value], self.STORAGE[b.value]

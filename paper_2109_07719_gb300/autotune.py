@@ -102,7 +102,7 @@ def autotune(sim, q0, qd0, T_probe: int = 16, reps: int = 3, k: int = 1, use_cac
             continue                                   # the model cannot run on these kernels
         if cand[2] == 2 and "pipelined" not in sim.last_storage():
             continue                                   # ran one-lane in a direction: not this candidate
-        if cand[2] == 5 and not any(s.startswith(("pipelined", "aligned")) for s in sim.last_storage()):
+        if cand[2] == 5 and not any(s.startswith(("pipelined", "aligned", "floating")) for s in sim.last_storage()):
             continue                                   # the automatic choice was the one-warp family
         times[cand] = t
     best = choose(times)

@@ -601,6 +601,23 @@ SD void chain_bias_in(const Sys<T, PT>& s, Col<T> q, Col<T> qd, Col<const T> tau
   }
 }
 
+// The free joint's position step for the body velocity nu: p' = p + dt R(quat) nu_v,
+// quat' = normalize(quat + dt/2 quat (x) (nu_w, 0)); x = (p, quat).
+template <class A> SD void free_advance(A* x, const A* nu, A dt) {
+  const A qt[4] = {x[3], x[4], x[5], x[6]};
+  const V3<A> dp = mul(quat_R(qt[0], qt[1], qt[2], qt[3]), V3<A>{nu[3], nu[4], nu[5]});
+  x[0] = x[0] + dt * dp.x;
+  x[1] = x[1] + dt * dp.y;
+  x[2] = x[2] + dt * dp.z;
+  const A wq[4] = {nu[0], nu[1], nu[2], A(0)};
+  A r[4];
+  quat_mul(qt, wq, r);
+  A raw[4];
+  for (int i = 0; i < 4; ++i) raw[i] = qt[i] + A(0.5) * dt * r[i];
+  const A n = sqrt_t(raw[0] * raw[0] + raw[1] * raw[1] + raw[2] * raw[2] + raw[3] * raw[3]);
+  for (int i = 0; i < 4; ++i) x[3 + i] = raw[i] / n;
+}
+
 // Integrates x -> x' in place from the qdd on the tape, plus the contact
 // velocity change C_DV of the contact tape ct when given.  The state columns may
 // be wider than the step's scalar (A = double with T = float: the running state
@@ -625,18 +642,10 @@ SD void integrate_in(const Sys<T, PT, TL, AL>& s, Col<A> q, Col<A> qd, A dt, int
         qd[vo + i] = v1;
         nu[i] = integ == I_SEMI_IMPLICIT ? v1 : v0;
       }
-      A qt[4] = {q[qo + 3], q[qo + 4], q[qo + 5], q[qo + 6]};
-      V3<A> dp = mul(quat_R(qt[0], qt[1], qt[2], qt[3]), V3<A>{nu[3], nu[4], nu[5]});
-      q[qo] = q[qo] + dt * dp.x;
-      q[qo + 1] = q[qo + 1] + dt * dp.y;
-      q[qo + 2] = q[qo + 2] + dt * dp.z;
-      A wq[4] = {nu[0], nu[1], nu[2], A(0)};
-      A r[4];
-      quat_mul(qt, wq, r);
-      A raw[4];
-      for (int i = 0; i < 4; ++i) raw[i] = qt[i] + A(0.5) * dt * r[i];
-      A n = sqrt_t(raw[0] * raw[0] + raw[1] * raw[1] + raw[2] * raw[2] + raw[3] * raw[3]);
-      for (int i = 0; i < 4; ++i) q[qo + 3 + i] = raw[i] / n;
+      A x[7];
+      for (int i = 0; i < 7; ++i) x[i] = q[qo + i];
+      free_advance(x, nu, dt);
+      for (int i = 0; i < 7; ++i) q[qo + i] = x[i];
     }
   }
 }
@@ -646,35 +655,15 @@ SD void integrate(const Sys<T, PT, TL, AL>& s, Col<T> q, Col<T> qd, T dt, int in
 }
 
 // ------------------------------------------------------------------ adjoint
-// Integrator adjoint of one link (folded into the pass-3 adjoint loop): turns the
-// adjoint of x^{k+1} held in (gq, gqd) into the direct part of the adjoint of x^k
-// for this link's coordinates and returns the adjoint of its qdd in qddb[0..nv).
-template <class T, class PT, int TL, int AL>
-SD void integrator_adjoint(const Sys<T, PT, TL, AL>& s, int l, int jt, int qo, int vo, Col<const T> q,
-                           Col<const T> qd, Col<T> gq, Col<T> gqd, T dt, int integ, T* qddb,
-                           const T* ct = nullptr) {
+// Adjoint of a free joint's integration from the quaternion qt with the velocity nu of
+// its position step: turns the adjoint of x^{k+1} held in (gq, gqd) into the direct part
+// of that of x^k and returns the adjoint of qdd in qddb[0..6).
+template <class T>
+SD void free_integrator_adjoint(const T* qt, const T* nu, Col<T> gq, Col<T> gqd, int qo, int vo, T dt, int integ,
+                                T* qddb) {
   const T half = T(0.5);
-  if (jt == J_REVOLUTE) {
-    const T qb = gq[qo], vb = gqd[vo];
-    if (integ == I_SEMI_IMPLICIT) {
-      const T vt = vb + dt * qb;
-      gqd[vo] = vt;
-      qddb[0] = dt * vt;
-    } else {
-      gqd[vo] = vb + dt * qb;
-      qddb[0] = dt * vb;
-    }
-    return;
-  }
-  T nu[6], nub[6];
-  for (int i = 0; i < 6; ++i) {
-    const T v0 = qd[vo + i];
-    T v1 = v0 + dt * s.tp(l, T_QDD + i);
-    if (ct) v1 += ctr(ct, l, C_DV + i);
-    nu[i] = integ == I_SEMI_IMPLICIT ? v1 : v0;
-    nub[i] = gqd[vo + i];
-  }
-  const T qt[4] = {q[qo + 3], q[qo + 4], q[qo + 5], q[qo + 6]};
+  T nub[6];
+  for (int i = 0; i < 6; ++i) nub[i] = gqd[vo + i];
   const T wq[4] = {nu[0], nu[1], nu[2], T(0)};
   T r[4], raw[4];
   quat_mul(qt, wq, r);
@@ -717,6 +706,36 @@ SD void integrator_adjoint(const Sys<T, PT, TL, AL>& s, int l, int jt, int qo, i
       qddb[i] = dt * nub[i];
     }
   }
+}
+
+// Integrator adjoint of one link (folded into the pass-3 adjoint loop): turns the
+// adjoint of x^{k+1} held in (gq, gqd) into the direct part of the adjoint of x^k
+// for this link's coordinates and returns the adjoint of its qdd in qddb[0..nv).
+template <class T, class PT, int TL, int AL>
+SD void integrator_adjoint(const Sys<T, PT, TL, AL>& s, int l, int jt, int qo, int vo, Col<const T> q,
+                           Col<const T> qd, Col<T> gq, Col<T> gqd, T dt, int integ, T* qddb,
+                           const T* ct = nullptr) {
+  if (jt == J_REVOLUTE) {
+    const T qb = gq[qo], vb = gqd[vo];
+    if (integ == I_SEMI_IMPLICIT) {
+      const T vt = vb + dt * qb;
+      gqd[vo] = vt;
+      qddb[0] = dt * vt;
+    } else {
+      gqd[vo] = vb + dt * qb;
+      qddb[0] = dt * vb;
+    }
+    return;
+  }
+  T nu[6];
+  for (int i = 0; i < 6; ++i) {
+    const T v0 = qd[vo + i];
+    T v1 = v0 + dt * s.tp(l, T_QDD + i);
+    if (ct) v1 += ctr(ct, l, C_DV + i);
+    nu[i] = integ == I_SEMI_IMPLICIT ? v1 : v0;
+  }
+  const T qt[4] = {q[qo + 3], q[qo + 4], q[qo + 5], q[qo + 6]};
+  free_integrator_adjoint(qt, nu, gq, gqd, qo, vo, dt, integ, qddb);
 }
 
 // Requires aba_forward(q, qd, tau) to have filled the tape.  On entry gq, gqd hold

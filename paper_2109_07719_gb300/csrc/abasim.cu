@@ -368,6 +368,7 @@ int sim_create(const sim_model_desc* d, sim_handle** out) {
   }
   cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
   h->all_chains = !any_contact;
+  h->unconstrained = !any_contact;
   h->all_revolute = !any_contact;
   for (int i = 0; i < h->L_total && h->all_revolute; ++i)
     if (d->joint_type[i] != SIM_REVOLUTE) h->all_revolute = false;
@@ -399,9 +400,9 @@ int sim_create(const sim_model_desc* d, sim_handle** out) {
   if (rc == SIM_OK) rc = alloc(&h->tape, (size_t)maxL * NTAPE * Bpad * h->scalar, "tape");
   if (rc == SIM_OK) rc = alloc(&h->adj, (size_t)maxL * NADJ * Bpad * h->scalar, "adjoint tape");
   if (rc == SIM_OK) rc = alloc(&h->gm_acc, (size_t)maxL * B * h->scalar, "mass-gradient buffer");
-  if (rc == SIM_OK && h->all_revolute)
-    rc = alloc(&h->wtape2, (size_t)maxL * NWT * Bpad * h->scalar, "second world-aligned tape");
-  if (rc == SIM_OK && h->all_revolute && h->wdepth > 0)
+  if (rc == SIM_OK && h->unconstrained)
+    rc = alloc(&h->wtape2, ((size_t)maxL * NWT + NWF) * Bpad * h->scalar, "second world-aligned tape");
+  if (rc == SIM_OK && h->unconstrained && h->wdepth > 0)
     rc = alloc(&h->wstk, (size_t)2 * h->wdepth * WSW * Bpad * h->scalar, "world-aligned stacks");
   if (rc == SIM_OK) rc = alloc((void**)&h->status, B * sizeof(int), "status");
   if (rc == SIM_OK) rc = alloc((void**)&h->sys_of_slot, B * sizeof(int), "slot order");

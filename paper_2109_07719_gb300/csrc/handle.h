@@ -30,7 +30,7 @@ struct sim_handle {
   int* nqv = nullptr;        // [B]  nq | nv << 16
   void* tape = nullptr;      // [maxL][NTAPE][B] scalar
   void* adj = nullptr;       // [maxL][NADJ][B] scalar
-  void* wtape2 = nullptr;    // [maxL][NWT][B] scalar: the pipelined world-aligned adjoint's second tape
+  void* wtape2 = nullptr;    // [maxL * NWT + NWF][B] scalar: the pipelined world-aligned adjoint's second tape
   void* wstk = nullptr;      // [2][wdepth][WSW][B] scalar: the world-aligned passes' stacks of parent values
   int wdepth = 0;            // entries a system's stack holds at most (depth-first nesting of its branchings)
   void* gm_acc = nullptr;    // [maxL][B] scalar
@@ -49,7 +49,8 @@ struct sim_handle {
   int last_storage = 0, last_storage_bwd = 0;
   int sms = 0;
   bool all_chains = false;   // every system a serial chain of revolute joints (the pipelined adjoint)
-  bool all_revolute = false; // every joint revolute and no contact spheres or limits (the world-aligned kernels)
+  bool all_revolute = false; // every joint revolute and no contact spheres or limits
+  bool unconstrained = false; // no contact spheres or limits (the world-aligned kernels; FR ones unless all_revolute)
   bool state64 = false;      // sim_rollout accumulates the state in FP64 (SIM_FP32_D64 only)
   void* x64 = nullptr;       // [nq_max + nv_max][B] double: that state
   std::vector<int> h_sys_of_slot;

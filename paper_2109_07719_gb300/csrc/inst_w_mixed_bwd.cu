@@ -6,10 +6,11 @@ namespace abasim {
 namespace host {
 
 template <class T, class DT>
-BackwardKernel<T> wbackward_kernel(bool onchip) {
-  return onchip ? k_wbackward<T, DT, true> : k_wbackward<T, DT, false>;
+BackwardKernel<T> wbackward_kernel(bool onchip, bool fr) {
+  if (fr) return onchip ? k_wbackward<T, DT, true, true> : k_wbackward<T, DT, false, true>;
+  return onchip ? k_wbackward<T, DT, true, false> : k_wbackward<T, DT, false, false>;
 }
-template BackwardKernel<float> wbackward_kernel<float, double>(bool);
+template BackwardKernel<float> wbackward_kernel<float, double>(bool, bool);
 
 }  // namespace host
 }  // namespace abasim

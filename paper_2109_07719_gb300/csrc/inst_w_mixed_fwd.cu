@@ -6,10 +6,11 @@ namespace abasim {
 namespace host {
 
 template <class T, class DT>
-RolloutKernel<T> wrollout_kernel(bool onchip) {
-  return onchip ? k_wrollout<T, DT, true> : k_wrollout<T, DT, false>;
+RolloutKernel<T> wrollout_kernel(bool onchip, bool fr) {
+  if (fr) return onchip ? k_wrollout<T, DT, true, true> : k_wrollout<T, DT, false, true>;
+  return onchip ? k_wrollout<T, DT, true, false> : k_wrollout<T, DT, false, false>;
 }
-template RolloutKernel<float> wrollout_kernel<float, double>(bool);
+template RolloutKernel<float> wrollout_kernel<float, double>(bool, bool);
 
 }  // namespace host
 }  // namespace abasim

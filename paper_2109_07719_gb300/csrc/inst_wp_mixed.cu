@@ -6,10 +6,11 @@ namespace abasim {
 namespace host {
 
 template <class T, class DT>
-BackwardKernel<T> wbackward_pipe_kernel(bool onchip) {
-  return onchip ? k_wbackward_pipe<T, DT, true> : k_wbackward_pipe<T, DT, false>;
+BackwardKernel<T> wbackward_pipe_kernel(bool onchip, bool fr) {
+  if (fr) return onchip ? k_wbackward_pipe<T, DT, true, true> : k_wbackward_pipe<T, DT, false, true>;
+  return onchip ? k_wbackward_pipe<T, DT, true, false> : k_wbackward_pipe<T, DT, false, false>;
 }
-template BackwardKernel<float> wbackward_pipe_kernel<float, double>(bool);
+template BackwardKernel<float> wbackward_pipe_kernel<float, double>(bool, bool);
 
 }  // namespace host
 }  // namespace abasim

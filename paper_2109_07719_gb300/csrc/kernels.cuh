@@ -773,11 +773,11 @@ BackwardKernel<T> backward_pipe_kernel();
 // The world-aligned kernels (tape on chip or in global memory), instantiated in
 // their own units.
 template <class T, class DT>
-RolloutKernel<T> wrollout_kernel(bool onchip);
+RolloutKernel<T> wrollout_kernel(bool onchip, bool fr);
 template <class T, class DT>
-BackwardKernel<T> wbackward_kernel(bool onchip);
+BackwardKernel<T> wbackward_kernel(bool onchip, bool fr);
 template <class T, class DT>
-BackwardKernel<T> wbackward_pipe_kernel(bool onchip);
+BackwardKernel<T> wbackward_pipe_kernel(bool onchip, bool fr);
 
 // One step with tangents: the state, torque and tape are dual numbers staged in
 // the caller's workspace [tile][...][lane]; model constants stay plain.
@@ -930,8 +930,9 @@ int choose_w(sim_handle* h, K k_on, K k_off, bool bwd, bool* onchip, size_t* byt
   if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory limit query");
   const int tiles = h->block / LANES;
   const int nx = h->nq_max + h->nv_max;
-  const size_t need_on = (size_t)tiles * w_smem_per_tile(h->maxL, nx, h->nv_max, bwd, true, h->wdepth * WSW) * LANES * sizeof(T);
-  const size_t need_off = (size_t)tiles * w_smem_per_tile(h->maxL, nx, h->nv_max, bwd, false, 0) * LANES * sizeof(T);
+  const bool fr = !h->all_revolute;
+  const size_t need_on = (size_t)tiles * w_smem_per_tile(h->maxL, nx, h->nv_max, bwd, true, h->wdepth * WSW, fr) * LANES * sizeof(T);
+  const size_t need_off = (size_t)tiles * w_smem_per_tile(h->maxL, nx, h->nv_max, bwd, false, 0, fr) * LANES * sizeof(T);
   if (need_off > (size_t)limit) return fail(h, SIM_EUNSUPPORTED, "the working state does not fit in shared memory");
   e = cudaFuncSetAttribute((const void*)k_off, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need_off);
   if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory opt-in");
@@ -959,24 +960,25 @@ int choose_w(sim_handle* h, K k_on, K k_off, bool bwd, bool* onchip, size_t* byt
   return SIM_OK;
 }
 
-// The world-aligned path applies to models of revolute joints without contact
-// spheres or limits whose state and input streams fit a block's shared memory,
-// under SIM_TAPE_ALIGNED, or under SIM_TAPE_AUTO unless the link-frame two-warp
-// kernels apply and run faster: the pipelined rollout of serial chains short
-// enough for its on-chip tapes, and the link-frame pipelined adjoint of such
-// chains when the world-aligned one's two tapes do not fit a block or the
-// pivots are FP64 (7-DOF chains, FP32, per 1000-step rollout: world-aligned
-// adjoint 10.8 ms against 13.1; with FP64 pivots 40.3 against 34.5).
+// The world-aligned path applies to models without contact spheres or limits whose
+// state and input streams fit a block's shared memory: under SIM_TAPE_ALIGNED (all
+// joints revolute), or under SIM_TAPE_AUTO unless the link-frame two-warp rollout of
+// serial chains applies.  Floating bases take it under SIM_TAPE_AUTO: rollout +
+// adjoint of 8192 quadrupeds over 60 steps (FP32 + FP64 D-solves) 15.6 -> 11.3 ms
+// against the link-frame one-warp kernels, 1024 humanoids over 60 steps (FP32) 10.95
+// -> 4.39 ms.  The link-frame pipelined adjoint of chains is kept with FP64 pivots.
 template <class T, class DT>
 bool use_aligned(const sim_handle* h, bool rollout, int k) {
-  if (!h->all_revolute || (rollout && h->state64)) return false;
+  const bool fr = !h->all_revolute;
+  if (!h->unconstrained || (rollout && h->state64)) return false;
+  if (fr && h->tape_space != SIM_TAPE_AUTO) return false;
   if (h->tape_space != SIM_TAPE_AUTO && h->tape_space != SIM_TAPE_ALIGNED &&
       h->tape_space != SIM_TAPE_ALIGNED_PIPELINED)
     return false;
   int limit = 0;
   if (cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device) != cudaSuccess) return false;
   const int nx = h->nq_max + h->nv_max;
-  const size_t streams = (size_t)(h->block / LANES) * w_smem_per_tile(h->maxL, nx, h->nv_max, !rollout, false, 0) * LANES *
+  const size_t streams = (size_t)(h->block / LANES) * w_smem_per_tile(h->maxL, nx, h->nv_max, !rollout, false, 0, fr) * LANES *
                          sizeof(T);
   if (streams > (size_t)limit) return false;
   if (h->tape_space != SIM_TAPE_AUTO || !h->all_chains) return true;
@@ -985,20 +987,21 @@ bool use_aligned(const sim_handle* h, bool rollout, int k) {
                          (size_t)pipe_smem_per_tile(h->maxL, nx, h->nv_max) * LANES * sizeof(T) <= (size_t)limit;
   if (!link_pipe) return true;
   return sizeof(DT) == sizeof(T) &&
-         (size_t)wpipe_smem_per_tile(h->maxL, nx, h->nv_max, true, h->wdepth * WSW) * LANES * sizeof(T) <= (size_t)limit;
+         (size_t)wpipe_smem_per_tile(h->maxL, nx, h->nv_max, true, h->wdepth * WSW, fr) * LANES * sizeof(T) <= (size_t)limit;
 }
 
 template <class T, class DT>
 int launch_wrollout(sim_handle* h, const void* q0, const void* qd0, const void* tau, int64_t T_, int k, void* ckpt,
                     void* qT, void* qdT, void* traj, void* stream) {
   DevModel<T> m = dev_model<T>(h);
-  const RolloutKernel<T> k_on = wrollout_kernel<T, DT>(true), k_off = wrollout_kernel<T, DT>(false);
+  const RolloutKernel<T> k_on = wrollout_kernel<T, DT>(true, !h->all_revolute),
+                         k_off = wrollout_kernel<T, DT>(false, !h->all_revolute);
   bool onchip = false;
   size_t shm = 0;
   int rc = choose_w<T>(h, k_on, k_off, false, &onchip, &shm);
   if (rc != SIM_OK) return rc;
   const RolloutKernel<T> kern = onchip ? k_on : k_off;
-  h->last_storage = onchip ? 4 : 5;
+  h->last_storage = (h->all_revolute ? 4 : 8) + (onchip ? 0 : 1);
   int grid = 0;
   rc = launch_shape(h, kern, &grid, &m.persistent, shm, stream);
   if (rc != SIM_OK) return rc;
@@ -1019,12 +1022,13 @@ int launch_wbackward_pipe(sim_handle* h, const void* ckpt, const void* tau, int6
   cudaError_t e = cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
   if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory limit query");
   const int nx = h->nq_max + h->nv_max;
-  const size_t need_on = (size_t)wpipe_smem_per_tile(h->maxL, nx, h->nv_max, true, h->wdepth * WSW) * LANES * sizeof(T);
-  const size_t need_off = (size_t)wpipe_smem_per_tile(h->maxL, nx, h->nv_max, false, 0) * LANES * sizeof(T);
-  const bool onchip = need_on <= (size_t)limit;
+  const bool fr = !h->all_revolute;
+  const size_t need_on = (size_t)wpipe_smem_per_tile(h->maxL, nx, h->nv_max, true, h->wdepth * WSW, fr) * LANES * sizeof(T);
+  const size_t need_off = (size_t)wpipe_smem_per_tile(h->maxL, nx, h->nv_max, false, 0, fr) * LANES * sizeof(T);
+  const bool onchip = need_on <= (size_t)limit && (!fr || (h->B + LANES - 1) / LANES <= std::max(1, h->sms));
   if (!onchip && !h->wtape2) return fail(h, SIM_EUNSUPPORTED, "no second tape for the pipelined adjoint");
   const size_t shm = onchip ? need_on : need_off;
-  const BackwardKernel<T> kern = wbackward_pipe_kernel<T, DT>(onchip);
+  const BackwardKernel<T> kern = wbackward_pipe_kernel<T, DT>(onchip, fr);
   e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
   if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory opt-in");
   if (!onchip) {  // shared memory for the blocks an SM holds at once, the rest of the SM's storage as L1
@@ -1032,7 +1036,7 @@ int launch_wbackward_pipe(sim_handle* h, const void* ckpt, const void* tau, int6
                              l1_carveout(h, LANES, shm));
     if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory carve-out");
   }
-  h->last_storage_bwd = onchip ? 6 : 7;
+  h->last_storage_bwd = (fr ? 10 : 6) + (onchip ? 0 : 1);
   int grid = 0;
   int rc = launch_shape(h, kern, &grid, &m.persistent, shm, stream, 2 * LANES, LANES);
   if (rc != SIM_OK) return rc;
@@ -1057,13 +1061,14 @@ int launch_wbackward(sim_handle* h, const void* ckpt, const void* tau, int64_t T
   DevModel<T> m = dev_model<T>(h);
   if (k == 1 && T_ > 0 && h->tape_space != SIM_TAPE_ALIGNED)
     return launch_wbackward_pipe<T, DT>(h, ckpt, tau, T_, gqT, gqdT, gtraj, gq0, gqd0, gtau, gmass, stream);
-  const BackwardKernel<T> k_on = wbackward_kernel<T, DT>(true), k_off = wbackward_kernel<T, DT>(false);
+  const BackwardKernel<T> k_on = wbackward_kernel<T, DT>(true, !h->all_revolute),
+                          k_off = wbackward_kernel<T, DT>(false, !h->all_revolute);
   bool onchip = false;
   size_t shm = 0;
   int rc = choose_w<T>(h, k_on, k_off, true, &onchip, &shm);
   if (rc != SIM_OK) return rc;
   const BackwardKernel<T> kern = onchip ? k_on : k_off;
-  h->last_storage_bwd = onchip ? 4 : 5;
+  h->last_storage_bwd = (h->all_revolute ? 4 : 8) + (onchip ? 0 : 1);
   int grid = 0;
   rc = launch_shape(h, kern, &grid, &m.persistent, shm, stream);
   if (rc != SIM_OK) return rc;

@@ -1,6 +1,5 @@
 // Batched rollout and adjoint kernels of the world-aligned step (wstep.cuh) for
-// models whose joints are all revolute and that have no contact spheres or joint
-// limits.  Thread i handles slot i (systems sorted by link count, longest first);
+// models without contact spheres or joint limits (FR: link 0 may be a free joint).  Thread i handles slot i (systems sorted by link count, longest first);
 // the tape and adjoint record are tile-major, [tile][link][field][lane], in
 // shared memory when a block's tiles fit (ONCHIP), else in the handle's global
 // scratch with the working state and the prefetched input streams still on chip.
@@ -10,6 +9,11 @@
 
 namespace abasim {
 namespace host {
+
+// Scalars per system of one tape: the links' words, then the free root's record.
+__host__ __device__ __forceinline__ long long w_tape_words(int maxL, bool fr) {
+  return (long long)maxL * NWT + (fr ? NWF : 0);
+}
 
 // Scalars per 32-system tile a world-aligned kernel keeps in shared memory: the
 // working state (x for the rollout, the state adjoint and the per-link
@@ -22,10 +26,10 @@ namespace host {
 // footprint leaves most of the SM's L1 to the prefetched tape lines (staging the
 // inputs on chip instead cost more in L1 than it saved in misses).
 __host__ __device__ __forceinline__ long long w_smem_per_tile(int maxL, int nx, int nv, bool bwd, bool onchip,
-                                                              int sd) {
+                                                              int sd, bool fr) {
   const long long state = nx + (bwd ? maxL : 0);
   if (!onchip) return state;
-  return (long long)maxL * (NWT + (bwd ? NWA : 0) + NPRM_W + 1) + sd + state + 2LL * (nv + (bwd ? nx : 0));
+  return w_tape_words(maxL, fr) + (long long)maxL * ((bwd ? NWA : 0) + NPRM_W + 1) + sd + state + 2LL * (nv + (bwd ? nx : 0));
 }
 
 // Stack `which` (0, or 1 for the second warp of the pipelined adjoint) of a tile's
@@ -48,16 +52,16 @@ struct WTile {
   void* stream;
 };
 
-template <class T, bool BWD, bool ONCHIP>
+template <class T, bool BWD, bool ONCHIP, bool FR>
 __device__ __forceinline__ WTile w_tile(int maxL, int nx, int nv, int sd, int lane) {
   const int tb = threadIdx.x / LANES;
   const long long L = maxL;
   T* base =
-      reinterpret_cast<T*>(g_smem) + (long long)tb * w_smem_per_tile(maxL, nx, nv, BWD, ONCHIP, sd) * LANES + lane;
+      reinterpret_cast<T*>(g_smem) + (long long)tb * w_smem_per_tile(maxL, nx, nv, BWD, ONCHIP, sd, FR) * LANES + lane;
   WTile t{};
   if (ONCHIP) {
     t.tape = base;
-    base += L * NWT * LANES;
+    base += w_tape_words(maxL, FR) * LANES;
     t.adj = base;
     if (BWD) base += L * NWA * LANES;
     t.prm = base;
@@ -77,7 +81,7 @@ __device__ __forceinline__ WTile w_tile(int maxL, int nx, int nv, int sd, int la
 
 // The system view of a slot: constants, meta words and tape on chip (copied in
 // here) or in global memory.
-template <class T, bool BWD, bool ONCHIP>
+template <class T, bool BWD, bool ONCHIP, bool FR>
 __device__ __forceinline__ WSys<T> wsys_of(const DevModel<T>& m, int slot) {
   const long long tile = slot / LANES, lane = slot % LANES;
   const long long L = m.maxL;
@@ -85,20 +89,21 @@ __device__ __forceinline__ WSys<T> wsys_of(const DevModel<T>& m, int slot) {
   const int* gmeta = m.meta + tile * L * LANES + lane;
   const int nl = m.nl[slot];
   if (ONCHIP) {
-    const WTile t = w_tile<T, BWD, ONCHIP>(m.maxL, m.nq_max + m.nv_max, m.nv_max, m.wdepth * WSW, (int)lane);
+    const WTile t = w_tile<T, BWD, ONCHIP, FR>(m.maxL, m.nq_max + m.nv_max, m.nv_max, m.wdepth * WSW, (int)lane);
     T* sp = (T*)t.prm;
     constexpr int MS = (int)(sizeof(T) / sizeof(int));
     for (int l = 0; l < nl; ++l) {
       for (int f = 0; f < NPRM_W; ++f) sp[(l * NPRM_W + f) * LANES] = gprm[(l * NPRM + f) * LANES];
       t.meta[l * LANES * MS] = gmeta[l * LANES];
     }
-    return WSys<T>{sp, t.meta, (T*)t.tape, (T*)t.adj, nl, MS, NPRM_W, 0, (T*)t.stk};
+    return WSys<T>{sp, t.meta, (T*)t.tape, (T*)t.adj, nl, MS, NPRM_W, 0, (T*)t.stk, (T*)t.tape + L * NWT * LANES};
   }
-  return WSys<T>{gprm, gmeta, m.tape + tile * L * NWT * LANES + lane, m.adj + tile * L * NWA * LANES + lane, nl, 1,
-                 NPRM, m.pf, w_stack(m, 0, tile, lane)};
+  T* tape = m.tape + tile * w_tape_words(m.maxL, FR) * LANES + lane;
+  return WSys<T>{gprm, gmeta, tape, m.adj + tile * L * NWA * LANES + lane, nl, 1, NPRM, m.pf,
+                 w_stack(m, 0, tile, lane), tape + L * NWT * LANES};
 }
 
-template <class T, class DT, bool ONCHIP>
+template <class T, class DT, bool ONCHIP, bool FR>
 __device__ __forceinline__ void wrollout_one(const DevModel<T>& m, int slot, const T* __restrict__ q0,
                                              const T* __restrict__ qd0, const T* __restrict__ tau, long long Tn,
                                              int k, T* ckpt, T* qT, T* qdT, T* traj) {
@@ -106,8 +111,8 @@ __device__ __forceinline__ void wrollout_one(const DevModel<T>& m, int slot, con
   const long long B = m.B;
   const int nqm = m.nq_max, nvm = m.nv_max, NX = nqm + nvm;
   const V3<T> g{m.g0, m.g1, m.g2};
-  const WSys<T> s = wsys_of<T, false, ONCHIP>(m, slot);
-  const WTile st = w_tile<T, false, ONCHIP>(m.maxL, NX, nvm, m.wdepth * WSW, slot % LANES);
+  const WSys<T> s = wsys_of<T, false, ONCHIP, FR>(m, slot);
+  const WTile st = w_tile<T, false, ONCHIP, FR>(m.maxL, NX, nvm, m.wdepth * WSW, slot % LANES);
   const Col<T> q{(T*)st.state, LANES}, qd{(T*)st.state + nqm * LANES, LANES};
   const int nv = m.nqv[slot] >> 16;
   T* sbuf = (T*)st.stream;  // ONCHIP: [2][nvm][LANES], tau one step ahead
@@ -140,7 +145,7 @@ __device__ __forceinline__ void wrollout_one(const DevModel<T>& m, int slot, con
     } else if (t + 1 < Tn && m.pf > 0) {
       for (int d = 0; d < nv; ++d) pf_line(tau + ((t + 1) * nvm + d) * B + b);
     }
-    wstep_forward<T, DT, false, true>(s, Col<const T>{q.p, LANES}, Col<const T>{qd.p, LANES}, tau_t, g, m.dt,
+    wstep_forward<T, DT, false, true, FR>(s, Col<const T>{q.p, LANES}, Col<const T>{qd.p, LANES}, tau_t, g, m.dt,
                                       m.integ, q, qd);
     if (traj) {
       T* c = traj + (t + 1) * NX * B + b;
@@ -157,7 +162,7 @@ __device__ __forceinline__ void wrollout_one(const DevModel<T>& m, int slot, con
   for (int d = 0; d < nvm; ++d) qdT[d * B + b] = qd[d];
 }
 
-template <class T, class DT, bool ONCHIP>
+template <class T, class DT, bool ONCHIP, bool FR>
 __device__ __forceinline__ void wbackward_one(const DevModel<T>& m, int slot, const T* __restrict__ ckpt,
                                               const T* __restrict__ tau, long long Tn, int k,
                                               const T* __restrict__ gqT, const T* __restrict__ gqdT,
@@ -168,8 +173,8 @@ __device__ __forceinline__ void wbackward_one(const DevModel<T>& m, int slot, co
   const int nqm = m.nq_max, nvm = m.nv_max, NX = nqm + nvm;
   const int nq = m.nqv[slot] & 0xffff, nv = m.nqv[slot] >> 16;
   const V3<T> g{m.g0, m.g1, m.g2};
-  const WSys<T> s = wsys_of<T, true, ONCHIP>(m, slot);
-  const WTile st = w_tile<T, true, ONCHIP>(m.maxL, NX, nvm, m.wdepth * WSW, slot % LANES);
+  const WSys<T> s = wsys_of<T, true, ONCHIP, FR>(m, slot);
+  const WTile st = w_tile<T, true, ONCHIP, FR>(m.maxL, NX, nvm, m.wdepth * WSW, slot % LANES);
   const Col<T> gq{(T*)st.state, LANES}, gqd{(T*)st.state + nqm * LANES, LANES}, gm{(T*)st.gm, LANES};
   T* sbuf = (T*)st.stream;  // [2][NX + nvm][LANES]: x^t and tau^t, one step ahead (k = 1)
   for (int d = 0; d < nqm; ++d) {
@@ -184,9 +189,9 @@ __device__ __forceinline__ void wbackward_one(const DevModel<T>& m, int slot, co
   }
   for (int l = 0; l < s.nl; ++l) gm[l] = T(0);
   auto step_back = [&](long long t, Col<const T> q, Col<const T> qd, Col<const T> tau_t) {
-    wstep_forward<T, DT, true, false>(s, q, qd, tau_t, g, m.dt, m.integ, Col<T>{nullptr, 0}, Col<T>{nullptr, 0});
+    wstep_forward<T, DT, true, false, FR>(s, q, qd, tau_t, g, m.dt, m.integ, Col<T>{nullptr, 0}, Col<T>{nullptr, 0});
     T* gt = gtau + t * nvm * B + b;
-    wstep_adjoint<T, DT>(s, gq, gqd, Col<T>{gt, B}, gm, m.dt, m.integ);
+    wstep_adjoint<T, DT, FR>(s, gq, gqd, Col<T>{gt, B}, gm, m.dt, m.integ, g);
     for (int d = nv; d < nvm; ++d) gt[d * B] = T(0);
     if (gtraj) {
       const T* gx = gtraj + t * NX * B + b;
@@ -235,7 +240,7 @@ __device__ __forceinline__ void wbackward_one(const DevModel<T>& m, int slot, co
         for (long long j = 1; j < t1 - t0; ++j) {
           const T* prev = ring + (j - 1) * NX * B + slot;
           T* cur = ring + j * NX * B + slot;
-          wstep_forward<T, DT, false, true>(s, Col<const T>{prev, B}, Col<const T>{prev + nqm * B, B},
+          wstep_forward<T, DT, false, true, FR>(s, Col<const T>{prev, B}, Col<const T>{prev + nqm * B, B},
                                             Col<const T>{tau + (t0 + j - 1) * nvm * B + b, B}, g, m.dt, m.integ,
                                             Col<T>{cur, B}, Col<T>{cur + nqm * B, B});
         }
@@ -246,11 +251,11 @@ __device__ __forceinline__ void wbackward_one(const DevModel<T>& m, int slot, co
           T* cur = ring + slot;
           x = t == t0 ? xs : cur;
           if (t > t0) {
-            wstep_forward<T, DT, false, true>(s, Col<const T>{xs, B}, Col<const T>{xs + nqm * B, B},
+            wstep_forward<T, DT, false, true, FR>(s, Col<const T>{xs, B}, Col<const T>{xs + nqm * B, B},
                                               Col<const T>{tau + t0 * nvm * B + b, B}, g, m.dt, m.integ,
                                               Col<T>{cur, B}, Col<T>{cur + nqm * B, B});
             for (long long j = t0 + 1; j < t; ++j)
-              wstep_forward<T, DT, false, true>(s, Col<const T>{cur, B}, Col<const T>{cur + nqm * B, B},
+              wstep_forward<T, DT, false, true, FR>(s, Col<const T>{cur, B}, Col<const T>{cur + nqm * B, B},
                                                 Col<const T>{tau + j * nvm * B + b, B}, g, m.dt, m.integ,
                                                 Col<T>{cur, B}, Col<T>{cur + nqm * B, B});
           }
@@ -269,17 +274,17 @@ __device__ __forceinline__ void wbackward_one(const DevModel<T>& m, int slot, co
   for (int l = 0; l < s.nl; ++l) gm_acc[l * B + slot] = gm[l];
 }
 
-template <class T, class DT, bool ONCHIP>
+template <class T, class DT, bool ONCHIP, bool FR>
 __global__ void k_wrollout(DevModel<T> m, const T* __restrict__ q0, const T* __restrict__ qd0,
                            const T* __restrict__ tau, long long Tn, int k, T* ckpt, T* qT, T* qdT, T* traj) {
-  ABASIM_FOR_EACH_SLOT(m, wrollout_one<T, DT, ONCHIP>(m, slot, q0, qd0, tau, Tn, k, ckpt, qT, qdT, traj))
+  ABASIM_FOR_EACH_SLOT(m, wrollout_one<T, DT, ONCHIP, FR>(m, slot, q0, qd0, tau, Tn, k, ckpt, qT, qdT, traj))
 }
 
-template <class T, class DT, bool ONCHIP>
+template <class T, class DT, bool ONCHIP, bool FR>
 __global__ void k_wbackward(DevModel<T> m, const T* __restrict__ ckpt, const T* __restrict__ tau, long long Tn,
                             int k, const T* __restrict__ gqT, const T* __restrict__ gqdT,
                             const T* __restrict__ gtraj, T* gq0, T* gqd0, T* gtau, T* gm_acc, T* ring) {
-  ABASIM_FOR_EACH_SLOT(m, wbackward_one<T, DT, ONCHIP>(m, slot, ckpt, tau, Tn, k, gqT, gqdT, gtraj, gq0, gqd0,
+  ABASIM_FOR_EACH_SLOT(m, wbackward_one<T, DT, ONCHIP, FR>(m, slot, ckpt, tau, Tn, k, gqT, gqdT, gtraj, gq0, gqd0,
                                                        gtau, gm_acc, ring))
 }
 

@@ -1,5 +1,5 @@
 // The pipelined adjoint of the world-aligned step: two warps per 32-system tile,
-// for revolute models without contacts or limits and a checkpoint every step.
+// for models without contacts or limits and a checkpoint every step.
 // With every step's initial state checkpointed, the recompute of step t (Sec. 3.2,
 // Eq. 7: Z^t = G(x^t)) does not depend on the adjoint of step t + 1, so a producer
 // warp recomputes step t into one of two tapes while a consumer warp runs the
@@ -23,13 +23,14 @@ namespace host {
 // two warps' stacks of parent values (sd scalars per system each) and the
 // producer's double-buffered inputs (x^t, tau^t).  Without ONCHIP the producer
 // reads its inputs from global memory, their lines prefetched a step ahead.
-__host__ __device__ __forceinline__ long long wpipe_smem_per_tile(int maxL, int nx, int nv, bool onchip, int sd) {
+__host__ __device__ __forceinline__ long long wpipe_smem_per_tile(int maxL, int nx, int nv, bool onchip, int sd,
+                                                                  bool fr) {
   const long long state = nx + maxL;
   if (!onchip) return state;
-  return (long long)maxL * (2 * NWT + NWA + NPRM_W + 1) + 2LL * sd + state + 2LL * (nx + nv);
+  return 2 * w_tape_words(maxL, fr) + (long long)maxL * (NWA + NPRM_W + 1) + 2LL * sd + state + 2LL * (nx + nv);
 }
 
-template <class T, class DT, bool ONCHIP>
+template <class T, class DT, bool ONCHIP, bool FR>
 __global__ void __launch_bounds__(2 * LANES, 1)
 k_wbackward_pipe(DevModel<T> m, const T* __restrict__ ckpt, const T* __restrict__ tau, long long Tn, int k,
                  const T* __restrict__ gqT, const T* __restrict__ gqdT, const T* __restrict__ gtraj, T* gq0,
@@ -39,6 +40,7 @@ k_wbackward_pipe(DevModel<T> m, const T* __restrict__ ckpt, const T* __restrict_
   const long long B = m.B;
   const int nqm = m.nq_max, nvm = m.nv_max, NX = nqm + nvm;
   const long long L = m.maxL;
+  const long long TW = w_tape_words(m.maxL, FR);
   const V3<T> g{m.g0, m.g1, m.g2};
   constexpr int MS = (int)(sizeof(T) / sizeof(int));
   T* base = reinterpret_cast<T*>(g_smem);
@@ -46,8 +48,8 @@ k_wbackward_pipe(DevModel<T> m, const T* __restrict__ ckpt, const T* __restrict_
   T* s_stk = nullptr;
   const long long sdw = (long long)m.wdepth * WSW;  // stack scalars per system
   if (ONCHIP) {
-    s_tape = base;  // [2][L][NWT][LANES]
-    base += 2 * L * NWT * LANES;
+    s_tape = base;  // [2][tape words][LANES]
+    base += 2 * TW * LANES;
     s_adj = base;
     base += L * NWA * LANES;
     s_prm = base;
@@ -79,16 +81,16 @@ k_wbackward_pipe(DevModel<T> m, const T* __restrict__ ckpt, const T* __restrict_
     }
     __syncthreads();
     auto tape_of = [&](int buf) -> T* {
-      if (ONCHIP) return s_tape + buf * L * NWT * LANES + lane;
-      return (buf ? tape2 : m.tape) + (long long)unit * L * NWT * LANES + lane;
+      if (ONCHIP) return s_tape + buf * TW * LANES + lane;
+      return (buf ? tape2 : m.tape) + (long long)unit * TW * LANES + lane;
     };
     const int who = consumer ? 1 : 0;  // each warp walks its own stack
     auto sys_of_buf = [&](int buf) -> WSys<T> {
       if (ONCHIP)
         return WSys<T>{s_prm + lane, meta_l, tape_of(buf), s_adj + lane, nl, MS, NPRM_W, 0,
-                       s_stk + who * sdw * LANES + lane};
+                       s_stk + who * sdw * LANES + lane, tape_of(buf) + L * NWT * LANES};
       return WSys<T>{gprm, gmeta, tape_of(buf), m.adj + (long long)unit * L * NWA * LANES + lane, nl, 1, NPRM, m.pf,
-                     w_stack(m, who, unit, lane)};
+                     w_stack(m, who, unit, lane), tape_of(buf) + L * NWT * LANES};
     };
     // the producer's inputs of step t: x^t and tau^t (the system's own coordinates)
     auto fetch = [&](long long t, int buf) {
@@ -134,12 +136,12 @@ k_wbackward_pipe(DevModel<T> m, const T* __restrict__ ckpt, const T* __restrict_
           const WSys<T> sp = sys_of_buf(buf);
           if (ONCHIP) {
             const T* x = s_in + buf * W * LANES + lane;
-            wstep_forward<T, DT, true, false>(sp, Col<const T>{x, LANES}, Col<const T>{x + nqm * LANES, LANES},
+            wstep_forward<T, DT, true, false, FR>(sp, Col<const T>{x, LANES}, Col<const T>{x + nqm * LANES, LANES},
                                               Col<const T>{x + NX * LANES, LANES}, g, m.dt, m.integ,
                                               Col<T>{nullptr, 0}, Col<T>{nullptr, 0});
           } else {
             const T* x = ckpt + t * NX * B + b;
-            wstep_forward<T, DT, true, false>(sp, Col<const T>{x, B}, Col<const T>{x + nqm * B, B},
+            wstep_forward<T, DT, true, false, FR>(sp, Col<const T>{x, B}, Col<const T>{x + nqm * B, B},
                                               Col<const T>{tau + t * nvm * B + b, B}, g, m.dt, m.integ,
                                               Col<T>{nullptr, 0}, Col<T>{nullptr, 0});
           }
@@ -153,7 +155,7 @@ k_wbackward_pipe(DevModel<T> m, const T* __restrict__ ckpt, const T* __restrict_
         if (act) {
           const WSys<T> sc = sys_of_buf(buf);
           T* gt = gtau + t * nvm * B + b;
-          wstep_adjoint<T, DT>(sc, gq, gqd, Col<T>{gt, B}, gm, m.dt, m.integ);
+          wstep_adjoint<T, DT, FR>(sc, gq, gqd, Col<T>{gt, B}, gm, m.dt, m.integ, g);
           for (int d = nv; d < nvm; ++d) gt[d * B] = T(0);
           if (gtraj) {
             const T* gx = gtraj + t * NX * B + b;

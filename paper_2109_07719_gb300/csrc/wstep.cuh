@@ -74,6 +74,10 @@ namespace abasim {
 enum : int {
   W_R = 0, W_V = 9, W_U = 15, W_DI = 21, W_u = 23, W_D = 24, W_AP = 27, W_QDD = 33, W_QD = 34, W_RW = 35, NWT = 38
 };
+// Record of a free root (FR kernels; link 0 only), [field][lane]: its articulated
+// inertia, qdd, and the quaternion and velocity the step started from.  Its link's
+// tape words hold R whole, the rotated COM inertia in W_U and its acceleration in W_AP.
+enum : int { WF_IA = 0, WF_QDD = 21, WF_Q = 27, WF_QD = 31, NWF = 37 };
 // Per-link adjoint record, [link][field][lane]: W = -w and lambda.
 enum : int { WA_W = 0, WA_L = 6, NWA = 7 };
 // One entry of the stack of parent values, [entry][field][lane]: (R, v), a or W in
@@ -95,6 +99,7 @@ template <class T> struct WSys {
   int pstride = NPRM;
   int pf = 0;  // prm, meta, tape and adj in global memory: prefetch this many links ahead (0: none)
   T* stk = nullptr;  // [entry][WSW][LANES]: the stack of parent values (see the tree data flow above)
+  T* root = nullptr; // [NWF][LANES]: the free root's record (FR only)
   SD T P(int l, int f) const { return prm[(l * pstride + f) * LANES]; }
   SD int M(int l) const { return meta[l * LANES * mstride]; }
   SD T& tp(int l, int f) const { return tape[(l * NWT + f) * LANES]; }
@@ -265,8 +270,9 @@ template <class T> SD void body_terms(T m, V3<T> rw, const S3<T>& Ic, SV<T> v, S
 // One step for the state (q, qd) and joint force tau.  ADJ: also store what the
 // adjoint reads.  INTEG: integrate into (qo, qdo) in the acceleration pass (they may
 // alias q, qd: a link's own coordinates are read before they are written, and no
-// pass after it reads the state).
-template <class T, class DT, bool ADJ, bool INTEG>
+// pass after it reads the state).  FR: link 0 may be a free joint (R = E_tree^T R(quat),
+// S = R on both halves, so D = I^A in world axes: one Cholesky solve).
+template <class T, class DT, bool ADJ, bool INTEG, bool FR = false>
 SD void wstep_forward(const WSys<T>& s, Col<const T> q, Col<const T> qd, Col<const T> tau, V3<T> grav, T dt,
                       int integ, Col<T> qo, Col<T> qdo) {
   T* tp = s.tape;
@@ -284,6 +290,26 @@ SD void wstep_forward(const WSys<T>& s, Col<const T> q, Col<const T> qd, Col<con
       }
       const int m = s.M(l);
       const int par = meta_parent(m);
+      if (FR && meta_jtype(m) == J_FREE) {
+        const int qo = meta_qoff(m), vo = meta_voff(m);
+        const T qt[4] = {q[qo + 3], q[qo + 4], q[qo + 5], q[qo + 6]};
+        T w[6];
+        for (int i = 0; i < 6; ++i) w[i] = qd[vo + i];
+        R_prev = mTm(wprm_m3(s, l, P_E), quat_R(qt[0], qt[1], qt[2], qt[3]));
+        v_prev = SV<T>{mul(R_prev, V3<T>{w[0], w[1], w[2]}), mul(R_prev, V3<T>{w[3], w[4], w[5]})};
+        wm3(tp, NWT, l, W_R, R_prev);
+        wsv(tp, NWT, l, W_V, v_prev);
+        if (ADJ) {
+          for (int i = 0; i < 4; ++i) s.root[(WF_Q + i) * LANES] = qt[i];
+          for (int i = 0; i < 6; ++i) s.root[(WF_QD + i) * LANES] = w[i];
+        }
+        if (meta_treechild(m)) {
+          wm3(s.stk, WSW, sp, 0, R_prev);
+          wsv(s.stk, WSW, sp, 9, v_prev);
+          ++sp;
+        }
+        continue;
+      }
       T sn, cs;
       sincos_t(q[meta_qoff(m)], &sn, &cs);
       const T vl = qd[meta_voff(m)];
@@ -332,6 +358,7 @@ SD void wstep_forward(const WSys<T>& s, Col<const T> q, Col<const T> qd, Col<con
       const int par = meta_parent(m), vo = meta_voff(m);
       const M3<T> R = wm3(tp, NWT, l, W_R);
       const SV<T> v = wsv(tp, NWT, l, W_V);
+      const bool fr = FR && meta_jtype(m) == J_FREE;
       const V3<T> sx = col2(R);
       const T vl = qd[vo];
       const T tl = tau[vo] - s.P(l, P_DAMP) * vl;
@@ -343,7 +370,10 @@ SD void wstep_forward(const WSys<T>& s, Col<const T> q, Col<const T> qd, Col<con
       SV<T> pA;
       body_terms(s.P(l, P_M), rw, Ic, v, IA, pA);
       if (ADJ) {
-        put_inertia(s, l, Ic);
+        if (fr)
+          ws3(tp, NWT, l, W_U, Ic);
+        else
+          put_inertia(s, l, Ic);
         wv3(tp, NWT, l, W_RW, rw);
       }
       if (carry) {
@@ -354,6 +384,13 @@ SD void wstep_forward(const WSys<T>& s, Col<const T> q, Col<const T> qd, Col<con
         --sp;
         IA += wsi(s.stk, WSW, sp, 0);
         pA += wsv(s.stk, WSW, sp, 21);
+      }
+      if (fr) {  // D = I^A, u = R tau - p^A
+        const SV<T> f{mul(R, V3<T>{tau[vo], tau[vo + 1], tau[vo + 2]}),
+                      mul(R, V3<T>{tau[vo + 3], tau[vo + 4], tau[vo + 5]})};
+        if (ADJ) wsi(s.root, 0, 0, WF_IA, IA);
+        wsv(tp, NWT, l, W_AP, spd_solve<T, DT>(IA, f - pA));
+        continue;
       }
       const SV<T> U{mul(IA.A, sx), mulT(IA.B, sx)};
       const DT Di = DT(1) / (DT)dot(sx, U.w);
@@ -392,6 +429,33 @@ SD void wstep_forward(const WSys<T>& s, Col<const T> q, Col<const T> qd, Col<con
     }
     const int m = s.M(l);
     const int par = meta_parent(m), vi = meta_voff(m);
+    if (FR && meta_jtype(m) == J_FREE) {
+      const M3<T> R = wm3(tp, NWT, l, W_R);
+      const SV<T> a = wsv(tp, NWT, l, W_AP), b = a - a0;
+      const V3<T> bw = mulT(R, b.w), bv = mulT(R, b.v);
+      const T qdd[6] = {bw.x, bw.y, bw.z, bv.x, bv.y, bv.z};
+      if (ADJ)
+        for (int i = 0; i < 6; ++i) s.root[(WF_QDD + i) * LANES] = qdd[i];
+      if (meta_treechild(m)) {
+        wsv(s.stk, WSW, sp, 0, a);
+        ++sp;
+      }
+      if (INTEG) {
+        const int qi = meta_qoff(m);
+        T nu[6], x[7];
+        for (int i = 0; i < 6; ++i) {
+          const T v0 = qd[vi + i];
+          const T v1 = v0 + dt * qdd[i];
+          qdo[vi + i] = v1;
+          nu[i] = integ == I_SEMI_IMPLICIT ? v1 : v0;
+        }
+        for (int i = 0; i < 7; ++i) x[i] = q[qi + i];
+        free_advance(x, nu, dt);
+        for (int i = 0; i < 7; ++i) qo[qi + i] = x[i];
+      }
+      a_prev = a;
+      continue;
+    }
     const V3<T> sx = col2(wm3(tp, NWT, l, W_R));
     const SV<T> v = wsv(tp, NWT, l, W_V);
     const SV<T> U = wsv(tp, NWT, l, W_U);
@@ -455,9 +519,11 @@ template <class T> SD BodyGrad<T> body_grad(T m, V3<T> rw, const S3<T>& Ic, SV<T
 
 // Requires wstep_forward<ADJ = true>(q, qd, tau) to have filled the tape.  On entry
 // (gq, gqd) hold the adjoint of x^{k+1}; on exit that of x^k.  Writes the adjoint
-// of tau into gtau and adds dPhi/dm of every link into gm.
+// of tau into gtau and adds dPhi/dm of every link into gm.  FR (link 0 may be a free
+// joint) needs the gravity: the only motion a free root's orientation turns against.
 template <class T, class DT, bool FR = false>
-SD void wstep_adjoint(const WSys<T>& s, Col<T> gq, Col<T> gqd, Col<T> gtau, Col<T> gm, T dt, int integ) {
+SD void wstep_adjoint(const WSys<T>& s, Col<T> gq, Col<T> gqd, Col<T> gtau, Col<T> gm, T dt, int integ,
+                      V3<T> grav = zero3<T>()) {
   T* tp = s.tape;
   T* ad = s.adj;
   const int nl = s.nl;
@@ -473,6 +539,33 @@ SD void wstep_adjoint(const WSys<T>& s, Col<T> gq, Col<T> gqd, Col<T> gtau, Col<
       }
       const int m = s.M(l);
       const int par = meta_parent(m), qi = meta_qoff(m), vi = meta_voff(m);
+      if (FR && meta_jtype(m) == J_FREE) {  // lambda_root = (I^A)^-1 (R qddb + y)
+        T qt[4], nu[6], qddb6[6];
+        for (int i = 0; i < 4; ++i) qt[i] = s.root[(WF_Q + i) * LANES];
+        for (int i = 0; i < 6; ++i) {
+          nu[i] = s.root[(WF_QD + i) * LANES];
+          if (integ == I_SEMI_IMPLICIT) nu[i] += dt * s.root[(WF_QDD + i) * LANES];
+        }
+        free_integrator_adjoint(qt, nu, gq, gqd, qi, vi, dt, integ, qddb6);
+        const M3<T> R = wm3(tp, NWT, l, W_R);
+        SV<T> y{mul(R, V3<T>{qddb6[0], qddb6[1], qddb6[2]}), mul(R, V3<T>{qddb6[3], qddb6[4], qddb6[5]})};
+        if (carry) y += cy;
+        carry = false;
+        if (meta_treechild(m)) {
+          --sp;
+          y += wsv(s.stk, WSW, sp, 0);
+        }
+        const SV<T> w = spd_solve<T, DT>(wsi(s.root, 0, 0, WF_IA), y);
+        wsv(ad, NWA, l, WA_W, zeroSV<T>() - w);
+        const V3<T> lw = mulT(R, w.w), lv = mulT(R, w.v);
+        gtau[vi] = lw.x;
+        gtau[vi + 1] = lw.y;
+        gtau[vi + 2] = lw.z;
+        gtau[vi + 3] = lv.x;
+        gtau[vi + 4] = lv.y;
+        gtau[vi + 5] = lv.z;
+        continue;
+      }
       T qddb;
       {
         const T qb = gq[qi], vb = gqd[vi];
@@ -516,6 +609,14 @@ SD void wstep_adjoint(const WSys<T>& s, Col<T> gq, Col<T> gqd, Col<T> gtau, Col<
       }
       const int m = s.M(l);
       const int par = meta_parent(m), vi = meta_voff(m);
+      if (FR && meta_jtype(m) == J_FREE) {
+        W_prev = wsv(ad, NWA, l, WA_W);
+        if (meta_treechild(m)) {
+          wsv(s.stk, WSW, sp, 0, W_prev);
+          ++sp;
+        }
+        continue;
+      }
       SV<T> W = zeroSV<T>();
       if (par >= 0) {
         SV<T> Wp = W_prev;
@@ -553,11 +654,14 @@ SD void wstep_adjoint(const WSys<T>& s, Col<T> gq, Col<T> gqd, Col<T> gtau, Col<
       }
       const int m = s.M(l);
       const int par = meta_parent(m), qi = meta_qoff(m), vi = meta_voff(m);
+      const bool fr = FR && meta_jtype(m) == J_FREE;
       const V3<T> sx = wcol2(tp, l);
       const SV<T> v = wsv(tp, NWT, l, W_V), ap = wsv(tp, NWT, l, W_AP), W = wsv(ad, NWA, l, WA_W);
-      const T vl = s.tp(l, W_QD);
-      const SV<T> a{ap.w + s.tp(l, W_QDD) * sx, ap.v};
-      BodyGrad<T> g = body_grad(s.P(l, P_M), wv3(tp, NWT, l, W_RW), get_inertia(s, l), v, a, W);
+      const T vl = fr ? T(0) : s.tp(l, W_QD);
+      const T qdd = fr ? T(0) : s.tp(l, W_QDD);
+      const SV<T> a{ap.w + qdd * sx, ap.v};
+      const S3<T> Ic = fr ? ws3(tp, NWT, l, W_U) : get_inertia(s, l);
+      BodyGrad<T> g = body_grad(s.P(l, P_M), wv3(tp, NWT, l, W_RW), Ic, v, a, W);
       gm[l] += g.mb;
       if (carry) {
         g.vb += cv;
@@ -570,6 +674,18 @@ SD void wstep_adjoint(const WSys<T>& s, Col<T> gq, Col<T> gqd, Col<T> gtau, Col<
         g.vb += wsv(s.stk, WSW, sp, 0);
         g.ab += wsv(s.stk, WSW, sp, 6);
         g.F += wsv(s.stk, WSW, sp, 12);
+      }
+      if (fr) {  // v = R qd, a = R qdd + [0; -g]: only the gravity does not turn with R
+        const M3<T> R = wm3(tp, NWT, l, W_R);
+        const V3<T> bw = mulT(R, g.vb.w), bv = mulT(R, g.vb.v);
+        const T vv[6] = {bw.x, bw.y, bw.z, bv.x, bv.y, bv.z};
+        for (int i = 0; i < 6; ++i) gqd[vi + i] += vv[i];
+        const M3<T> EJb = mmT(outer(mulT(R, g.ab.v), zero3<T>() - grav), wprm_m3(s, l, P_E));  // E = E_J E_t
+        T qb[4] = {T(0), T(0), T(0), T(0)};
+        quat_R_adj(s.root[WF_Q * LANES], s.root[(WF_Q + 1) * LANES], s.root[(WF_Q + 2) * LANES],
+                   s.root[(WF_Q + 3) * LANES], transpose(EJb), qb);
+        for (int i = 0; i < 4; ++i) gq[qi + 3 + i] += qb[i];
+        continue;
       }
       // c = v x [s qd; 0] = -qd e with e = [s x v_w; s x v_v]; b = [s x ab_w; s x ab_v]
       const SV<T> e{cross(sx, v.w), cross(sx, v.v)}, b{cross(sx, g.ab.w), cross(sx, g.ab.v)};
