@@ -400,10 +400,12 @@ int sim_create(const sim_model_desc* d, sim_handle** out) {
   if (rc == SIM_OK) rc = alloc(&h->tape, (size_t)maxL * NTAPE * Bpad * h->scalar, "tape");
   if (rc == SIM_OK) rc = alloc(&h->adj, (size_t)maxL * NADJ * Bpad * h->scalar, "adjoint tape");
   if (rc == SIM_OK) rc = alloc(&h->gm_acc, (size_t)maxL * B * h->scalar, "mass-gradient buffer");
-  if (rc == SIM_OK && h->unconstrained)
-    rc = alloc(&h->wtape2, ((size_t)maxL * NWT + NWF) * Bpad * h->scalar, "second world-aligned tape");
+  // the pipelined adjoint's tapes share the link-frame tape's buffer where they fit in it
+  const size_t ring_words = (size_t)WPIPE_TAPES * (maxL * NWT + (h->all_revolute ? 0 : NWF));
+  if (rc == SIM_OK && h->unconstrained && ring_words > (size_t)maxL * NTAPE)
+    rc = alloc(&h->wtapes, ring_words * Bpad * h->scalar, "world-aligned tapes");
   if (rc == SIM_OK && h->unconstrained && h->wdepth > 0)
-    rc = alloc(&h->wstk, (size_t)2 * h->wdepth * WSW * Bpad * h->scalar, "world-aligned stacks");
+    rc = alloc(&h->wstk, (size_t)(WPIPE_TAPES + 1) * h->wdepth * WSW * Bpad * h->scalar, "world-aligned stacks");
   if (rc == SIM_OK) rc = alloc((void**)&h->status, B * sizeof(int), "status");
   if (rc == SIM_OK) rc = alloc((void**)&h->sys_of_slot, B * sizeof(int), "slot order");
   if (rc == SIM_OK) rc = put(h->sys_of_slot, order.data(), B * sizeof(int));
@@ -431,7 +433,7 @@ int sim_create(const sim_model_desc* d, sim_handle** out) {
 void sim_destroy(sim_handle* h) {
   if (!h) return;
   void* ptrs[] = {h->prm, h->meta, h->nl, h->nqv, h->tape, h->adj, h->gm_acc, h->link_slot,
-                  h->status, h->sys_of_slot, h->counter, h->ctape, h->csys, h->x64, h->wtape2, h->wstk};
+                  h->status, h->sys_of_slot, h->counter, h->ctape, h->csys, h->x64, h->wtapes, h->wstk};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   delete h;

@@ -30,8 +30,8 @@ struct sim_handle {
   int* nqv = nullptr;        // [B]  nq | nv << 16
   void* tape = nullptr;      // [maxL][NTAPE][B] scalar
   void* adj = nullptr;       // [maxL][NADJ][B] scalar
-  void* wtape2 = nullptr;    // [maxL * NWT + NWF][B] scalar: the pipelined world-aligned adjoint's second tape
-  void* wstk = nullptr;      // [2][wdepth][WSW][B] scalar: the world-aligned passes' stacks of parent values
+  void* wtapes = nullptr;    // [WPIPE_TAPES][maxL * NWT + NWF][B] scalar: the pipelined adjoint's tapes (null: in tape)
+  void* wstk = nullptr;      // [WPIPE_TAPES + 1][wdepth][WSW][B] scalar: the warps' stacks of parent values
   int wdepth = 0;            // entries a system's stack holds at most (depth-first nesting of its branchings)
   void* gm_acc = nullptr;    // [maxL][B] scalar
   int* link_slot = nullptr;  // [L_total] -> l * B + slot

@@ -10,6 +10,7 @@
 #include "contact.cuh"
 #include "dual.cuh"
 #include "handle.h"
+#include "wstep.cuh"
 
 namespace abasim {
 namespace host {
@@ -38,7 +39,7 @@ template <class T> struct DevModel {
   ContactParams<T> cp;
   double dt64;   // the time step in FP64
   double* x64;   // FP64 running state [nq_max + nv_max][B] of the rollout (null: off; FP32 + FP64 D only)
-  int pf;        // world-aligned kernels with a global tape: prefetch distance in links (0: none)
+  int pf;        // world-aligned kernels with a global tape: links a record is staged ahead (0: none)
   T* stk;        // world-aligned kernels: two stacks of parent values [2][tiles][wdepth][WSW][lane] (null: none)
   int wdepth;    // entries per stack
 };
@@ -49,7 +50,7 @@ template <class T> DevModel<T> dev_model(const sim_handle* h) {
                      (T)h->g[0], (T)h->g[1], (T)h->g[2], h->integrator, 0, 0,
                      h->replay == SIM_REPLAY_QUADRATIC, (T*)h->ctape, (T*)h->csys,
                      ContactParams<T>{(T)h->friction, (T)h->erp, h->pgs_iterations}, h->dt,
-                     h->state64 ? (double*)h->x64 : nullptr, h->prefetch, (T*)h->wstk, h->wdepth};
+                     h->state64 ? (double*)h->x64 : nullptr, std::min(h->prefetch, RING_AHEAD), (T*)h->wstk, h->wdepth};
 }
 
 extern __shared__ __align__(16) unsigned char g_smem[];
@@ -115,11 +116,6 @@ template <class T> __device__ __forceinline__ void cp_async(T* smem_dst, const T
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(dst), "l"(gsrc) : "memory");
   else
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst), "l"(gsrc) : "memory");
-}
-// 16-byte copy bypassing L1 (both addresses 16-byte aligned).
-__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gsrc) {
-  const unsigned dst = (unsigned)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(gsrc) : "memory");
 }
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_wait_all_but_newest() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
@@ -920,41 +916,56 @@ inline int l1_carveout(const sim_handle* h, int slots_per_block, size_t bytes) {
   return (int)std::min(100LL, std::max(1LL, (100 * want + sm_smem - 1) / sm_smem));
 }
 
-// Storage of a world-aligned launch: the tape on chip when a block's tiles fit the
-// per-block opt-in limit and that adds no wave of blocks over the global-tape
-// kernel (whose blocks still keep their state and input streams on chip).
+// Scalars per tile of a world-aligned kernel's working state (w_smem_per_tile's, without
+// the rings).
+inline long long w_state_per_tile(const sim_handle* h, bool bwd) {
+  return h->nq_max + h->nv_max + (bwd ? h->maxL : 0);
+}
+
+// Storage of a world-aligned one-warp launch: the tape on chip when a block's tiles fit the
+// per-block opt-in limit and that adds no wave of blocks over the global-tape kernel.  The
+// latter's rings take shared memory too: where a block of h->block threads with them would
+// not fit, it runs fewer tiles per block (*threads), then stages fewer links ahead.
 template <class T, class K>
-int choose_w(sim_handle* h, K k_on, K k_off, bool bwd, bool* onchip, size_t* bytes) {
+int choose_w(sim_handle* h, K k_on, K k_off, bool bwd, bool* onchip, int* threads, int* ahead, size_t* bytes) {
   int limit = 0;
   cudaError_t e = cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
   if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory limit query");
-  const int tiles = h->block / LANES;
   const int nx = h->nq_max + h->nv_max;
   const bool fr = !h->all_revolute;
-  const size_t need_on = (size_t)tiles * w_smem_per_tile(h->maxL, nx, h->nv_max, bwd, true, h->wdepth * WSW, fr) * LANES * sizeof(T);
-  const size_t need_off = (size_t)tiles * w_smem_per_tile(h->maxL, nx, h->nv_max, bwd, false, 0, fr) * LANES * sizeof(T);
+  auto need = [&](bool on, int tiles, int ah) {
+    return (size_t)tiles * w_smem_per_tile(h->maxL, nx, h->nv_max, bwd, on, h->wdepth * WSW, fr, ah) * LANES * sizeof(T);
+  };
+  int tiles = h->block / LANES;
+  while (tiles > 1 && need(false, tiles, *ahead) > (size_t)limit) --tiles;
+  while (*ahead > 0 && need(false, tiles, *ahead) > (size_t)limit) --*ahead;
+  const size_t need_on = need(true, h->block / LANES, 0), need_off = need(false, tiles, *ahead);
   if (need_off > (size_t)limit) return fail(h, SIM_EUNSUPPORTED, "the working state does not fit in shared memory");
   e = cudaFuncSetAttribute((const void*)k_off, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need_off);
   if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory opt-in");
   // the global-tape kernel: shared memory for the blocks an SM holds at once, the rest of the SM's
-  // unified L1 / shared storage as L1 for the tape lines the passes prefetch
+  // unified L1 / shared storage as L1 for the stacks
   e = cudaFuncSetAttribute((const void*)k_off, cudaFuncAttributePreferredSharedMemoryCarveout,
-                           l1_carveout(h, h->block, need_off));
+                           l1_carveout(h, tiles * LANES, need_off));
   if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory carve-out");
   *onchip = false;
+  *threads = tiles * LANES;
   *bytes = need_off;
   if (need_on > (size_t)limit) return SIM_OK;
   e = cudaFuncSetAttribute((const void*)k_on, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need_on);
   if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory opt-in");
   int per_on = 0, per_off = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_on, k_on, h->block, need_on);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_off, k_off, h->block, need_off);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_off, k_off, *threads, need_off);
   if (e != cudaSuccess) return cuda_fail(h, e, "occupancy query");
-  const long long units = (h->B + h->block - 1) / h->block;
   const long long sms = std::max(1, h->sms);
-  auto waves = [&](int per_sm) { return per_sm > 0 ? (units + sms * per_sm - 1) / (sms * per_sm) : 1LL << 40; };
-  if (waves(per_on) <= waves(per_off)) {
+  auto waves = [&](int per_sm, int block) {
+    const long long units = (h->B + block - 1) / block;
+    return per_sm > 0 ? (units + sms * per_sm - 1) / (sms * per_sm) : 1LL << 40;
+  };
+  if (waves(per_on, h->block) <= waves(per_off, *threads)) {
     *onchip = true;
+    *threads = h->block;
     *bytes = need_on;
   }
   return SIM_OK;
@@ -966,7 +977,7 @@ int choose_w(sim_handle* h, K k_on, K k_off, bool bwd, bool* onchip, size_t* byt
 // serial chains applies.  Floating bases take it under SIM_TAPE_AUTO: rollout +
 // adjoint of 8192 quadrupeds over 60 steps (FP32 + FP64 D-solves) 15.6 -> 11.3 ms
 // against the link-frame one-warp kernels, 1024 humanoids over 60 steps (FP32) 10.95
-// -> 4.39 ms.  The link-frame pipelined adjoint of chains is kept with FP64 pivots.
+// -> 4.39 ms.
 template <class T, class DT>
 bool use_aligned(const sim_handle* h, bool rollout, int k) {
   const bool fr = !h->all_revolute;
@@ -977,17 +988,10 @@ bool use_aligned(const sim_handle* h, bool rollout, int k) {
     return false;
   int limit = 0;
   if (cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device) != cudaSuccess) return false;
-  const int nx = h->nq_max + h->nv_max;
-  const size_t streams = (size_t)(h->block / LANES) * w_smem_per_tile(h->maxL, nx, h->nv_max, !rollout, false, 0, fr) * LANES *
-                         sizeof(T);
+  const size_t streams = (size_t)(h->block / LANES) * w_state_per_tile(h, !rollout) * LANES * sizeof(T);
   if (streams > (size_t)limit) return false;
-  if (h->tape_space != SIM_TAPE_AUTO || !h->all_chains) return true;
-  if (rollout) return !(h->maxL <= PIPE_MAX_LINKS);
-  const bool link_pipe = sizeof(T) == 4 && k == 1 &&
-                         (size_t)pipe_smem_per_tile(h->maxL, nx, h->nv_max) * LANES * sizeof(T) <= (size_t)limit;
-  if (!link_pipe) return true;
-  return sizeof(DT) == sizeof(T) &&
-         (size_t)wpipe_smem_per_tile(h->maxL, nx, h->nv_max, true, h->wdepth * WSW, fr) * LANES * sizeof(T) <= (size_t)limit;
+  if (h->tape_space != SIM_TAPE_AUTO || !h->all_chains || !rollout) return true;
+  return h->maxL > PIPE_MAX_LINKS;
 }
 
 template <class T, class DT>
@@ -998,21 +1002,22 @@ int launch_wrollout(sim_handle* h, const void* q0, const void* qd0, const void* 
                          k_off = wrollout_kernel<T, DT>(false, !h->all_revolute);
   bool onchip = false;
   size_t shm = 0;
-  int rc = choose_w<T>(h, k_on, k_off, false, &onchip, &shm);
+  int threads = 0;
+  int rc = choose_w<T>(h, k_on, k_off, false, &onchip, &threads, &m.pf, &shm);
   if (rc != SIM_OK) return rc;
   const RolloutKernel<T> kern = onchip ? k_on : k_off;
   h->last_storage = (h->all_revolute ? 4 : 8) + (onchip ? 0 : 1);
   int grid = 0;
-  rc = launch_shape(h, kern, &grid, &m.persistent, shm, stream);
+  rc = launch_shape(h, kern, &grid, &m.persistent, shm, stream, threads);
   if (rc != SIM_OK) return rc;
-  kern<<<grid, h->block, shm, S(stream)>>>(m, (const T*)q0, (const T*)qd0, (const T*)tau, (long long)T_, k,
+  kern<<<grid, threads, shm, S(stream)>>>(m, (const T*)q0, (const T*)qd0, (const T*)tau, (long long)T_, k,
                                            (T*)ckpt, (T*)qT, (T*)qdT, (T*)traj);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? SIM_OK : cuda_fail(h, e, "rollout launch");
 }
 
-// The pipelined world-aligned adjoint (two warps per 32-system tile, k = 1):
-// tapes on chip when one tile's fit a block, else in global memory.
+// The pipelined world-aligned adjoint (k = 1): one consumer warp and np producer warps per
+// 32-system tile, their tapes on chip when they fit a block, else in global memory.
 template <class T, class DT>
 int launch_wbackward_pipe(sim_handle* h, const void* ckpt, const void* tau, int64_t T_, const void* gqT,
                           const void* gqdT, const void* gtraj, void* gq0, void* gqd0, void* gtau, void* gmass,
@@ -1023,11 +1028,24 @@ int launch_wbackward_pipe(sim_handle* h, const void* ckpt, const void* tau, int6
   if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory limit query");
   const int nx = h->nq_max + h->nv_max;
   const bool fr = !h->all_revolute;
-  const size_t need_on = (size_t)wpipe_smem_per_tile(h->maxL, nx, h->nv_max, true, h->wdepth * WSW, fr) * LANES * sizeof(T);
-  const size_t need_off = (size_t)wpipe_smem_per_tile(h->maxL, nx, h->nv_max, false, 0, fr) * LANES * sizeof(T);
-  const bool onchip = need_on <= (size_t)limit && (!fr || (h->B + LANES - 1) / LANES <= std::max(1, h->sms));
-  if (!onchip && !h->wtape2) return fail(h, SIM_EUNSUPPORTED, "no second tape for the pipelined adjoint");
-  const size_t shm = onchip ? need_on : need_off;
+  const int tiles = (h->B + LANES - 1) / LANES, sms = std::max(1, h->sms);
+  auto need = [&](bool on, int np, int ah) {
+    return (size_t)wpipe_smem_per_tile(h->maxL, nx, h->nv_max, on, h->wdepth * WSW, fr, np, ah) * LANES * sizeof(T);
+  };
+  const bool onchip = need(true, 1, 0) <= (size_t)limit && (!fr || tiles <= sms);
+  // Producers: three while every tile has an SM to itself (4096 7-link chains, on chip: 6.96
+  // us a step with one, 5.60, 4.94 with three, 5.5 with four or five; 1024 humanoids, global
+  // tapes: 36.5, 31.6, 29.6).  With more tiles than that the SMs are shared: on chip the
+  // two producers that take no more tapes than one, so that two blocks fit an SM (16384
+  // chains 13.3 us, 19.3 with three); with global tapes one (8192 quadrupeds FP32 26.6 us,
+  // 31.9 with three; 16384 trees the same with any), but three where the FP64 pipe is what
+  // the producers share out (quadrupeds with FP64 D-solves 92.1 -> 63.9 us).
+  int np = tiles <= sms || (!onchip && sizeof(DT) == 8) ? WPIPE_TAPES : onchip ? 2 : 1;
+  while (np > 1 && need(onchip, np, onchip ? 0 : std::min(1, m.pf)) > (size_t)limit) --np;
+  while (!onchip && m.pf > 0 && need(false, np, m.pf) > (size_t)limit) --m.pf;
+  const size_t shm = need(onchip, np, m.pf);
+  if (shm > (size_t)limit) return fail(h, SIM_EUNSUPPORTED, "the working state does not fit in shared memory");
+  const int threads = (np + 1) * LANES;
   const BackwardKernel<T> kern = wbackward_pipe_kernel<T, DT>(onchip, fr);
   e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
   if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory opt-in");
@@ -1038,11 +1056,11 @@ int launch_wbackward_pipe(sim_handle* h, const void* ckpt, const void* tau, int6
   }
   h->last_storage_bwd = (fr ? 10 : 6) + (onchip ? 0 : 1);
   int grid = 0;
-  int rc = launch_shape(h, kern, &grid, &m.persistent, shm, stream, 2 * LANES, LANES);
+  int rc = launch_shape(h, kern, &grid, &m.persistent, shm, stream, threads, LANES);
   if (rc != SIM_OK) return rc;
-  kern<<<grid, 2 * LANES, shm, S(stream)>>>(m, (const T*)ckpt, (const T*)tau, (long long)T_, 1, (const T*)gqT,
-                                            (const T*)gqdT, (const T*)gtraj, (T*)gq0, (T*)gqd0, (T*)gtau,
-                                            (T*)h->gm_acc, (T*)h->wtape2);
+  kern<<<grid, threads, shm, S(stream)>>>(m, (const T*)ckpt, (const T*)tau, (long long)T_, 1, (const T*)gqT,
+                                          (const T*)gqdT, (const T*)gtraj, (T*)gq0, (T*)gqd0, (T*)gtau,
+                                          (T*)h->gm_acc, (T*)(h->wtapes ? h->wtapes : h->tape));
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(h, e, "backward launch");
   if (gmass) {
@@ -1065,14 +1083,15 @@ int launch_wbackward(sim_handle* h, const void* ckpt, const void* tau, int64_t T
                           k_off = wbackward_kernel<T, DT>(false, !h->all_revolute);
   bool onchip = false;
   size_t shm = 0;
-  int rc = choose_w<T>(h, k_on, k_off, true, &onchip, &shm);
+  int threads = 0;
+  int rc = choose_w<T>(h, k_on, k_off, true, &onchip, &threads, &m.pf, &shm);
   if (rc != SIM_OK) return rc;
   const BackwardKernel<T> kern = onchip ? k_on : k_off;
   h->last_storage_bwd = (h->all_revolute ? 4 : 8) + (onchip ? 0 : 1);
   int grid = 0;
-  rc = launch_shape(h, kern, &grid, &m.persistent, shm, stream);
+  rc = launch_shape(h, kern, &grid, &m.persistent, shm, stream, threads);
   if (rc != SIM_OK) return rc;
-  kern<<<grid, h->block, shm, S(stream)>>>(m, (const T*)ckpt, (const T*)tau, (long long)T_, k, (const T*)gqT,
+  kern<<<grid, threads, shm, S(stream)>>>(m, (const T*)ckpt, (const T*)tau, (long long)T_, k, (const T*)gqT,
                                            (const T*)gqdT, (const T*)gtraj, (T*)gq0, (T*)gqd0, (T*)gtau,
                                            (T*)h->gm_acc, (T*)work);
   cudaError_t e = cudaGetLastError();

@@ -10,6 +10,9 @@
 namespace abasim {
 namespace host {
 
+// Asks for the line at p (a step's inputs, one step ahead) to be brought into L2.
+__device__ __forceinline__ void pf_line(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // Scalars per system of one tape: the links' words, then the free root's record.
 __host__ __device__ __forceinline__ long long w_tape_words(int maxL, bool fr) {
   return (long long)maxL * NWT + (fr ? NWF : 0);
@@ -21,15 +24,14 @@ __host__ __device__ __forceinline__ long long w_tape_words(int maxL, bool fr) {
 // the adjoint, the adjoint record), the model constants and meta words, the stack
 // of parent values (sd scalars per system) and a double buffer for the per-step
 // inputs (tau, plus x^t for the adjoint) fetched one step ahead.  Without ONCHIP
-// the stack is in the handle's global scratch and the inputs are read from global
-// memory with their lines prefetched a step ahead, and the small shared-memory
-// footprint leaves most of the SM's L1 to the prefetched tape lines (staging the
-// inputs on chip instead cost more in L1 than it saved in misses).
+// the stack and the records are in the handle's global scratch, and the warp's ring
+// stages the records of the `ahead` next links (wstep.cuh).
 __host__ __device__ __forceinline__ long long w_smem_per_tile(int maxL, int nx, int nv, bool bwd, bool onchip,
-                                                              int sd, bool fr) {
+                                                              int sd, bool fr, int ahead) {
   const long long state = nx + (bwd ? maxL : 0);
-  if (!onchip) return state;
-  return w_tape_words(maxL, fr) + (long long)maxL * ((bwd ? NWA : 0) + NPRM_W + 1) + sd + state + 2LL * (nv + (bwd ? nx : 0));
+  if (!onchip) return state + (ahead + 1LL) * (bwd ? RING_ADJ : RING_FWD);
+  return w_tape_words(maxL, fr) + (long long)maxL * ((bwd ? NWA : 0) + NPRM_W + 1) + sd + state +
+         2LL * (nv + (bwd ? nx : 0));
 }
 
 // Stack `which` (0, or 1 for the second warp of the pipelined adjoint) of a tile's
@@ -41,27 +43,29 @@ __device__ __forceinline__ T* w_stack(const DevModel<T>& m, int which, long long
   return m.stk + ((long long)which * tiles + tile) * m.wdepth * WSW * LANES + lane;
 }
 
-struct WTile {
-  void* tape;
-  void* adj;
-  void* prm;
+template <class T> struct WTile {
+  T* tape;
+  T* adj;
+  T* prm;
   int* meta;
-  void* stk;
-  void* state;
-  void* gm;
-  void* stream;
+  T* stk;
+  T* ring;  // at lane 0
+  T* state;
+  T* gm;
+  T* stream;
 };
 
 template <class T, bool BWD, bool ONCHIP, bool FR>
-__device__ __forceinline__ WTile w_tile(int maxL, int nx, int nv, int sd, int lane) {
+__device__ __forceinline__ WTile<T> w_tile(const DevModel<T>& m, int lane) {
   const int tb = threadIdx.x / LANES;
-  const long long L = maxL;
-  T* base =
-      reinterpret_cast<T*>(g_smem) + (long long)tb * w_smem_per_tile(maxL, nx, nv, BWD, ONCHIP, sd, FR) * LANES + lane;
-  WTile t{};
+  const long long L = m.maxL;
+  const int nx = m.nq_max + m.nv_max, sd = m.wdepth * WSW;
+  T* base = reinterpret_cast<T*>(g_smem) +
+            (long long)tb * w_smem_per_tile(m.maxL, nx, m.nv_max, BWD, ONCHIP, sd, FR, m.pf) * LANES + lane;
+  WTile<T> t{};
   if (ONCHIP) {
     t.tape = base;
-    base += w_tape_words(maxL, FR) * LANES;
+    base += w_tape_words(m.maxL, FR) * LANES;
     t.adj = base;
     if (BWD) base += L * NWA * LANES;
     t.prm = base;
@@ -70,6 +74,9 @@ __device__ __forceinline__ WTile w_tile(int maxL, int nx, int nv, int sd, int la
     base += L * LANES;
     t.stk = base;
     base += (long long)sd * LANES;
+  } else {
+    t.ring = base - lane;
+    base += (m.pf + 1LL) * (BWD ? RING_ADJ : RING_FWD) * LANES;
   }
   t.state = base;
   base += (long long)nx * LANES;
@@ -79,43 +86,46 @@ __device__ __forceinline__ WTile w_tile(int maxL, int nx, int nv, int sd, int la
   return t;
 }
 
-// The system view of a slot: constants, meta words and tape on chip (copied in
-// here) or in global memory.
+// The system view of a slot: constants, meta words and tape on chip (copied in here) or
+// in global memory.  Every lane of the warp calls it; a lane past the batch has nl = 0.
 template <class T, bool BWD, bool ONCHIP, bool FR>
-__device__ __forceinline__ WSys<T> wsys_of(const DevModel<T>& m, int slot) {
+__device__ __forceinline__ WSys<T, !ONCHIP> wsys_of(const DevModel<T>& m, int slot, bool act) {
   const long long tile = slot / LANES, lane = slot % LANES;
   const long long L = m.maxL;
   const T* gprm = m.prm + tile * L * NPRM * LANES + lane;
   const int* gmeta = m.meta + tile * L * LANES + lane;
-  const int nl = m.nl[slot];
-  if (ONCHIP) {
-    const WTile t = w_tile<T, BWD, ONCHIP, FR>(m.maxL, m.nq_max + m.nv_max, m.nv_max, m.wdepth * WSW, (int)lane);
-    T* sp = (T*)t.prm;
+  const int nl = act ? m.nl[slot] : 0;
+  const WTile<T> t = w_tile<T, BWD, ONCHIP, FR>(m, (int)lane);
+  if constexpr (ONCHIP) {
     constexpr int MS = (int)(sizeof(T) / sizeof(int));
     for (int l = 0; l < nl; ++l) {
-      for (int f = 0; f < NPRM_W; ++f) sp[(l * NPRM_W + f) * LANES] = gprm[(l * NPRM + f) * LANES];
+      for (int f = 0; f < NPRM_W; ++f) t.prm[(l * NPRM_W + f) * LANES] = gprm[(l * NPRM + f) * LANES];
       t.meta[l * LANES * MS] = gmeta[l * LANES];
     }
-    return WSys<T>{sp, t.meta, (T*)t.tape, (T*)t.adj, nl, MS, NPRM_W, 0, (T*)t.stk, (T*)t.tape + L * NWT * LANES};
+    return WSys<T>{t.prm, t.meta, t.tape, t.adj, nl, MS, NPRM_W, t.stk, t.tape + L * NWT * LANES};
+  } else {
+    T* tape = m.tape + tile * w_tape_words(m.maxL, FR) * LANES + lane;
+    return WSys<T, true>{gprm, gmeta, tape, m.adj + tile * L * NWA * LANES + lane, nl, 1, NPRM,
+                         w_stack(m, 0, tile, lane), tape + L * NWT * LANES,
+                         __reduce_max_sync(0xffffffffu, nl), t.ring, m.pf, (int)lane};
   }
-  T* tape = m.tape + tile * w_tape_words(m.maxL, FR) * LANES + lane;
-  return WSys<T>{gprm, gmeta, tape, m.adj + tile * L * NWA * LANES + lane, nl, 1, NPRM, m.pf,
-                 w_stack(m, 0, tile, lane), tape + L * NWT * LANES};
 }
 
+// One system's rollout.  Without ONCHIP every lane of a warp takes part (act: the lane has
+// a system; the others only help to stage records).
 template <class T, class DT, bool ONCHIP, bool FR>
-__device__ __forceinline__ void wrollout_one(const DevModel<T>& m, int slot, const T* __restrict__ q0,
+__device__ __forceinline__ void wrollout_one(const DevModel<T>& m, int slot, bool act, const T* __restrict__ q0,
                                              const T* __restrict__ qd0, const T* __restrict__ tau, long long Tn,
                                              int k, T* ckpt, T* qT, T* qdT, T* traj) {
-  const int b = m.sys_of_slot[slot];
+  const int b = act ? m.sys_of_slot[slot] : 0;
   const long long B = m.B;
   const int nqm = m.nq_max, nvm = m.nv_max, NX = nqm + nvm;
   const V3<T> g{m.g0, m.g1, m.g2};
-  const WSys<T> s = wsys_of<T, false, ONCHIP, FR>(m, slot);
-  const WTile st = w_tile<T, false, ONCHIP, FR>(m.maxL, NX, nvm, m.wdepth * WSW, slot % LANES);
-  const Col<T> q{(T*)st.state, LANES}, qd{(T*)st.state + nqm * LANES, LANES};
-  const int nv = m.nqv[slot] >> 16;
-  T* sbuf = (T*)st.stream;  // ONCHIP: [2][nvm][LANES], tau one step ahead
+  const WSys<T, !ONCHIP> s = wsys_of<T, false, ONCHIP, FR>(m, slot, act);
+  const WTile<T> st = w_tile<T, false, ONCHIP, FR>(m, slot % LANES);
+  const Col<T> q{st.state, LANES}, qd{st.state + nqm * LANES, LANES};
+  const int nv = act ? m.nqv[slot] >> 16 : 0;
+  T* sbuf = st.stream;  // ONCHIP: [2][nvm][LANES], tau one step ahead
   if (ONCHIP) {
     if (Tn > 0)
       for (int d = 0; d < nvm; ++d) cp_async(sbuf + d * LANES, tau + (long long)d * B + b);
@@ -123,16 +133,14 @@ __device__ __forceinline__ void wrollout_one(const DevModel<T>& m, int slot, con
   }
   for (int d = 0; d < nqm; ++d) q[d] = q0[d * B + b];
   for (int d = 0; d < nvm; ++d) qd[d] = qd0[d * B + b];
-  if (traj) {
-    for (int d = 0; d < nqm; ++d) traj[d * B + b] = q[d];
-    for (int d = 0; d < nvm; ++d) traj[(nqm + d) * B + b] = qd[d];
-  }
+  auto put = [&](T* c) {  // the state x into a [NX][B] array
+    if (!act) return;
+    for (int d = 0; d < nqm; ++d) c[d * B + b] = q[d];
+    for (int d = 0; d < nvm; ++d) c[(nqm + d) * B + b] = qd[d];
+  };
+  if (traj) put(traj);
   for (long long t = 0; t < Tn; ++t) {
-    if (ckpt && t % k == 0) {
-      T* c = ckpt + (t / k) * NX * B + b;
-      for (int d = 0; d < nqm; ++d) c[d * B] = q[d];
-      for (int d = 0; d < nvm; ++d) c[(nqm + d) * B] = qd[d];
-    }
+    if (ckpt && t % k == 0) put(ckpt + (t / k) * NX * B);
     Col<const T> tau_t{tau + t * nvm * B + b, B};
     if (ONCHIP) {
       if (t + 1 < Tn) {
@@ -146,14 +154,11 @@ __device__ __forceinline__ void wrollout_one(const DevModel<T>& m, int slot, con
       for (int d = 0; d < nv; ++d) pf_line(tau + ((t + 1) * nvm + d) * B + b);
     }
     wstep_forward<T, DT, false, true, FR>(s, Col<const T>{q.p, LANES}, Col<const T>{qd.p, LANES}, tau_t, g, m.dt,
-                                      m.integ, q, qd);
-    if (traj) {
-      T* c = traj + (t + 1) * NX * B + b;
-      for (int d = 0; d < nqm; ++d) c[d * B] = q[d];
-      for (int d = 0; d < nvm; ++d) c[(nqm + d) * B] = qd[d];
-    }
+                                          m.integ, q, qd);
+    if (traj) put(traj + (t + 1) * NX * B);
   }
   if (ONCHIP) cp_wait_all();
+  if (!act) return;
   bool ok = true;
   for (int d = 0; d < nqm; ++d) ok &= finite_t(q[d]);
   for (int d = 0; d < nvm; ++d) ok &= finite_t(qd[d]);
@@ -163,20 +168,21 @@ __device__ __forceinline__ void wrollout_one(const DevModel<T>& m, int slot, con
 }
 
 template <class T, class DT, bool ONCHIP, bool FR>
-__device__ __forceinline__ void wbackward_one(const DevModel<T>& m, int slot, const T* __restrict__ ckpt,
+__device__ __forceinline__ void wbackward_one(const DevModel<T>& m, int slot, bool act, const T* __restrict__ ckpt,
                                               const T* __restrict__ tau, long long Tn, int k,
                                               const T* __restrict__ gqT, const T* __restrict__ gqdT,
                                               const T* __restrict__ gtraj, T* gq0, T* gqd0, T* gtau, T* gm_acc,
                                               T* ring) {
-  const int b = m.sys_of_slot[slot];
+  const int b = act ? m.sys_of_slot[slot] : 0;
   const long long B = m.B;
   const int nqm = m.nq_max, nvm = m.nv_max, NX = nqm + nvm;
-  const int nq = m.nqv[slot] & 0xffff, nv = m.nqv[slot] >> 16;
+  const int nq = act ? m.nqv[slot] & 0xffff : 0, nv = act ? m.nqv[slot] >> 16 : 0;
+  const int rs = act ? slot : 0;  // this lane's column of the replay ring
   const V3<T> g{m.g0, m.g1, m.g2};
-  const WSys<T> s = wsys_of<T, true, ONCHIP, FR>(m, slot);
-  const WTile st = w_tile<T, true, ONCHIP, FR>(m.maxL, NX, nvm, m.wdepth * WSW, slot % LANES);
-  const Col<T> gq{(T*)st.state, LANES}, gqd{(T*)st.state + nqm * LANES, LANES}, gm{(T*)st.gm, LANES};
-  T* sbuf = (T*)st.stream;  // [2][NX + nvm][LANES]: x^t and tau^t, one step ahead (k = 1)
+  const WSys<T, !ONCHIP> s = wsys_of<T, true, ONCHIP, FR>(m, slot, act);
+  const WTile<T> st = w_tile<T, true, ONCHIP, FR>(m, slot % LANES);
+  const Col<T> gq{st.state, LANES}, gqd{st.state + nqm * LANES, LANES}, gm{st.gm, LANES};
+  T* sbuf = st.stream;  // ONCHIP: [2][NX + nvm][LANES]: x^t and tau^t, one step ahead (k = 1)
   for (int d = 0; d < nqm; ++d) {
     T v = d < nq ? gqT[d * B + b] : T(0);
     if (gtraj && d < nq) v += gtraj[(Tn * NX + d) * B + b];
@@ -192,12 +198,18 @@ __device__ __forceinline__ void wbackward_one(const DevModel<T>& m, int slot, co
     wstep_forward<T, DT, true, false, FR>(s, q, qd, tau_t, g, m.dt, m.integ, Col<T>{nullptr, 0}, Col<T>{nullptr, 0});
     T* gt = gtau + t * nvm * B + b;
     wstep_adjoint<T, DT, FR>(s, gq, gqd, Col<T>{gt, B}, gm, m.dt, m.integ, g);
-    for (int d = nv; d < nvm; ++d) gt[d * B] = T(0);
+    if (act)
+      for (int d = nv; d < nvm; ++d) gt[d * B] = T(0);
     if (gtraj) {
       const T* gx = gtraj + t * NX * B + b;
       for (int d = 0; d < nq; ++d) gq[d] += gx[d * B];
       for (int d = 0; d < nv; ++d) gqd[d] += gx[(nqm + d) * B];
     }
+  };
+  auto replay = [&](const T* from, T* to, long long t) {  // one step from state `from` to state `to`
+    wstep_forward<T, DT, false, true, FR>(s, Col<const T>{from, B}, Col<const T>{from + nqm * B, B},
+                                          Col<const T>{tau + t * nvm * B + b, B}, g, m.dt, m.integ, Col<T>{to, B},
+                                          Col<T>{to + nqm * B, B});
   };
   if (k == 1 && ONCHIP) {
     const int W = NX + nvm;
@@ -235,35 +247,27 @@ __device__ __forceinline__ void wbackward_one(const DevModel<T>& m, int slot, co
       const long long t1 = (t0 + k < Tn) ? t0 + k : Tn;
       const T* xs = ckpt + seg * NX * B + b;
       if (!m.quadratic) {  // replay the segment once, keeping its states (ring by slot)
-        T* r0 = ring + slot;
-        for (int d = 0; d < NX; ++d) r0[d * B] = xs[d * B];
-        for (long long j = 1; j < t1 - t0; ++j) {
-          const T* prev = ring + (j - 1) * NX * B + slot;
-          T* cur = ring + j * NX * B + slot;
-          wstep_forward<T, DT, false, true, FR>(s, Col<const T>{prev, B}, Col<const T>{prev + nqm * B, B},
-                                            Col<const T>{tau + (t0 + j - 1) * nvm * B + b, B}, g, m.dt, m.integ,
-                                            Col<T>{cur, B}, Col<T>{cur + nqm * B, B});
-        }
+        T* r0 = ring + rs;
+        if (act)
+          for (int d = 0; d < NX; ++d) r0[d * B] = xs[d * B];
+        for (long long j = 1; j < t1 - t0; ++j)
+          replay(ring + (j - 1) * NX * B + rs, ring + j * NX * B + rs, t0 + j - 1);
       }
       for (long long t = t1 - 1; t >= t0; --t) {
-        const T* x = ring + (t - t0) * NX * B + slot;
+        const T* x = ring + (t - t0) * NX * B + rs;
         if (m.quadratic) {  // recompute x^t from the segment checkpoint: t - t0 steps
-          T* cur = ring + slot;
+          T* cur = ring + rs;
           x = t == t0 ? xs : cur;
           if (t > t0) {
-            wstep_forward<T, DT, false, true, FR>(s, Col<const T>{xs, B}, Col<const T>{xs + nqm * B, B},
-                                              Col<const T>{tau + t0 * nvm * B + b, B}, g, m.dt, m.integ,
-                                              Col<T>{cur, B}, Col<T>{cur + nqm * B, B});
-            for (long long j = t0 + 1; j < t; ++j)
-              wstep_forward<T, DT, false, true, FR>(s, Col<const T>{cur, B}, Col<const T>{cur + nqm * B, B},
-                                                Col<const T>{tau + j * nvm * B + b, B}, g, m.dt, m.integ,
-                                                Col<T>{cur, B}, Col<T>{cur + nqm * B, B});
+            replay(xs, cur, t0);
+            for (long long j = t0 + 1; j < t; ++j) replay(cur, cur, j);
           }
         }
         step_back(t, Col<const T>{x, B}, Col<const T>{x + nqm * B, B}, Col<const T>{tau + t * nvm * B + b, B});
       }
     }
   }
+  if (!act) return;
   bool ok = true;
   for (int d = 0; d < nq; ++d) ok &= finite_t(gq[d]);
   for (int d = 0; d < nv; ++d) ok &= finite_t(gqd[d]);
@@ -274,18 +278,30 @@ __device__ __forceinline__ void wbackward_one(const DevModel<T>& m, int slot, co
   for (int l = 0; l < s.nl; ++l) gm_acc[l * B + slot] = gm[l];
 }
 
+// Runs `...` for every slot of this block's work units.  The lanes of a warp that stages
+// records run it together, those past the batch with act false.
+#define ABASIM_FOR_EACH_WSLOT(m, ...)                                        \
+  int unit = (m).persistent ? next_unit((m).counter) : (int)blockIdx.x;      \
+  while ((long long)unit * blockDim.x < (m).B) {                             \
+    const int slot = unit * blockDim.x + threadIdx.x;                        \
+    const bool act = slot < (m).B;                                           \
+    if (ONCHIP ? act : slot / LANES * LANES < (m).B) { __VA_ARGS__; }        \
+    if (!(m).persistent) break;                                              \
+    unit = next_unit((m).counter);                                           \
+  }
+
 template <class T, class DT, bool ONCHIP, bool FR>
 __global__ void k_wrollout(DevModel<T> m, const T* __restrict__ q0, const T* __restrict__ qd0,
                            const T* __restrict__ tau, long long Tn, int k, T* ckpt, T* qT, T* qdT, T* traj) {
-  ABASIM_FOR_EACH_SLOT(m, wrollout_one<T, DT, ONCHIP, FR>(m, slot, q0, qd0, tau, Tn, k, ckpt, qT, qdT, traj))
+  ABASIM_FOR_EACH_WSLOT(m, wrollout_one<T, DT, ONCHIP, FR>(m, slot, act, q0, qd0, tau, Tn, k, ckpt, qT, qdT, traj))
 }
 
 template <class T, class DT, bool ONCHIP, bool FR>
 __global__ void k_wbackward(DevModel<T> m, const T* __restrict__ ckpt, const T* __restrict__ tau, long long Tn,
                             int k, const T* __restrict__ gqT, const T* __restrict__ gqdT,
                             const T* __restrict__ gtraj, T* gq0, T* gqd0, T* gtau, T* gm_acc, T* ring) {
-  ABASIM_FOR_EACH_SLOT(m, wbackward_one<T, DT, ONCHIP, FR>(m, slot, ckpt, tau, Tn, k, gqT, gqdT, gtraj, gq0, gqd0,
-                                                       gtau, gm_acc, ring))
+  ABASIM_FOR_EACH_WSLOT(m, wbackward_one<T, DT, ONCHIP, FR>(m, slot, act, ckpt, tau, Tn, k, gqT, gqdT, gtraj, gq0,
+                                                            gqd0, gtau, gm_acc, ring))
 }
 
 }  // namespace host

@@ -66,20 +66,20 @@
 
 namespace abasim {
 
-// Per-link tape of the world-aligned step, [link][field][lane]: orientation R, whose
-// first two columns give way, when the adjoint will read the tape, to the rotated
-// COM inertia R I_com R^T (the third column is the joint axis s); velocity v; U;
-// 1/D (hi/lo pair); u, then the adjoint's wb; the joint offset d; and for the adjoint
-// a', qdd, the joint rate qd and the COM offset R com.
+// Per-link tape of the world-aligned step, [link][field][lane]: U; 1/D (hi/lo pair); u,
+// then the adjoint's wb; orientation R, whose first two columns give way, when the
+// adjoint will read the tape, to the rotated COM inertia R I_com R^T (the third column
+// is the joint axis s); velocity v; the joint offset d; and for the adjoint a', qdd, the
+// joint rate qd and the COM offset R com.  Ordered so that what a pass reads is one range.
 enum : int {
-  W_R = 0, W_V = 9, W_U = 15, W_DI = 21, W_u = 23, W_D = 24, W_AP = 27, W_QDD = 33, W_QD = 34, W_RW = 35, NWT = 38
+  W_U = 0, W_DI = 6, W_u = 8, W_R = 9, W_V = 18, W_D = 24, W_AP = 27, W_QDD = 33, W_QD = 34, W_RW = 35, NWT = 38
 };
 // Record of a free root (FR kernels; link 0 only), [field][lane]: its articulated
-// inertia, qdd, and the quaternion and velocity the step started from.  Its link's
-// tape words hold R whole, the rotated COM inertia in W_U and its acceleration in W_AP.
-enum : int { WF_IA = 0, WF_QDD = 21, WF_Q = 27, WF_QD = 31, NWF = 37 };
-// Per-link adjoint record, [link][field][lane]: W = -w and lambda.
-enum : int { WA_W = 0, WA_L = 6, NWA = 7 };
+// inertia, qdd, the quaternion and velocity the step started from and the rotated COM
+// inertia.  Its link's tape words hold R whole and its acceleration in W_AP.
+enum : int { WF_IA = 0, WF_QDD = 21, WF_Q = 27, WF_QD = 31, WF_IC = 37, NWF = 43 };
+// Per-link adjoint record, [link][field][lane]: W = -w.
+enum : int { WA_W = 0, NWA = 6 };
 // One entry of the stack of parent values, [entry][field][lane]: (R, v), a or W in
 // the outward passes, (shift(I^a, d), p^a), y or the adjoints of (v, a, W) in the
 // passes that run leaves -> root.
@@ -89,7 +89,8 @@ constexpr int WSW = 27;
 constexpr int NPRM_W = P_DAMP + 1;
 
 // View of one system for the world-aligned step (pointers at this system's lane).
-template <class T> struct WSys {
+// STG: the records are in global memory and each pass stages them through `ring`.
+template <class T, bool STG = false> struct WSys {
   const T* prm;     // [maxL][pstride][LANES]
   const int* meta;  // [maxL][LANES] ints, mstride apart
   T* tape;          // [maxL][NWT][LANES]
@@ -97,30 +98,114 @@ template <class T> struct WSys {
   int nl;
   int mstride = 1;
   int pstride = NPRM;
-  int pf = 0;  // prm, meta, tape and adj in global memory: prefetch this many links ahead (0: none)
   T* stk = nullptr;  // [entry][WSW][LANES]: the stack of parent values (see the tree data flow above)
   T* root = nullptr; // [NWF][LANES]: the free root's record (FR only)
+  int links = -1;    // STG: links the warp walks (its longest system's; every lane walks them together)
+  T* ring = nullptr; // STG: this warp's ring in shared memory, [ahead + 1][rows][LANES], at lane 0
+  int ahead = 2;     // STG: links a record is fetched ahead of its use, 0 .. RING_AHEAD
+  int lane = 0;
   SD T P(int l, int f) const { return prm[(l * pstride + f) * LANES]; }
   SD int M(int l) const { return meta[l * LANES * mstride]; }
   SD T& tp(int l, int f) const { return tape[(l * NWT + f) * LANES]; }
   SD T& ad(int l, int f) const { return adj[(l * NWA + f) * LANES]; }
+  SD int walk() const { return STG ? links : nl; }
 };
 
-// Prefetch into L1 of the cache lines holding fields [f0, f0 + n) of link l of a
-// [link][stride][LANES] global array (a warp's 32 lanes share each line).  The
-// passes run one thread per system through its links in a fixed order and
-// touch the same fields of every link, so they ask for link l +- pf's lines while
-// link l computes (pf from sim_set_prefetch, 2 by default): with a global tape, a
-// warp then waits for memory once per pass instead of once per link.
-SD void pf_line(const void* p) {
-#ifdef __CUDA_ARCH__
-  asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
+// Staged records.  A pass walks its links in a fixed order and reads the same fields of
+// each, so with the records in global memory the warp copies the next links' rows (32
+// systems' words of one field, 128 or 256 bytes) into a shared-memory ring with 16-byte
+// cp.async a few links ahead, and the pass reads shared memory.  Prefetching the same
+// lines into L1 left the passes waiting for L2 (27 % L1 hits: the tape's lines have been
+// written since); with the ring a 64-link chain tile's rollout step went from 123 to 86 us,
+// 1500 trees of 2-40 links with segment replay from 17.3 to 12.6 ms over 48 steps.  It
+// takes 3 x rows x 128 bytes a warp and a quarter of the instructions (four rows each).
+constexpr int RING_AHEAD = 2;
+// rows a warp's ring needs: the forward passes', the adjoint passes'
+constexpr int RING_FWD = 29, RING_ADJ = 36;
+// producers of the pipelined adjoint at most, each with a tape; in global memory, one stack
+// of parent values for each of its warps is beside them
+constexpr int WPIPE_TAPES = 3;
+
+#ifdef __CUDACC__
+__device__ __forceinline__ void stage_cp16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void stage_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+__device__ __forceinline__ void stage_wait(int newer) {  // all but the `newer` newest groups are in place
+  if (newer >= 2)
+    asm volatile("cp.async.wait_group 2;\n" ::: "memory");
+  else if (newer == 1)
+    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+  else
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+}
 #endif
-}
-template <class T> SD void pf_fields(const T* base, int stride, int l, int f0, int n) {
-  for (int i = 0; i < n; ++i) pf_line(base + (l * stride + f0 + i) * LANES);
-}
-template <class T> SD void pf_meta(const WSys<T>& s, int l) { pf_line(s.meta + l * LANES * s.mstride); }
+
+// The records of one pass over `n` links from `first` in steps of `dir`: tape fields
+// [TF, TF + TN), model constants [PF, PF + PN), adjoint fields [AF, AF + AN).  next() makes
+// the following link's records readable through t, p and a (indexed by field; at this
+// lane).  All lanes of the warp call it together when staging.
+template <class T, bool STG, int TF, int TN, int PF, int PN, int AF = 0, int AN = 0> struct Records {
+  static constexpr int ROWS = TN + PN + AN;
+  static_assert(ROWS <= RING_ADJ, "ring rows");
+  const WSys<T, STG>& s;
+  int first, dir, n, i = 0, slot = 0, fill = 0;
+  const T *t = nullptr, *p = nullptr, *a = nullptr;
+  SD Records(const WSys<T, STG>& sys, int first_, int dir_, int n_) : s(sys), first(first_), dir(dir_), n(n_) {
+    if constexpr (STG) {
+#ifdef __CUDA_ARCH__
+      __syncwarp();  // the previous pass has read its last slot and written its records
+      for (int j = 0; j < s.ahead; ++j) fetch(j);
+#endif
+    }
+  }
+  SD void fetch(int j) {
+#ifdef __CUDA_ARCH__
+    if (j < n) {
+      const int l = first + dir * j;
+      constexpr int PER = 16 / sizeof(T), CH = LANES / PER;  // words per copy, copies per row
+      T* dst = s.ring + (long long)fill * ROWS * LANES;
+      copy<TN * CH>(dst, s.tape - s.lane + (l * NWT + TF) * LANES);
+      copy<PN * CH>(dst + TN * LANES, s.prm - s.lane + (l * s.pstride + PF) * LANES);
+      if (AN) copy<AN * CH>(dst + (TN + PN) * LANES, s.adj - s.lane + (l * NWA + AF) * LANES);
+    }
+    fill = fill == s.ahead ? 0 : fill + 1;
+    stage_commit();
+#endif
+  }
+  template <int COPIES> SD void copy(T* dst, const T* src) {
+#ifdef __CUDA_ARCH__
+    constexpr int PER = 16 / sizeof(T);
+#pragma unroll
+    for (int c0 = 0; c0 < COPIES; c0 += LANES) {
+      const int c = c0 + s.lane;
+      if (c0 + LANES <= COPIES || c < COPIES) stage_cp16(dst + c * PER, src + c * PER);
+    }
+#endif
+  }
+  SD void next() {
+    if constexpr (STG) {
+#ifdef __CUDA_ARCH__
+      __syncwarp();  // every lane is done with the slot that is filled next
+      fetch(i + s.ahead);
+      stage_wait(s.ahead);
+      __syncwarp();
+      const T* r = s.ring + (long long)slot * ROWS * LANES + s.lane;
+      t = r - TF * LANES;
+      p = r + (TN - PF) * LANES;
+      a = r + (TN + PN - AF) * LANES;
+      slot = slot == s.ahead ? 0 : slot + 1;
+#endif
+    } else {
+      const int l = first + dir * i;
+      t = s.tape + l * NWT * LANES;
+      p = s.prm + l * s.pstride * LANES;
+      a = s.adj + l * NWA * LANES;
+    }
+    ++i;
+  }
+};
 
 template <class T> SD V3<T> wv3(T* base, int stride, int l, int f) {
   const T* p = base + (l * stride + f) * LANES;
@@ -164,39 +249,34 @@ template <class T> SD void wsi(T* base, int stride, int l, int f, const SI<T>& v
   ws3(base, stride, l, f + 15, v.C);
 }
 
-// field helpers of a link: model constants, the joint axis, the rotated COM inertia in
-// the first two columns of the tape's R, and 1/D
-template <class T> SD V3<T> wprm_v3(const WSys<T>& s, int l, int f) { return {s.P(l, f), s.P(l, f + 1), s.P(l, f + 2)}; }
-template <class T> SD M3<T> wprm_m3(const WSys<T>& s, int l, int f) {
+// fields of one record (a pointer at this lane, rows LANES apart)
+template <class T> SD T fld(const T* r, int f) { return r[f * LANES]; }
+template <class T> SD V3<T> fld_v3(const T* r, int f) { return {fld(r, f), fld(r, f + 1), fld(r, f + 2)}; }
+template <class T> SD SV<T> fld_sv(const T* r, int f) { return {fld_v3(r, f), fld_v3(r, f + 3)}; }
+template <class T> SD S3<T> fld_s3(const T* r, int f) {
+  return {fld(r, f), fld(r, f + 1), fld(r, f + 2), fld(r, f + 3), fld(r, f + 4), fld(r, f + 5)};
+}
+template <class T> SD M3<T> fld_m3(const T* r, int f) {
   M3<T> m;
-  for (int i = 0; i < 9; ++i) m.a[i] = s.P(l, f + i);
+  for (int i = 0; i < 9; ++i) m.a[i] = fld(r, f + i);
   return m;
 }
-template <class T> SD S3<T> wprm_s3(const WSys<T>& s, int l, int f) {
-  return {s.P(l, f), s.P(l, f + 1), s.P(l, f + 2), s.P(l, f + 3), s.P(l, f + 4), s.P(l, f + 5)};
+// the joint axis: the third column of the record's R
+template <class T> SD V3<T> fld_axis(const T* r) { return {fld(r, W_R + 2), fld(r, W_R + 5), fld(r, W_R + 8)}; }
+// the rotated COM inertia in the first two columns of the record's R
+template <class T> SD S3<T> fld_inertia(const T* r) {
+  return {fld(r, W_R), fld(r, W_R + 1), fld(r, W_R + 3), fld(r, W_R + 4), fld(r, W_R + 6), fld(r, W_R + 7)};
 }
-template <class T> SD V3<T> wcol2(const T* tp, int l) {
-  const T* p = tp + (l * NWT + W_R) * LANES;
-  return {p[2 * LANES], p[5 * LANES], p[8 * LANES]};
+template <class T> SD void put_inertia(T* r, const S3<T>& v) {
+  const T x[6] = {v.xx, v.yy, v.zz, v.xy, v.xz, v.yz};
+  for (int i = 0; i < 6; ++i) r[(W_R + i + i / 2) * LANES] = x[i];
 }
-template <class T> SD void pf_col2(const T* tp, int stride, int l) {
-  for (int i = 2; i < 9; i += 3) pf_line(tp + (l * stride + W_R + i) * LANES);
-}
-template <class T> SD void put_inertia(const WSys<T>& s, int l, const S3<T>& v) {
-  s.tp(l, W_R) = v.xx; s.tp(l, W_R + 1) = v.yy; s.tp(l, W_R + 3) = v.zz;
-  s.tp(l, W_R + 4) = v.xy; s.tp(l, W_R + 6) = v.xz; s.tp(l, W_R + 7) = v.yz;
-}
-template <class T> SD S3<T> get_inertia(const WSys<T>& s, int l) {
-  return {s.tp(l, W_R), s.tp(l, W_R + 1), s.tp(l, W_R + 3), s.tp(l, W_R + 4), s.tp(l, W_R + 6), s.tp(l, W_R + 7)};
-}
-template <class T, class DT> SD void put_wdi(const WSys<T>& s, int l, DT di) {
+template <class T, class DT> SD void put_wdi(T* r, DT di) {
   const T hi = (T)di;
-  s.tp(l, W_DI) = hi;
-  s.tp(l, W_DI + 1) = (T)(di - (DT)hi);
+  r[W_DI * LANES] = hi;
+  r[(W_DI + 1) * LANES] = (T)(di - (DT)hi);
 }
-template <class T, class DT> SD DT get_wdi(const WSys<T>& s, int l) {
-  return (DT)s.tp(l, W_DI) + (DT)s.tp(l, W_DI + 1);
-}
+template <class T, class DT> SD DT fld_wdi(const T* r) { return (DT)fld(r, W_DI) + (DT)fld(r, W_DI + 1); }
 
 // ------------------------------------------------------------------ operators
 // third column of a rotation (the joint axis of a link turning about its z axis)
@@ -251,6 +331,42 @@ template <class T> SD SV<T> shift_force(SV<T> f, V3<T> d) { return {f.w + cross(
 // X m for X = (1, d): the parent's motion seen at the child's origin
 template <class T> SD SV<T> shift_motion(SV<T> m, V3<T> d) { return {m.w, m.v - cross(d, m.w)}; }
 
+// Per-link scalars of a pass from two coordinate columns (a at the link's position or
+// velocity offset, b at its velocity offset), read one link ahead of their use and the
+// meta words two ahead, so that no link waits for its own loads.
+template <class T, bool STG, bool AQ> struct Inputs {
+  const WSys<T, STG>& s;
+  Col<const T> ca, cb;
+  int l, dir, n, m1, m2;
+  T a1, b1;
+  int m;   // the link's meta word
+  T a, b;  // its scalars
+  SD Inputs(const WSys<T, STG>& sys, Col<const T> a_, Col<const T> b_, int first, int dir_, int n_)
+      : s(sys), ca(a_), cb(b_), l(first), dir(dir_), n(n_) {
+    m1 = m2 = 0;
+    a1 = b1 = T(0);
+    if (n > 0 && s.nl > 0) {
+      m1 = s.M(first);
+      m2 = n > 1 ? s.M(first + dir) : m1;
+      a1 = ca[AQ ? meta_qoff(m1) : meta_voff(m1)];
+      b1 = cb[meta_voff(m1)];
+    }
+  }
+  SD void next() {  // the scalars of the following link
+    m = m1;
+    a = a1;
+    b = b1;
+    m1 = m2;
+    if (!STG || s.nl > 0) {
+      a1 = ca[AQ ? meta_qoff(m1) : meta_voff(m1)];
+      b1 = cb[meta_voff(m1)];
+    }
+    const int l2 = l + 2 * dir;
+    if (l2 >= 0 && l2 < n) m2 = s.M(l2);
+    l += dir;
+  }
+};
+
 // ------------------------------------------------------------------ forward
 // a body's own terms: inertia about its joint in world axes and bias force, from its
 // COM inertia Ic and COM offset rw in world axes.  With vc the COM velocity the
@@ -272,66 +388,62 @@ template <class T> SD void body_terms(T m, V3<T> rw, const S3<T>& Ic, SV<T> v, S
 // alias q, qd: a link's own coordinates are read before they are written, and no
 // pass after it reads the state).  FR: link 0 may be a free joint (R = E_tree^T R(quat),
 // S = R on both halves, so D = I^A in world axes: one Cholesky solve).
-template <class T, class DT, bool ADJ, bool INTEG, bool FR = false>
-SD void wstep_forward(const WSys<T>& s, Col<const T> q, Col<const T> qd, Col<const T> tau, V3<T> grav, T dt,
+template <class T, class DT, bool ADJ, bool INTEG, bool FR = false, bool STG = false>
+SD void wstep_forward(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd, Col<const T> tau, V3<T> grav, T dt,
                       int integ, Col<T> qo, Col<T> qdo) {
   T* tp = s.tape;
-  const int nl = s.nl;
+  const int nl = s.nl, walk = s.walk();
   // outward: orientation, joint offset, velocity (a root takes R_p = 1, v_p = 0,
   // which gives its values exactly)
   {
+    Records<T, STG, 0, 0, P_E, 12> rec(s, 0, 1, walk);
+    Inputs<T, STG, true> in(s, q, qd, 0, 1, walk);
     M3<T> R_prev = eye3<T>();
     SV<T> v_prev = zeroSV<T>();
     int sp = 0;  // entries on the stack
-    for (int l = 0; l < nl; ++l) {
-      if (s.pf > 0 && l + s.pf < nl) {
-        pf_meta(s, l + s.pf);
-        pf_fields(s.prm, s.pstride, l + s.pf, P_E, 12);
-      }
-      const int m = s.M(l);
-      const int par = meta_parent(m);
+    for (int l = 0; l < walk; ++l) {
+      rec.next();
+      in.next();
+      if (STG && l >= nl) continue;
+      const int m = in.m;
+      const int par = meta_parent(m), qi = meta_qoff(m), vi = meta_voff(m);
+      T* w = tp + l * NWT * LANES;
+      M3<T> R;
+      SV<T> v;
       if (FR && meta_jtype(m) == J_FREE) {
-        const int qo = meta_qoff(m), vo = meta_voff(m);
-        const T qt[4] = {q[qo + 3], q[qo + 4], q[qo + 5], q[qo + 6]};
-        T w[6];
-        for (int i = 0; i < 6; ++i) w[i] = qd[vo + i];
-        R_prev = mTm(wprm_m3(s, l, P_E), quat_R(qt[0], qt[1], qt[2], qt[3]));
-        v_prev = SV<T>{mul(R_prev, V3<T>{w[0], w[1], w[2]}), mul(R_prev, V3<T>{w[3], w[4], w[5]})};
-        wm3(tp, NWT, l, W_R, R_prev);
-        wsv(tp, NWT, l, W_V, v_prev);
+        const T qt[4] = {q[qi + 3], q[qi + 4], q[qi + 5], q[qi + 6]};
+        T x[6];
+        for (int i = 0; i < 6; ++i) x[i] = qd[vi + i];
+        R = mTm(fld_m3(rec.p, P_E), quat_R(qt[0], qt[1], qt[2], qt[3]));
+        v = SV<T>{mul(R, V3<T>{x[0], x[1], x[2]}), mul(R, V3<T>{x[3], x[4], x[5]})};
         if (ADJ) {
           for (int i = 0; i < 4; ++i) s.root[(WF_Q + i) * LANES] = qt[i];
-          for (int i = 0; i < 6; ++i) s.root[(WF_QD + i) * LANES] = w[i];
+          for (int i = 0; i < 6; ++i) s.root[(WF_QD + i) * LANES] = x[i];
         }
-        if (meta_treechild(m)) {
-          wm3(s.stk, WSW, sp, 0, R_prev);
-          wsv(s.stk, WSW, sp, 9, v_prev);
-          ++sp;
+      } else {
+        T sn, cs;
+        sincos_t(in.a, &sn, &cs);
+        const T vl = in.b;
+        const M3<T> E = rotz_T_mm(sn, cs, fld_m3(rec.p, P_E));
+        M3<T> Rp = R_prev;
+        SV<T> vp = v_prev;
+        if (par < 0) {
+          Rp = eye3<T>();
+          vp = zeroSV<T>();
+        } else if (par != l - 1) {
+          Rp = wm3(s.stk, WSW, sp - 1, 0);
+          vp = wsv(s.stk, WSW, sp - 1, 9);
+          if (meta_lastsib(m)) --sp;
         }
-        continue;
+        const V3<T> d = mul(Rp, fld_v3(rec.p, P_R));
+        R = mmT(Rp, E);
+        v = shift_motion(vp, d);
+        v.w += vl * col2(R);
+        wv3(w, 0, 0, W_D, d);
+        if (ADJ) w[W_QD * LANES] = vl;
       }
-      T sn, cs;
-      sincos_t(q[meta_qoff(m)], &sn, &cs);
-      const T vl = qd[meta_voff(m)];
-      const M3<T> E = rotz_T_mm(sn, cs, wprm_m3(s, l, P_E));
-      M3<T> Rp = R_prev;
-      SV<T> vp = v_prev;
-      if (par < 0) {
-        Rp = eye3<T>();
-        vp = zeroSV<T>();
-      } else if (par != l - 1) {
-        Rp = wm3(s.stk, WSW, sp - 1, 0);
-        vp = wsv(s.stk, WSW, sp - 1, 9);
-        if (meta_lastsib(m)) --sp;
-      }
-      const V3<T> d = mul(Rp, wprm_v3(s, l, P_R));
-      const M3<T> R = mmT(Rp, E);
-      SV<T> v = shift_motion(vp, d);
-      v.w += vl * col2(R);
-      wv3(tp, NWT, l, W_D, d);
-      wm3(tp, NWT, l, W_R, R);
-      wsv(tp, NWT, l, W_V, v);
-      if (ADJ) s.tp(l, W_QD) = vl;
+      wm3(w, 0, 0, W_R, R);
+      wsv(w, 0, 0, W_V, v);
       if (meta_treechild(m)) {
         wm3(s.stk, WSW, sp, 0, R);
         wsv(s.stk, WSW, sp, 9, v);
@@ -344,37 +456,40 @@ SD void wstep_forward(const WSys<T>& s, Col<const T> q, Col<const T> qd, Col<con
   // inward: articulated inertias and bias forces, from each link's own terms and its
   // children's contributions
   {
+    Records<T, STG, W_R, W_AP - W_R, P_M, NPRM_W - P_M> rec(s, walk - 1, -1, walk);
+    Inputs<T, STG, false> in(s, tau, qd, walk - 1, -1, walk);
     SI<T> cI = zeroSI<T>();  // link l + 1's contribution when l is its parent
     SV<T> cp = zeroSV<T>();
     bool carry = false;
     int sp = 0;
-    for (int l = nl - 1; l >= 0; --l) {
-      if (s.pf > 0 && l - s.pf >= 0) {
-        pf_fields(tp, NWT, l - s.pf, W_R, 15);
-        pf_fields(tp, NWT, l - s.pf, W_D, 3);
-        pf_fields(s.prm, s.pstride, l - s.pf, P_M, NPRM_W - P_M);
-      }
-      const int m = s.M(l);
+    for (int l = walk - 1; l >= 0; --l) {
+      rec.next();
+      in.next();
+      if (STG && l >= nl) continue;
+      const int m = in.m;
       const int par = meta_parent(m), vo = meta_voff(m);
-      const M3<T> R = wm3(tp, NWT, l, W_R);
-      const SV<T> v = wsv(tp, NWT, l, W_V);
+      T* w = tp + l * NWT * LANES;
       const bool fr = FR && meta_jtype(m) == J_FREE;
+      const M3<T> R = fld_m3(rec.t, W_R);
+      const SV<T> v = fld_sv(rec.t, W_V);
       const V3<T> sx = col2(R);
-      const T vl = qd[vo];
-      const T tl = tau[vo] - s.P(l, P_DAMP) * vl;
+      const T vl = in.b;
+      const T tl = in.a - fld(rec.p, P_DAMP) * vl;
       const V3<T> sq = vl * sx;
       const SV<T> c{cross(v.w, sq), cross(v.v, sq)};
-      const S3<T> Ic = rot_sym(R, wprm_s3(s, l, P_IC));
-      const V3<T> rw = mul(R, wprm_v3(s, l, P_C));
+      const S3<T> Ic = rot_sym(R, fld_s3(rec.p, P_IC));
+      const V3<T> rw = mul(R, fld_v3(rec.p, P_C));
       SI<T> IA;
       SV<T> pA;
-      body_terms(s.P(l, P_M), rw, Ic, v, IA, pA);
+      body_terms(fld(rec.p, P_M), rw, Ic, v, IA, pA);
+      // the joint offset, 0 for a root (whose contribution to a parent is dropped)
+      V3<T> d = fld_v3(rec.t, W_D);
       if (ADJ) {
         if (fr)
-          ws3(tp, NWT, l, W_U, Ic);
+          ws3(s.root, 0, 0, WF_IC, Ic);
         else
-          put_inertia(s, l, Ic);
-        wv3(tp, NWT, l, W_RW, rw);
+          put_inertia(w, Ic);
+        wv3(w, 0, 0, W_RW, rw);
       }
       if (carry) {
         IA += cI;
@@ -389,17 +504,15 @@ SD void wstep_forward(const WSys<T>& s, Col<const T> q, Col<const T> qd, Col<con
         const SV<T> f{mul(R, V3<T>{tau[vo], tau[vo + 1], tau[vo + 2]}),
                       mul(R, V3<T>{tau[vo + 3], tau[vo + 4], tau[vo + 5]})};
         if (ADJ) wsi(s.root, 0, 0, WF_IA, IA);
-        wsv(tp, NWT, l, W_AP, spd_solve<T, DT>(IA, f - pA));
+        wsv(w, 0, 0, W_AP, spd_solve<T, DT>(IA, f - pA));
         continue;
       }
       const SV<T> U{mul(IA.A, sx), mulT(IA.B, sx)};
       const DT Di = DT(1) / (DT)dot(sx, U.w);
       const T u = tl - dot(sx, pA.w);
-      wsv(tp, NWT, l, W_U, U);
-      put_wdi<T, DT>(s, l, Di);
-      s.tp(l, W_u) = u;
-      // the contribution to the parent (computed for a root too, with d = 0, and dropped)
-      V3<T> d = wv3(tp, NWT, l, W_D);
+      wsv(w, 0, 0, W_U, U);
+      put_wdi<T, DT>(w, Di);
+      w[W_u * LANES] = u;
       if (par < 0) d = zero3<T>();
       const SI<T> Ia = minus_scaled_outer<T, DT>(IA, Di, U);
       const SV<T> pa = pA + mul(Ia, c) + (T)((DT)u * Di) * U;
@@ -420,26 +533,27 @@ SD void wstep_forward(const WSys<T>& s, Col<const T> q, Col<const T> qd, Col<con
     }
   }
   // outward: accelerations (and the integrator)
+  Records<T, STG, 0, W_AP, 0, 0> rec(s, 0, 1, walk);
+  Inputs<T, STG, true> in(s, q, qd, 0, 1, walk);
   const SV<T> a0{zero3<T>(), -grav};
   SV<T> a_prev = a0;
   int sp = 0;
-  for (int l = 0; l < nl; ++l) {
-    if (s.pf > 0 && l + s.pf < nl) {
-      pf_fields(tp, NWT, l + s.pf, W_R, W_AP - W_R);
-    }
-    const int m = s.M(l);
+  for (int l = 0; l < walk; ++l) {
+    rec.next();
+    in.next();
+    if (STG && l >= nl) continue;
+    const int m = in.m;
     const int par = meta_parent(m), vi = meta_voff(m);
+    T* w = tp + l * NWT * LANES;
+    SV<T> a;
     if (FR && meta_jtype(m) == J_FREE) {
-      const M3<T> R = wm3(tp, NWT, l, W_R);
-      const SV<T> a = wsv(tp, NWT, l, W_AP), b = a - a0;
+      const M3<T> R = fld_m3(rec.t, W_R);
+      a = wsv(w, 0, 0, W_AP);
+      const SV<T> b = a - a0;
       const V3<T> bw = mulT(R, b.w), bv = mulT(R, b.v);
       const T qdd[6] = {bw.x, bw.y, bw.z, bv.x, bv.y, bv.z};
       if (ADJ)
         for (int i = 0; i < 6; ++i) s.root[(WF_QDD + i) * LANES] = qdd[i];
-      if (meta_treechild(m)) {
-        wsv(s.stk, WSW, sp, 0, a);
-        ++sp;
-      }
       if (INTEG) {
         const int qi = meta_qoff(m);
         T nu[6], x[7];
@@ -453,42 +567,41 @@ SD void wstep_forward(const WSys<T>& s, Col<const T> q, Col<const T> qd, Col<con
         free_advance(x, nu, dt);
         for (int i = 0; i < 7; ++i) qo[qi + i] = x[i];
       }
-      a_prev = a;
-      continue;
-    }
-    const V3<T> sx = col2(wm3(tp, NWT, l, W_R));
-    const SV<T> v = wsv(tp, NWT, l, W_V);
-    const SV<T> U = wsv(tp, NWT, l, W_U);
-    const DT Di = get_wdi<T, DT>(s, l);
-    const T u = s.tp(l, W_u);
-    const T v0 = qd[vi];
-    const V3<T> sq = v0 * sx;
-    SV<T> ap = a0;
-    if (par >= 0) {
-      SV<T> apar = a_prev;
-      if (par != l - 1) {
-        apar = wsv(s.stk, WSW, sp - 1, 0);
-        if (meta_lastsib(m)) --sp;
+    } else {
+      const V3<T> sx = fld_axis(rec.t);
+      const SV<T> v = fld_sv(rec.t, W_V);
+      const SV<T> U = fld_sv(rec.t, W_U);
+      const DT Di = fld_wdi<T, DT>(rec.t);
+      const T u = fld(rec.t, W_u);
+      const T v0 = in.b;
+      const V3<T> sq = v0 * sx;
+      SV<T> ap = a0;
+      if (par >= 0) {
+        SV<T> apar = a_prev;
+        if (par != l - 1) {
+          apar = wsv(s.stk, WSW, sp - 1, 0);
+          if (meta_lastsib(m)) --sp;
+        }
+        ap = shift_motion(apar, fld_v3(rec.t, W_D));
       }
-      ap = shift_motion(apar, wv3(tp, NWT, l, W_D));
-    }
-    ap += SV<T>{cross(v.w, sq), cross(v.v, sq)};
-    const T qdd = (T)(((DT)u - (DT)dot(U, ap)) * Di);
-    const SV<T> a{ap.w + qdd * sx, ap.v};
-    if (ADJ) {
-      wsv(tp, NWT, l, W_AP, ap);
-      s.tp(l, W_QDD) = qdd;
+      ap += SV<T>{cross(v.w, sq), cross(v.v, sq)};
+      const T qdd = (T)(((DT)u - (DT)dot(U, ap)) * Di);
+      a = SV<T>{ap.w + qdd * sx, ap.v};
+      if (ADJ) {
+        wsv(w, 0, 0, W_AP, ap);
+        w[W_QDD * LANES] = qdd;
+      }
+      if (INTEG) {
+        const int qi = meta_qoff(m);
+        const T v1 = v0 + dt * qdd;
+        const T q1 = in.a + dt * (integ == I_SEMI_IMPLICIT ? v1 : v0);
+        qdo[vi] = v1;
+        qo[qi] = q1;
+      }
     }
     if (meta_treechild(m)) {
       wsv(s.stk, WSW, sp, 0, a);
       ++sp;
-    }
-    if (INTEG) {
-      const int qi = meta_qoff(m);
-      const T v1 = v0 + dt * qdd;
-      const T q1 = q[qi] + dt * (integ == I_SEMI_IMPLICIT ? v1 : v0);
-      qdo[vi] = v1;
-      qo[qi] = q1;
     }
     a_prev = a;
   }
@@ -521,24 +634,29 @@ template <class T> SD BodyGrad<T> body_grad(T m, V3<T> rw, const S3<T>& Ic, SV<T
 // (gq, gqd) hold the adjoint of x^{k+1}; on exit that of x^k.  Writes the adjoint
 // of tau into gtau and adds dPhi/dm of every link into gm.  FR (link 0 may be a free
 // joint) needs the gravity: the only motion a free root's orientation turns against.
-template <class T, class DT, bool FR = false>
-SD void wstep_adjoint(const WSys<T>& s, Col<T> gq, Col<T> gqd, Col<T> gtau, Col<T> gm, T dt, int integ,
+template <class T, class DT, bool FR = false, bool STG = false>
+SD void wstep_adjoint(const WSys<T, STG>& s, Col<T> gq, Col<T> gqd, Col<T> gtau, Col<T> gm, T dt, int integ,
                       V3<T> grav = zero3<T>()) {
   T* tp = s.tape;
   T* ad = s.adj;
-  const int nl = s.nl;
+  const int nl = s.nl, walk = s.walk();
   // the integrator's adjoint and the inward half of lambda = M^-1 qddb (leaves -> root)
   {
+    Records<T, STG, 0, W_AP, 0, 0> rec(s, walk - 1, -1, walk);
     SV<T> cy = zeroSV<T>();
     bool carry = false;
     int sp = 0;
-    for (int l = nl - 1; l >= 0; --l) {
-      if (s.pf > 0 && l - s.pf >= 0) {
-        pf_col2(tp, NWT, l - s.pf);
-        pf_fields(tp, NWT, l - s.pf, W_U, W_AP - W_U);
-      }
+    for (int l = walk - 1; l >= 0; --l) {
+      rec.next();
+      if (STG && l >= nl) continue;
       const int m = s.M(l);
       const int par = meta_parent(m), qi = meta_qoff(m), vi = meta_voff(m);
+      SV<T> y = carry ? cy : zeroSV<T>();
+      carry = false;
+      if (meta_treechild(m)) {
+        --sp;
+        y += wsv(s.stk, WSW, sp, 0);
+      }
       if (FR && meta_jtype(m) == J_FREE) {  // lambda_root = (I^A)^-1 (R qddb + y)
         T qt[4], nu[6], qddb6[6];
         for (int i = 0; i < 4; ++i) qt[i] = s.root[(WF_Q + i) * LANES];
@@ -547,23 +665,13 @@ SD void wstep_adjoint(const WSys<T>& s, Col<T> gq, Col<T> gqd, Col<T> gtau, Col<
           if (integ == I_SEMI_IMPLICIT) nu[i] += dt * s.root[(WF_QDD + i) * LANES];
         }
         free_integrator_adjoint(qt, nu, gq, gqd, qi, vi, dt, integ, qddb6);
-        const M3<T> R = wm3(tp, NWT, l, W_R);
-        SV<T> y{mul(R, V3<T>{qddb6[0], qddb6[1], qddb6[2]}), mul(R, V3<T>{qddb6[3], qddb6[4], qddb6[5]})};
-        if (carry) y += cy;
-        carry = false;
-        if (meta_treechild(m)) {
-          --sp;
-          y += wsv(s.stk, WSW, sp, 0);
-        }
+        const M3<T> R = fld_m3(rec.t, W_R);
+        y += SV<T>{mul(R, V3<T>{qddb6[0], qddb6[1], qddb6[2]}), mul(R, V3<T>{qddb6[3], qddb6[4], qddb6[5]})};
         const SV<T> w = spd_solve<T, DT>(wsi(s.root, 0, 0, WF_IA), y);
         wsv(ad, NWA, l, WA_W, zeroSV<T>() - w);
         const V3<T> lw = mulT(R, w.w), lv = mulT(R, w.v);
-        gtau[vi] = lw.x;
-        gtau[vi + 1] = lw.y;
-        gtau[vi + 2] = lw.z;
-        gtau[vi + 3] = lv.x;
-        gtau[vi + 4] = lv.y;
-        gtau[vi + 5] = lv.z;
+        const T lam[6] = {lw.x, lw.y, lw.z, lv.x, lv.y, lv.z};
+        for (int i = 0; i < 6; ++i) gtau[vi + i] = lam[i];
         continue;
       }
       T qddb;
@@ -573,18 +681,12 @@ SD void wstep_adjoint(const WSys<T>& s, Col<T> gq, Col<T> gqd, Col<T> gtau, Col<
         gqd[vi] = vt;
         qddb = dt * (integ == I_SEMI_IMPLICIT ? vt : vb);
       }
-      SV<T> y = carry ? cy : zeroSV<T>();
-      carry = false;
-      if (meta_treechild(m)) {
-        --sp;
-        y += wsv(s.stk, WSW, sp, 0);
-      }
-      const V3<T> sx = wcol2(tp, l);
-      const SV<T> U = wsv(tp, NWT, l, W_U);
-      const T wb = (T)((DT)(qddb + dot(sx, y.w)) * get_wdi<T, DT>(s, l));
+      const V3<T> sx = fld_axis(rec.t);
+      const SV<T> U = fld_sv(rec.t, W_U);
+      const T wb = (T)((DT)(qddb + dot(sx, y.w)) * fld_wdi<T, DT>(rec.t));
       s.tp(l, W_u) = wb;
       if (par >= 0) {
-        const SV<T> yp = shift_force(y - wb * U, wv3(tp, NWT, l, W_D));
+        const SV<T> yp = shift_force(y - wb * U, fld_v3(rec.t, W_D));
         if (par == l - 1) {
           cy = yp;
           carry = true;
@@ -599,40 +701,33 @@ SD void wstep_adjoint(const WSys<T>& s, Col<T> gq, Col<T> gqd, Col<T> gtau, Col<
   }
   // the outward half: lambda, W = -w (root -> leaves)
   {
+    Records<T, STG, 0, W_AP, P_DAMP, 1> rec(s, 0, 1, walk);
     SV<T> W_prev = zeroSV<T>();
     int sp = 0;
-    for (int l = 0; l < nl; ++l) {
-      if (s.pf > 0 && l + s.pf < nl) {
-        pf_col2(tp, NWT, l + s.pf);
-        pf_fields(tp, NWT, l + s.pf, W_U, W_AP - W_U);
-        pf_line(s.prm + ((l + s.pf) * s.pstride + P_DAMP) * LANES);
-      }
+    for (int l = 0; l < walk; ++l) {
+      rec.next();
+      if (STG && l >= nl) continue;
       const int m = s.M(l);
       const int par = meta_parent(m), vi = meta_voff(m);
-      if (FR && meta_jtype(m) == J_FREE) {
-        W_prev = wsv(ad, NWA, l, WA_W);
-        if (meta_treechild(m)) {
-          wsv(s.stk, WSW, sp, 0, W_prev);
-          ++sp;
-        }
-        continue;
-      }
       SV<T> W = zeroSV<T>();
-      if (par >= 0) {
-        SV<T> Wp = W_prev;
-        if (par != l - 1) {
-          Wp = wsv(s.stk, WSW, sp - 1, 0);
-          if (meta_lastsib(m)) --sp;
+      if (FR && meta_jtype(m) == J_FREE) {
+        W = wsv(ad, NWA, l, WA_W);
+      } else {
+        if (par >= 0) {
+          SV<T> Wp = W_prev;
+          if (par != l - 1) {
+            Wp = wsv(s.stk, WSW, sp - 1, 0);
+            if (meta_lastsib(m)) --sp;
+          }
+          W = shift_motion(Wp, fld_v3(rec.t, W_D));
         }
-        W = shift_motion(Wp, wv3(tp, NWT, l, W_D));
+        const SV<T> U = fld_sv(rec.t, W_U);
+        const T lam = fld(rec.t, W_u) + (T)((DT)dot(U, W) * fld_wdi<T, DT>(rec.t));
+        W.w = W.w - lam * fld_axis(rec.t);
+        wsv(ad, NWA, l, WA_W, W);
+        gtau[vi] = lam;
+        gqd[vi] -= fld(rec.p, P_DAMP) * lam;
       }
-      const SV<T> U = wsv(tp, NWT, l, W_U);
-      const T lam = s.tp(l, W_u) + (T)((DT)dot(U, W) * get_wdi<T, DT>(s, l));
-      W.w = W.w - lam * wcol2(tp, l);
-      s.ad(l, WA_L) = lam;
-      wsv(ad, NWA, l, WA_W, W);
-      gtau[vi] = lam;
-      gqd[vi] -= s.P(l, P_DAMP) * lam;
       if (meta_treechild(m)) {
         wsv(s.stk, WSW, sp, 0, W);
         ++sp;
@@ -642,26 +737,23 @@ SD void wstep_adjoint(const WSys<T>& s, Col<T> gq, Col<T> gqd, Col<T> gtau, Col<
   }
   // the derivative of L (leaves -> root)
   {
+    Records<T, STG, W_R, NWT - W_R, P_M, 1, WA_W, 6> rec(s, walk - 1, -1, walk);
     SV<T> cv = zeroSV<T>(), ca = zeroSV<T>(), cw = zeroSV<T>();
     bool carry = false;
     int sp = 0;
-    for (int l = nl - 1; l >= 0; --l) {
-      if (s.pf > 0 && l - s.pf >= 0) {
-        pf_fields(tp, NWT, l - s.pf, W_R, 15);
-        pf_fields(tp, NWT, l - s.pf, W_D, NWT - W_D);
-        pf_fields(ad, NWA, l - s.pf, 0, NWA);
-        pf_line(s.prm + ((l - s.pf) * s.pstride + P_M) * LANES);
-      }
+    for (int l = walk - 1; l >= 0; --l) {
+      rec.next();
+      if (STG && l >= nl) continue;
       const int m = s.M(l);
       const int par = meta_parent(m), qi = meta_qoff(m), vi = meta_voff(m);
       const bool fr = FR && meta_jtype(m) == J_FREE;
-      const V3<T> sx = wcol2(tp, l);
-      const SV<T> v = wsv(tp, NWT, l, W_V), ap = wsv(tp, NWT, l, W_AP), W = wsv(ad, NWA, l, WA_W);
-      const T vl = fr ? T(0) : s.tp(l, W_QD);
-      const T qdd = fr ? T(0) : s.tp(l, W_QDD);
+      const V3<T> sx = fld_axis(rec.t);
+      const SV<T> v = fld_sv(rec.t, W_V), ap = fld_sv(rec.t, W_AP), W = fld_sv(rec.a, WA_W);
+      const T vl = fr ? T(0) : fld(rec.t, W_QD);
+      const T qdd = fr ? T(0) : fld(rec.t, W_QDD);
       const SV<T> a{ap.w + qdd * sx, ap.v};
-      const S3<T> Ic = fr ? ws3(tp, NWT, l, W_U) : get_inertia(s, l);
-      BodyGrad<T> g = body_grad(s.P(l, P_M), wv3(tp, NWT, l, W_RW), Ic, v, a, W);
+      const S3<T> Ic = fr ? ws3(s.root, 0, 0, WF_IC) : fld_inertia(rec.t);
+      BodyGrad<T> g = body_grad(fld(rec.p, P_M), fld_v3(rec.t, W_RW), Ic, v, a, W);
       gm[l] += g.mb;
       if (carry) {
         g.vb += cv;
@@ -676,11 +768,13 @@ SD void wstep_adjoint(const WSys<T>& s, Col<T> gq, Col<T> gqd, Col<T> gtau, Col<
         g.F += wsv(s.stk, WSW, sp, 12);
       }
       if (fr) {  // v = R qd, a = R qdd + [0; -g]: only the gravity does not turn with R
-        const M3<T> R = wm3(tp, NWT, l, W_R);
+        const M3<T> R = fld_m3(rec.t, W_R);
         const V3<T> bw = mulT(R, g.vb.w), bv = mulT(R, g.vb.v);
         const T vv[6] = {bw.x, bw.y, bw.z, bv.x, bv.y, bv.z};
         for (int i = 0; i < 6; ++i) gqd[vi + i] += vv[i];
-        const M3<T> EJb = mmT(outer(mulT(R, g.ab.v), zero3<T>() - grav), wprm_m3(s, l, P_E));  // E = E_J E_t
+        M3<T> Et;
+        for (int i = 0; i < 9; ++i) Et.a[i] = s.P(l, P_E + i);
+        const M3<T> EJb = mmT(outer(mulT(R, g.ab.v), zero3<T>() - grav), Et);  // E = E_J E_t
         T qb[4] = {T(0), T(0), T(0), T(0)};
         quat_R_adj(s.root[WF_Q * LANES], s.root[(WF_Q + 1) * LANES], s.root[(WF_Q + 2) * LANES],
                    s.root[(WF_Q + 3) * LANES], transpose(EJb), qb);
@@ -695,7 +789,7 @@ SD void wstep_adjoint(const WSys<T>& s, Col<T> gq, Col<T> gqd, Col<T> gtau, Col<
       // joint's own parts along s drop out)
       gq[qi] += dot(ap + vl * e, b) - dot(e, g.vb) - dot(sx, cross(W.w, g.F.w) + cross(W.v, g.F.v));
       if (par >= 0) {
-        const V3<T> d = wv3(tp, NWT, l, W_D);
+        const V3<T> d = fld_v3(rec.t, W_D);
         cv = shift_force(g.vb, d);
         ca = shift_force(g.ab, d);
         cw = shift_force(g.F, d);
