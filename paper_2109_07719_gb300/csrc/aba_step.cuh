@@ -23,6 +23,7 @@
 #endif
 
 #include "spatial.cuh"
+#include "twofloat.cuh"
 
 namespace abasim {
 
@@ -101,6 +102,7 @@ template <> SD void sincos_t<double>(double x, double* s, double* c) {
 #endif
 }
 template <class T> SD T sqrt_t(T x) { return sqrt(x); }
+template <> SD FF sqrt_t<FF>(FF x) { return ff_sqrt(x); }
 
 // Tape and adjoint layouts.  LAY_FULL holds every field (any tree, any joint).
 // The pipelined adjoint of serial chains of revolute joints uses two compact
@@ -279,8 +281,8 @@ template <class T> SD SV<T> chol6_solve(const T* L, SV<T> b) {
 
 // ------------------------------------------------------------------ D-solve scalar
 // The articulated-inertia solves (D = S^T I^A S, 1/D, U D^-1 U^T, the free root's
-// 6x6 solve) run in the scalar DT: the storage type T, or double in the mixed
-// FP32 + FP64 mode.  1/D is kept on the tape as a hi/lo pair of T words.
+// 6x6 solve) run in the scalar DT: the storage type T, or 48-bit float pairs in the
+// mixed mode (FF, twofloat.cuh).  1/D is kept on the tape as a hi/lo pair of T words.
 template <class T, class DT, class PT, int TL, int AL> SD void put_di(const Sys<T, PT, TL, AL>& s, int l, DT di) {
   const T hi = (T)di;
   s.tp(l, T_DI) = hi;
@@ -299,15 +301,19 @@ template <class DT, class T> SD SI<DT> si_cast(const SI<T>& I) {
 template <class DT, class T> SD SV<DT> sv_cast(const SV<T>& v) {
   return SV<DT>{{(DT)v.w.x, (DT)v.w.y, (DT)v.w.z}, {(DT)v.v.x, (DT)v.v.y, (DT)v.v.z}};
 }
-// I - di u u^T formed in DT, rounded to T
+// i - x u formed in DT, rounded to T
+template <class T, class DT> SD T minus_product(T i, DT x, T u) { return (T)((DT)i - x * (DT)u); }
+template <> SD float minus_product<float, FF>(float i, FF x, float u) { return ff_minus_product(i, x, u); }
+// I - di u u^T, each entry from x = di u formed in DT
 template <class T, class DT> SD SI<T> minus_scaled_outer(const SI<T>& I, DT di, SV<T> u) {
-  const SI<DT> Id = si_cast<DT>(I);
-  const SV<DT> ud = sv_cast<DT>(u);
-  const SI<DT> r = Id - scale(di, sym_outer(ud, ud));
+  const T v[6] = {u.w.x, u.w.y, u.w.z, u.v.x, u.v.y, u.v.z};
+  DT x[6];
+  for (int i = 0; i < 6; ++i) x[i] = di * (DT)v[i];
+  auto e = [&](T a, int i, int j) { return minus_product<T, DT>(a, x[i], v[j]); };
   SI<T> o;
-  o.A = S3<T>{(T)r.A.xx, (T)r.A.yy, (T)r.A.zz, (T)r.A.xy, (T)r.A.xz, (T)r.A.yz};
-  o.C = S3<T>{(T)r.C.xx, (T)r.C.yy, (T)r.C.zz, (T)r.C.xy, (T)r.C.xz, (T)r.C.yz};
-  for (int i = 0; i < 9; ++i) o.B.a[i] = (T)r.B.a[i];
+  o.A = S3<T>{e(I.A.xx, 0, 0), e(I.A.yy, 1, 1), e(I.A.zz, 2, 2), e(I.A.xy, 0, 1), e(I.A.xz, 0, 2), e(I.A.yz, 1, 2)};
+  for (int i = 0; i < 9; ++i) o.B.a[i] = e(I.B.a[i], i / 3, 3 + i % 3);
+  o.C = S3<T>{e(I.C.xx, 3, 3), e(I.C.yy, 4, 4), e(I.C.zz, 5, 5), e(I.C.xy, 3, 4), e(I.C.xz, 3, 5), e(I.C.yz, 4, 5)};
   return o;
 }
 // the free root's solve I^A x = b, Cholesky in DT

@@ -475,7 +475,7 @@ int sim_rollout(sim_handle* h, const void* q0, const void* qd0, const void* tau,
   switch (h->precision) {
     case SIM_FP64: return launch_rollout<double, double>(h, q0, qd0, tau, T, k, ckpt, qT, qdT, traj, stream);
     case SIM_FP32: return launch_rollout<float, float>(h, q0, qd0, tau, T, k, ckpt, qT, qdT, traj, stream);
-    default: return launch_rollout<float, double>(h, q0, qd0, tau, T, k, ckpt, qT, qdT, traj, stream);
+    default: return launch_rollout<float, FF>(h, q0, qd0, tau, T, k, ckpt, qT, qdT, traj, stream);
   }
 }
 
@@ -500,7 +500,7 @@ int sim_step_batch_static(sim_handle* h, const void* q, const void* qd, const vo
   switch (h->precision) {
     case SIM_FP64: return launch_step_static<double, double>(h, q, qd, tau, q_out, qd_out, stream);
     case SIM_FP32: return launch_step_static<float, float>(h, q, qd, tau, q_out, qd_out, stream);
-    default: return launch_step_static<float, double>(h, q, qd, tau, q_out, qd_out, stream);
+    default: return launch_step_static<float, FF>(h, q, qd, tau, q_out, qd_out, stream);
   }
 }
 
@@ -539,7 +539,7 @@ int sim_backward_rollout(sim_handle* h, const void* ckpt, const void* tau, int64
     case SIM_FP32:
       return launch_backward<float, float>(h, ckpt, tau, T, k, gqT, gqdT, g_traj, gq0, gqd0, gtau, gmass, work, stream);
     default:
-      return launch_backward<float, double>(h, ckpt, tau, T, k, gqT, gqdT, g_traj, gq0, gqd0, gtau, gmass, work, stream);
+      return launch_backward<float, FF>(h, ckpt, tau, T, k, gqT, gqdT, g_traj, gq0, gqd0, gtau, gmass, work, stream);
   }
 }
 

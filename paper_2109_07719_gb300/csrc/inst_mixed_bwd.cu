@@ -1,4 +1,4 @@
-// Explicit instantiation of the adjoint kernel for storage float, D-solves double,
+// Explicit instantiation of the adjoint kernel for storage float, D-solves in float pairs,
 // tape in global memory, and its launcher (the units compile in parallel).
 #include "kernels.cuh"
 
@@ -9,9 +9,9 @@ template <class T, class DT, int ST>
 BackwardKernel<T> backward_kernel() {
   return k_backward<T, DT, ST>;
 }
-template BackwardKernel<float> backward_kernel<float, double, ST_GLOBAL>();
+template BackwardKernel<float> backward_kernel<float, FF, ST_GLOBAL>();
 
-template int launch_backward<float, double>(sim_handle*, const void*, const void*, int64_t, int, const void*,
+template int launch_backward<float, FF>(sim_handle*, const void*, const void*, int64_t, int, const void*,
                                        const void*, const void*, void*, void*, void*, void*, void*, void*);
 
 }  // namespace host

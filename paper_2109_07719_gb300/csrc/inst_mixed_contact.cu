@@ -1,5 +1,5 @@
 // Explicit instantiation of the kernels of models with contact spheres for
-// storage float, D-solves double (global storage; the units compile in parallel).
+// storage float, D-solves in float pairs (global storage; the units compile in parallel).
 #include "kernels.cuh"
 
 namespace abasim {
@@ -13,8 +13,8 @@ template <class T, class DT>
 BackwardKernel<T> backward_contact_kernel() {
   return k_backward<T, DT, ST_GLOBAL, true>;
 }
-template RolloutKernel<float> rollout_contact_kernel<float, double>();
-template BackwardKernel<float> backward_contact_kernel<float, double>();
+template RolloutKernel<float> rollout_contact_kernel<float, FF>();
+template BackwardKernel<float> backward_contact_kernel<float, FF>();
 
 }  // namespace host
 }  // namespace abasim

@@ -1,5 +1,5 @@
 // Explicit instantiation of the world-aligned adjoint kernels for storage float, D-solves
-// double (tape on chip and in global memory; the units compile in parallel).
+// in float pairs (tape on chip and in global memory; the units compile in parallel).
 #include "kernels.cuh"
 
 namespace abasim {
@@ -10,7 +10,7 @@ BackwardKernel<T> wbackward_kernel(bool onchip, bool fr) {
   if (fr) return onchip ? k_wbackward<T, DT, true, true> : k_wbackward<T, DT, false, true>;
   return onchip ? k_wbackward<T, DT, true, false> : k_wbackward<T, DT, false, false>;
 }
-template BackwardKernel<float> wbackward_kernel<float, double>(bool, bool);
+template BackwardKernel<float> wbackward_kernel<float, FF>(bool, bool);
 
 }  // namespace host
 }  // namespace abasim

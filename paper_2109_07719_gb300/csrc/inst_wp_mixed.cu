@@ -1,5 +1,5 @@
 // Explicit instantiation of the pipelined world-aligned adjoint kernel for storage
-// float, D-solves double (tapes on chip and in global memory; the units compile in parallel).
+// float, D-solves in float pairs (tapes on chip and in global memory; the units compile in parallel).
 #include "kernels.cuh"
 
 namespace abasim {
@@ -10,7 +10,7 @@ BackwardKernel<T> wbackward_pipe_kernel(bool onchip, bool fr) {
   if (fr) return onchip ? k_wbackward_pipe<T, DT, true, true> : k_wbackward_pipe<T, DT, false, true>;
   return onchip ? k_wbackward_pipe<T, DT, true, false> : k_wbackward_pipe<T, DT, false, false>;
 }
-template BackwardKernel<float> wbackward_pipe_kernel<float, double>(bool, bool);
+template BackwardKernel<float> wbackward_pipe_kernel<float, FF>(bool, bool);
 
 }  // namespace host
 }  // namespace abasim

@@ -368,19 +368,27 @@ template <class T, bool STG, bool AQ> struct Inputs {
 };
 
 // ------------------------------------------------------------------ forward
-// a body's own terms: inertia about its joint in world axes and bias force, from its
-// COM inertia Ic and COM offset rw in world axes.  With vc the COM velocity the
-// momentum about the COM is (Ic w, m vc), and v x* h = [w x Ic w; w x m vc] there.
-template <class T> SD void body_terms(T m, V3<T> rw, const S3<T>& Ic, SV<T> v, SI<T>& IA, SV<T>& pA) {
+// adds a body's own terms to IA and pA: its inertia about its joint in world axes and its
+// bias force, from its COM inertia Ic and COM offset rw in world axes.  With vc the COM
+// velocity the momentum about the COM is (Ic w, m vc), and v x* h = [w x Ic w; w x m vc]
+// there.  Only the entries a body's inertia has are added (an x + 0 would stay an addition).
+template <class T> SD void add_body(T m, V3<T> rw, const S3<T>& Ic, SV<T> v, SI<T>& IA, SV<T>& pA) {
   const V3<T> g = m * rw;
   const T cc = dot(rw, g);
-  IA.A = S3<T>{Ic.xx + (cc - rw.x * g.x), Ic.yy + (cc - rw.y * g.y), Ic.zz + (cc - rw.z * g.z),
-               Ic.xy - rw.x * g.y, Ic.xz - rw.x * g.z, Ic.yz - rw.y * g.z};
-  IA.B = skew(g);
-  IA.C = S3<T>{m, m, m, T(0), T(0), T(0)};
+  IA.A += S3<T>{Ic.xx + (cc - rw.x * g.x), Ic.yy + (cc - rw.y * g.y), Ic.zz + (cc - rw.z * g.z),
+                Ic.xy - rw.x * g.y, Ic.xz - rw.x * g.z, Ic.yz - rw.y * g.z};
+  IA.B.a[1] -= g.z;
+  IA.B.a[2] += g.y;
+  IA.B.a[3] += g.z;
+  IA.B.a[5] -= g.x;
+  IA.B.a[6] -= g.y;
+  IA.B.a[7] += g.x;
+  IA.C.xx += m;
+  IA.C.yy += m;
+  IA.C.zz += m;
   const V3<T> vc = v.v + cross(v.w, rw);
   const V3<T> f = m * cross(v.w, vc);
-  pA = SV<T>{cross(v.w, mul(Ic, v.w)) + cross(rw, f), f};
+  pA += SV<T>{cross(v.w, mul(Ic, v.w)) + cross(rw, f), f};
 }
 
 // One step for the state (q, qd) and joint force tau.  ADJ: also store what the
@@ -458,9 +466,8 @@ SD void wstep_forward(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd, Co
   {
     Records<T, STG, W_R, W_AP - W_R, P_M, NPRM_W - P_M> rec(s, walk - 1, -1, walk);
     Inputs<T, STG, false> in(s, tau, qd, walk - 1, -1, walk);
-    SI<T> cI = zeroSI<T>();  // link l + 1's contribution when l is its parent
+    SI<T> cI = zeroSI<T>();  // link l + 1's contribution if l is its parent, else 0
     SV<T> cp = zeroSV<T>();
-    bool carry = false;
     int sp = 0;
     for (int l = walk - 1; l >= 0; --l) {
       rec.next();
@@ -479,9 +486,9 @@ SD void wstep_forward(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd, Co
       const SV<T> c{cross(v.w, sq), cross(v.v, sq)};
       const S3<T> Ic = rot_sym(R, fld_s3(rec.p, P_IC));
       const V3<T> rw = mul(R, fld_v3(rec.p, P_C));
-      SI<T> IA;
-      SV<T> pA;
-      body_terms(fld(rec.p, P_M), rw, Ic, v, IA, pA);
+      SI<T> IA = cI;
+      SV<T> pA = cp;
+      add_body(fld(rec.p, P_M), rw, Ic, v, IA, pA);
       // the joint offset, 0 for a root (whose contribution to a parent is dropped)
       V3<T> d = fld_v3(rec.t, W_D);
       if (ADJ) {
@@ -490,10 +497,6 @@ SD void wstep_forward(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd, Co
         else
           put_inertia(w, Ic);
         wv3(w, 0, 0, W_RW, rw);
-      }
-      if (carry) {
-        IA += cI;
-        pA += cp;
       }
       if (meta_treechild(m)) {
         --sp;
@@ -518,17 +521,19 @@ SD void wstep_forward(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd, Co
       const SV<T> pa = pA + mul(Ia, c) + (T)((DT)u * Di) * U;
       const SI<T> Y = shift(Ia, d);
       const SV<T> pn = shift_force(pa, d);
-      carry = par == l - 1 && par >= 0;
-      if (carry) {
-        cI = Y;
-        cp = pn;
-      } else if (par >= 0 && meta_lastsib(m)) {
-        wsi(s.stk, WSW, sp, 0, Y);
-        wsv(s.stk, WSW, sp, 21, pn);
-        ++sp;
-      } else if (par >= 0) {
-        wsi(s.stk, WSW, sp - 1, 0, wsi(s.stk, WSW, sp - 1, 0) + Y);
-        wsv(s.stk, WSW, sp - 1, 21, wsv(s.stk, WSW, sp - 1, 21) + pn);
+      cI = Y;
+      cp = pn;
+      if (par != l - 1 || par < 0) {
+        cI = zeroSI<T>();
+        cp = zeroSV<T>();
+        if (par >= 0 && meta_lastsib(m)) {
+          wsi(s.stk, WSW, sp, 0, Y);
+          wsv(s.stk, WSW, sp, 21, pn);
+          ++sp;
+        } else if (par >= 0) {
+          wsi(s.stk, WSW, sp - 1, 0, wsi(s.stk, WSW, sp - 1, 0) + Y);
+          wsv(s.stk, WSW, sp - 1, 21, wsv(s.stk, WSW, sp - 1, 21) + pn);
+        }
       }
     }
   }
