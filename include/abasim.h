@@ -140,8 +140,8 @@ typedef struct sim_handle sim_handle;
 
 /* Validate and pack a model (Sec. 2: state x = [q, qd], control u = tau), upload
  * its constants to the current device and allocate the per-step tape.  Each
- * system's links are stored in depth-first preorder (children in the model's
- * order); coordinates, masses and every result keep the model's numbering.
+ * system's links are stored in depth-first preorder (small subtrees first);
+ * coordinates, masses and every result keep the model's numbering.
  * Returns SIM_EINVAL with a message for an invalid tree, joint, axis, rotation or
  * inertia; SIM_ENOMEM / SIM_ECUDA for device failures.  *out is NULL on error. */
 int sim_create(const sim_model_desc* desc, sim_handle** out);
@@ -278,11 +278,11 @@ int sim_set_launch(sim_handle* h, int32_t threads, int32_t schedule);
  * the articulated inertias translates them from child to parent instead of
  * rotating and translating them (each body's inertia is rotated into world axes
  * once per step, off that serial chain).  Tape and adjoint record in shared
- * memory when a block's tiles fit, else in the handle's global scratch (whose
- * lines each pass prefetches sim_set_prefetch links ahead).  Links are stored in
- * depth-first preorder; the values a branching link hands to or collects from
- * its later children live on a per-system stack (in shared memory with an
- * on-chip tape, else in a handle buffer) as deep as the nesting of branchings.
+ * memory when a block's tiles fit, else in the handle's global scratch, staged
+ * through shared memory as each pass walks the links.  Links are stored in
+ * depth-first preorder, small subtrees first; the values a branching link hands to
+ * or collects from its later children live on a per-system stack (in shared memory
+ * where it fits, else in a handle buffer) at most log2(links) entries deep.
  * AUTO picks these kernels for such
  * models, except where the pipelined kernels apply (serial chains short enough
  * for their on-chip tapes) and where a system's state and input streams exceed a
@@ -308,12 +308,12 @@ int sim_set_tape_space(sim_handle* h, int32_t space);
  * a free joint (AUTO only).  Either pointer may be NULL.  No device work. */
 int sim_last_storage(const sim_handle* h, int32_t* rollout_mode, int32_t* backward_mode);
 
-/* Prefetch distance of the world-aligned kernels when their tape is in global
- * memory: while link l computes, each pass asks for the cache lines of the link
- * links_ahead further along its walk (and the next step's input lines), so a
- * warp's tape reads find L1 instead of waiting on L2 / HBM once per link.
- * 0 switches prefetching off; default 2; at most 16.  A tuning control (the
- * autotuner may set it); results do not depend on it. */
+/* Look-ahead of the world-aligned kernels when their tape is in global memory: each
+ * pass copies the records of the next links of its walk (and asks for the next
+ * step's input lines) into a shared-memory ring ahead of their use.  0 switches the
+ * look-ahead off (each link waits for its record); any other value (default 2; at
+ * most 16) keeps it at what the ring holds.  A tuning control; results do not
+ * depend on it. */
 int sim_set_prefetch(sim_handle* h, int32_t links_ahead);
 
 /* How sim_backward_rollout rebuilds the states inside a checkpoint segment when

@@ -224,7 +224,7 @@ class Simulator:
         return self.STORAGE[f.value], self.STORAGE[b.value]
 
     def set_prefetch(self, links_ahead: int = 2):
-        """How many links ahead the world-aligned global-tape passes prefetch (0: off)."""
+        """Look-ahead of the world-aligned global-tape passes (0: off; any other value: on)."""
         self._check(lib.sim_set_prefetch(self._h, int(links_ahead)), "sim_set_prefetch")
 
     def set_replay(self, mode: str = "segment"):

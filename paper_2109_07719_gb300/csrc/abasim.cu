@@ -313,7 +313,7 @@ int sim_create(const sim_model_desc* d, sim_handle** out) {
     nl[sl] = nl_sys[b];
     const int n = nl[sl], o = d->sys_link_offset[b];
     // coordinates keep the model's numbering; the links are stored in depth-first
-    // preorder (perm: stored position -> model link), children in model order
+    // preorder (perm: stored position -> model link), small subtrees first
     std::vector<int> qoff(n), voff(n);
     int qo = 0, vo = 0;
     for (int l = 0; l < n; ++l) {
@@ -322,8 +322,15 @@ int sim_create(const sim_model_desc* d, sim_handle** out) {
       qo += d->joint_type[o + l] == SIM_FREE ? 7 : 1;
       vo += d->joint_type[o + l] == SIM_FREE ? 6 : 1;
     }
-    const TreeOrder to = tree_order(d->parent + o, n);
-    const std::vector<int>& perm = to.perm;
+    const std::vector<int> light = light_first(d->parent + o, n);
+    std::vector<int> at(n), par(n), perm(n);
+    for (int l = 0; l < n; ++l) at[light[l]] = l;
+    for (int l = 0; l < n; ++l) {
+      const int p = d->parent[o + light[l]];
+      par[l] = p >= 0 ? at[p] : -1;
+    }
+    const TreeOrder to = tree_order(par.data(), n);
+    for (int l = 0; l < n; ++l) perm[l] = light[to.perm[l]];
     h->wdepth = std::max(h->wdepth, to.depth);
     for (int l = 0; l < n; ++l) {
       const int i = o + perm[l];

@@ -39,9 +39,10 @@ template <class T> struct DevModel {
   ContactParams<T> cp;
   double dt64;   // the time step in FP64
   double* x64;   // FP64 running state [nq_max + nv_max][B] of the rollout (null: off; FP32 + FP64 D only)
-  int pf;        // world-aligned kernels with a global tape: links a record is staged ahead (0: none)
+  int slots;     // world-aligned kernels with a global tape: slots of a warp's ring, 3 or 1 (no look-ahead)
   T* stk;        // world-aligned kernels: two stacks of parent values [2][tiles][wdepth][WSW][lane] (null: none)
   int wdepth;    // entries per stack
+  int sd;        // scalars of a system's stack in shared memory beside a global tape (0: in stk)
 };
 
 template <class T> DevModel<T> dev_model(const sim_handle* h) {
@@ -50,7 +51,7 @@ template <class T> DevModel<T> dev_model(const sim_handle* h) {
                      (T)h->g[0], (T)h->g[1], (T)h->g[2], h->integrator, 0, 0,
                      h->replay == SIM_REPLAY_QUADRATIC, (T*)h->ctape, (T*)h->csys,
                      ContactParams<T>{(T)h->friction, (T)h->erp, h->pgs_iterations}, h->dt,
-                     h->state64 ? (double*)h->x64 : nullptr, std::min(h->prefetch, RING_AHEAD), (T*)h->wstk, h->wdepth};
+                     h->state64 ? (double*)h->x64 : nullptr, h->prefetch > 0 ? 3 : 1, (T*)h->wstk, h->wdepth, 0};
 }
 
 extern __shared__ __align__(16) unsigned char g_smem[];
@@ -916,6 +917,17 @@ inline int l1_carveout(const sim_handle* h, int slots_per_block, size_t bytes) {
   return (int)std::min(100LL, std::max(1LL, (100 * want + sm_smem - 1) / sm_smem));
 }
 
+// Whether a global-tape block of `bytes` with its warps' stacks in shared memory fits, with
+// as many blocks an SM as the batch has, up to two: blocks are sorted by length, so those
+// that wait for room run beside the end of the long ones (adjoint of 16384 trees of 2-64
+// links 257 us a step with the stacks in global memory and three blocks an SM, 168 with them
+// here and two).
+inline bool stacks_fit(const sim_handle* h, int slots_per_block, size_t bytes, int limit) {
+  const long long units = (h->B + slots_per_block - 1) / slots_per_block, sms = std::max(1, h->sms);
+  const long long blocks = std::min(2LL, (units + sms - 1) / sms);
+  return blocks * ((long long)bytes + 1024) <= (long long)limit + 1024;
+}
+
 // Scalars per tile of a world-aligned kernel's working state (w_smem_per_tile's, without
 // the rings).
 inline long long w_state_per_tile(const sim_handle* h, bool bwd) {
@@ -925,21 +937,26 @@ inline long long w_state_per_tile(const sim_handle* h, bool bwd) {
 // Storage of a world-aligned one-warp launch: the tape on chip when a block's tiles fit the
 // per-block opt-in limit and that adds no wave of blocks over the global-tape kernel.  The
 // latter's rings take shared memory too: where a block of h->block threads with them would
-// not fit, it runs fewer tiles per block (*threads), then stages fewer links ahead.
+// not fit, it runs fewer tiles per block (*threads), then stages without looking ahead.
 template <class T, class K>
-int choose_w(sim_handle* h, K k_on, K k_off, bool bwd, bool* onchip, int* threads, int* ahead, size_t* bytes) {
+int choose_w(sim_handle* h, K k_on, K k_off, bool bwd, bool* onchip, int* threads, int* slots, int* sd,
+             size_t* bytes) {
   int limit = 0;
   cudaError_t e = cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
   if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory limit query");
   const int nx = h->nq_max + h->nv_max;
   const bool fr = !h->all_revolute;
-  auto need = [&](bool on, int tiles, int ah) {
-    return (size_t)tiles * w_smem_per_tile(h->maxL, nx, h->nv_max, bwd, on, h->wdepth * WSW, fr, ah) * LANES * sizeof(T);
+  auto need = [&](bool on, int tiles) {
+    return (size_t)tiles * w_smem_per_tile(h->maxL, nx, h->nv_max, bwd, on, on ? h->wdepth * WSW : *sd, fr, *slots) *
+           LANES * sizeof(T);
   };
   int tiles = h->block / LANES;
-  while (tiles > 1 && need(false, tiles, *ahead) > (size_t)limit) --tiles;
-  while (*ahead > 0 && need(false, tiles, *ahead) > (size_t)limit) --*ahead;
-  const size_t need_on = need(true, h->block / LANES, 0), need_off = need(false, tiles, *ahead);
+  *sd = 0;
+  while (tiles > 1 && need(false, tiles) > (size_t)limit) --tiles;
+  if (need(false, tiles) > (size_t)limit) *slots = 1;
+  *sd = h->wdepth * WSW;
+  if (!stacks_fit(h, tiles * LANES, need(false, tiles), limit)) *sd = 0;
+  const size_t need_on = need(true, h->block / LANES), need_off = need(false, tiles);
   if (need_off > (size_t)limit) return fail(h, SIM_EUNSUPPORTED, "the working state does not fit in shared memory");
   e = cudaFuncSetAttribute((const void*)k_off, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need_off);
   if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory opt-in");
@@ -1003,7 +1020,7 @@ int launch_wrollout(sim_handle* h, const void* q0, const void* qd0, const void* 
   bool onchip = false;
   size_t shm = 0;
   int threads = 0;
-  int rc = choose_w<T>(h, k_on, k_off, false, &onchip, &threads, &m.pf, &shm);
+  int rc = choose_w<T>(h, k_on, k_off, false, &onchip, &threads, &m.slots, &m.sd, &shm);
   if (rc != SIM_OK) return rc;
   const RolloutKernel<T> kern = onchip ? k_on : k_off;
   h->last_storage = (h->all_revolute ? 4 : 8) + (onchip ? 0 : 1);
@@ -1029,21 +1046,24 @@ int launch_wbackward_pipe(sim_handle* h, const void* ckpt, const void* tau, int6
   const int nx = h->nq_max + h->nv_max;
   const bool fr = !h->all_revolute;
   const int tiles = (h->B + LANES - 1) / LANES, sms = std::max(1, h->sms);
-  auto need = [&](bool on, int np, int ah) {
-    return (size_t)wpipe_smem_per_tile(h->maxL, nx, h->nv_max, on, h->wdepth * WSW, fr, np, ah) * LANES * sizeof(T);
+  auto need = [&](bool on, int np) {
+    return (size_t)wpipe_smem_per_tile(h->maxL, nx, h->nv_max, on, on ? h->wdepth * WSW : m.sd, fr, np, m.slots) * LANES *
+           sizeof(T);
   };
-  const bool onchip = need(true, 1, 0) <= (size_t)limit && (!fr || tiles <= sms);
-  // Producers: three while every tile has an SM to itself (4096 7-link chains, on chip: 6.96
-  // us a step with one, 5.60, 4.94 with three, 5.5 with four or five; 1024 humanoids, global
-  // tapes: 36.5, 31.6, 29.6).  With more tiles than that the SMs are shared: on chip the
-  // two producers that take no more tapes than one, so that two blocks fit an SM (16384
-  // chains 13.3 us, 19.3 with three); with global tapes one (8192 quadrupeds FP32 26.6 us,
-  // 31.9 with three; 16384 trees the same with any), but three where the FP64 pipe is what
-  // the producers share out (quadrupeds with FP64 D-solves 92.1 -> 63.9 us).
-  int np = tiles <= sms || (!onchip && sizeof(DT) == 8) ? WPIPE_TAPES : onchip ? 2 : 1;
-  while (np > 1 && need(onchip, np, onchip ? 0 : std::min(1, m.pf)) > (size_t)limit) --np;
-  while (!onchip && m.pf > 0 && need(false, np, m.pf) > (size_t)limit) --m.pf;
-  const size_t shm = need(onchip, np, m.pf);
+  const bool onchip = need(true, 1) <= (size_t)limit && (!fr || tiles <= sms);
+  // Producers: three while every tile has an SM to itself (4096 7-link chains, on chip: 6.3
+  // us a step with one, 5.4, 5.0 with three; 1024 humanoids, global tapes: 32.8, 30.1, 29.9;
+  // 1000 FP64 trees of 2-20 links 379, 325, 277).  With more tiles than that the SMs are
+  // shared: on chip the two producers that take no more tapes than one, so that two blocks
+  // fit an SM (16384 chains 12.5 us, 19.4 with three); with global tapes one, which also
+  // leaves room for the stacks (8192 quadrupeds FP32 24.1 us, 33.6 with three; 16384 trees
+  // 168, 259).
+  int np = tiles <= sms ? WPIPE_TAPES : onchip ? 2 : 1;
+  while (np > 1 && need(onchip, np) > (size_t)limit) --np;
+  if (need(onchip, np) > (size_t)limit) m.slots = 1;
+  m.sd = h->wdepth * WSW;
+  if (!stacks_fit(h, LANES, need(onchip, np), limit)) m.sd = 0;
+  const size_t shm = need(onchip, np);
   if (shm > (size_t)limit) return fail(h, SIM_EUNSUPPORTED, "the working state does not fit in shared memory");
   const int threads = (np + 1) * LANES;
   const BackwardKernel<T> kern = wbackward_pipe_kernel<T, DT>(onchip, fr);
@@ -1084,7 +1104,7 @@ int launch_wbackward(sim_handle* h, const void* ckpt, const void* tau, int64_t T
   bool onchip = false;
   size_t shm = 0;
   int threads = 0;
-  int rc = choose_w<T>(h, k_on, k_off, true, &onchip, &threads, &m.pf, &shm);
+  int rc = choose_w<T>(h, k_on, k_off, true, &onchip, &threads, &m.slots, &m.sd, &shm);
   if (rc != SIM_OK) return rc;
   const BackwardKernel<T> kern = onchip ? k_on : k_off;
   h->last_storage_bwd = (h->all_revolute ? 4 : 8) + (onchip ? 0 : 1);

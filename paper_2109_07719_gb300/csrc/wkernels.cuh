@@ -24,12 +24,12 @@ __host__ __device__ __forceinline__ long long w_tape_words(int maxL, bool fr) {
 // the adjoint, the adjoint record), the model constants and meta words, the stack
 // of parent values (sd scalars per system) and a double buffer for the per-step
 // inputs (tau, plus x^t for the adjoint) fetched one step ahead.  Without ONCHIP
-// the stack and the records are in the handle's global scratch, and the warp's ring
-// stages the records of the `ahead` next links (wstep.cuh).
+// the records are in the handle's global scratch and a ring of `slots` slots stages them
+// (wstep.cuh); the stack is here too if the launch has room (sd > 0).
 __host__ __device__ __forceinline__ long long w_smem_per_tile(int maxL, int nx, int nv, bool bwd, bool onchip,
-                                                              int sd, bool fr, int ahead) {
+                                                              int sd, bool fr, int slots) {
   const long long state = nx + (bwd ? maxL : 0);
-  if (!onchip) return state + (ahead + 1LL) * (bwd ? RING_ADJ : RING_FWD);
+  if (!onchip) return state + sd + (long long)slots * (bwd ? RING_ADJ : RING_FWD);
   return w_tape_words(maxL, fr) + (long long)maxL * ((bwd ? NWA : 0) + NPRM_W + 1) + sd + state +
          2LL * (nv + (bwd ? nx : 0));
 }
@@ -59,9 +59,9 @@ template <class T, bool BWD, bool ONCHIP, bool FR>
 __device__ __forceinline__ WTile<T> w_tile(const DevModel<T>& m, int lane) {
   const int tb = threadIdx.x / LANES;
   const long long L = m.maxL;
-  const int nx = m.nq_max + m.nv_max, sd = m.wdepth * WSW;
+  const int nx = m.nq_max + m.nv_max, sd = ONCHIP ? m.wdepth * WSW : m.sd;
   T* base = reinterpret_cast<T*>(g_smem) +
-            (long long)tb * w_smem_per_tile(m.maxL, nx, m.nv_max, BWD, ONCHIP, sd, FR, m.pf) * LANES + lane;
+            (long long)tb * w_smem_per_tile(m.maxL, nx, m.nv_max, BWD, ONCHIP, sd, FR, m.slots) * LANES + lane;
   WTile<T> t{};
   if (ONCHIP) {
     t.tape = base;
@@ -72,12 +72,12 @@ __device__ __forceinline__ WTile<T> w_tile(const DevModel<T>& m, int lane) {
     base += L * NPRM_W * LANES;
     t.meta = reinterpret_cast<int*>(base);
     base += L * LANES;
-    t.stk = base;
-    base += (long long)sd * LANES;
   } else {
     t.ring = base - lane;
-    base += (m.pf + 1LL) * (BWD ? RING_ADJ : RING_FWD) * LANES;
+    base += (long long)m.slots * (BWD ? RING_ADJ : RING_FWD) * LANES;
   }
+  t.stk = base;
+  base += (long long)sd * LANES;
   t.state = base;
   base += (long long)nx * LANES;
   t.gm = base;
@@ -106,8 +106,8 @@ __device__ __forceinline__ WSys<T, !ONCHIP> wsys_of(const DevModel<T>& m, int sl
   } else {
     T* tape = m.tape + tile * w_tape_words(m.maxL, FR) * LANES + lane;
     return WSys<T, true>{gprm, gmeta, tape, m.adj + tile * L * NWA * LANES + lane, nl, 1, NPRM,
-                         w_stack(m, 0, tile, lane), tape + L * NWT * LANES,
-                         __reduce_max_sync(0xffffffffu, nl), t.ring, m.pf, (int)lane};
+                         m.sd ? t.stk : w_stack(m, 0, tile, lane), tape + L * NWT * LANES,
+                         __reduce_max_sync(0xffffffffu, nl), t.ring, m.slots > 1, (int)lane};
   }
 }
 
@@ -150,7 +150,7 @@ __device__ __forceinline__ void wrollout_one(const DevModel<T>& m, int slot, boo
       cp_commit();
       cp_wait_all_but_newest();
       tau_t = Col<const T>{sbuf + (t & 1) * nvm * LANES, LANES};
-    } else if (t + 1 < Tn && m.pf > 0) {
+    } else if (t + 1 < Tn && m.slots > 1) {
       for (int d = 0; d < nv; ++d) pf_line(tau + ((t + 1) * nvm + d) * B + b);
     }
     wstep_forward<T, DT, false, true, FR>(s, Col<const T>{q.p, LANES}, Col<const T>{qd.p, LANES}, tau_t, g, m.dt,
@@ -231,7 +231,7 @@ __device__ __forceinline__ void wbackward_one(const DevModel<T>& m, int slot, bo
     cp_wait_all();
   } else if (k == 1) {  // inputs straight from global memory, the previous step's lines prefetched
     for (long long t = Tn - 1; t >= 0; --t) {
-      if (t > 0 && m.pf > 0) {
+      if (t > 0 && m.slots > 1) {
         const T* xn = ckpt + (t - 1) * NX * B + b;
         for (int d = 0; d < nq; ++d) pf_line(xn + d * B);
         for (int d = 0; d < nv; ++d) pf_line(xn + (nqm + d) * B);

@@ -29,11 +29,12 @@ __host__ __device__ __forceinline__ int wpipe_tapes(int np) { return np > 1 ? np
 // Scalars per tile: the state adjoint and per-link mass-gradient sums; with
 // ONCHIP also the tapes, the adjoint record, model constants and meta words, the
 // warps' stacks of parent values (sd scalars per system each) and each producer's
-// double-buffered inputs (x^t, tau^t); without ONCHIP the warps' rings.
+// double-buffered inputs (x^t, tau^t); without ONCHIP the warps' rings of `slots`
+// slots, and their stacks if the launch has room (sd > 0).
 __host__ __device__ __forceinline__ long long wpipe_smem_per_tile(int maxL, int nx, int nv, bool onchip, int sd,
-                                                                  bool fr, int np, int ahead) {
+                                                                  bool fr, int np, int slots) {
   const long long state = nx + maxL;
-  if (!onchip) return state + (ahead + 1LL) * (RING_ADJ + np * RING_FWD);
+  if (!onchip) return state + (np + 1LL) * sd + (long long)slots * (RING_ADJ + np * RING_FWD);
   return wpipe_tapes(np) * w_tape_words(maxL, fr) + (np + 1LL) * sd + (long long)maxL * (NWA + NPRM_W + 1) + state +
          2LL * np * (nx + nv);
 }
@@ -61,8 +62,8 @@ k_wbackward_pipe(DevModel<T> m, const T* __restrict__ ckpt, const T* __restrict_
   constexpr int MS = (int)(sizeof(T) / sizeof(int));
   T* base = reinterpret_cast<T*>(g_smem);
   T *s_tape = nullptr, *s_adj = nullptr, *s_prm = nullptr, *s_meta = nullptr, *s_in = nullptr;
-  T *s_stk = nullptr, *s_ring = nullptr;
-  const long long sdw = (long long)m.wdepth * WSW;  // stack scalars per system
+  T* s_ring = nullptr;
+  const long long sdw = ONCHIP ? (long long)m.wdepth * WSW : m.sd;  // stack scalars per system on chip
   if (ONCHIP) {
     s_tape = base;  // [NT][tape words][LANES]
     base += NT * TW * LANES;
@@ -72,12 +73,12 @@ k_wbackward_pipe(DevModel<T> m, const T* __restrict__ ckpt, const T* __restrict_
     base += L * NPRM_W * LANES;
     s_meta = base;
     base += L * LANES;
-    s_stk = base;  // [NP + 1][sdw][LANES]: one per warp
-    base += (NP + 1) * sdw * LANES;
   } else {
-    s_ring = base + (m.pf + 1LL) * LANES * (consumer ? 0 : RING_ADJ + (warp - 1) * RING_FWD);
-    base += (m.pf + 1LL) * LANES * (RING_ADJ + NP * RING_FWD);
+    s_ring = base + (long long)m.slots * LANES * (consumer ? 0 : RING_ADJ + (warp - 1) * RING_FWD);
+    base += (long long)m.slots * LANES * (RING_ADJ + NP * RING_FWD);
   }
+  T* s_stk = base + warp * sdw * LANES + lane;  // [NP + 1][sdw][LANES]: one per warp
+  base += (NP + 1) * sdw * LANES;
   T* s_state = base;
   T* s_gm = s_state + (long long)NX * LANES;
   const int W = NX + nvm;
@@ -103,12 +104,12 @@ k_wbackward_pipe(DevModel<T> m, const T* __restrict__ ckpt, const T* __restrict_
     auto sys_of_buf = [&](int buf) -> WSys<T, !ONCHIP> {
       if constexpr (ONCHIP) {
         T* tape = s_tape + buf * TW * LANES + lane;
-        return WSys<T>{s_prm + lane, meta_l, tape, s_adj + lane, nl, MS, NPRM_W, s_stk + warp * sdw * LANES + lane,
-                       tape + L * NWT * LANES};
+        return WSys<T>{s_prm + lane, meta_l, tape, s_adj + lane, nl, MS, NPRM_W, s_stk, tape + L * NWT * LANES};
       } else {
         T* tape = tapes + (buf * units + unit) * TW * LANES + lane;
         return WSys<T, true>{gprm, gmeta, tape, m.adj + (long long)unit * L * NWA * LANES + lane, nl, 1, NPRM,
-                             w_stack(m, warp, unit, lane), tape + L * NWT * LANES, links, s_ring, m.pf, lane};
+                             m.sd ? s_stk : w_stack(m, warp, unit, lane), tape + L * NWT * LANES, links, s_ring,
+                             m.slots > 1, lane};
       }
     };
     // a producer's inputs of step t: x^t and tau^t (the system's own coordinates)
@@ -131,7 +132,7 @@ k_wbackward_pipe(DevModel<T> m, const T* __restrict__ ckpt, const T* __restrict_
           if (act && t >= NP) fetch(t - NP, in ^ 1);
           cp_commit();
           cp_wait_all_but_newest();
-        } else if (act && t >= NP && m.pf > 0) {
+        } else if (act && t >= NP && m.slots > 1) {
           const T* xn = ckpt + (t - NP) * NX * B + b;
           for (int d = 0; d < nq; ++d) pf_line(xn + d * B);
           for (int d = 0; d < nv; ++d) pf_line(xn + (nqm + d) * B);

@@ -67,12 +67,14 @@
 namespace abasim {
 
 // Per-link tape of the world-aligned step, [link][field][lane]: U; 1/D (hi/lo pair); u,
-// then the adjoint's wb; orientation R, whose first two columns give way, when the
-// adjoint will read the tape, to the rotated COM inertia R I_com R^T (the third column
-// is the joint axis s); velocity v; the joint offset d; and for the adjoint a', qdd, the
-// joint rate qd and the COM offset R com.  Ordered so that what a pass reads is one range.
+// then the adjoint's wb; the joint offset d; the orientation R by columns, the joint axis
+// s = R e_z first, the other two giving way, when the adjoint will read the tape, to the
+// rotated COM inertia R I_com R^T; velocity v; and for the adjoint a', qdd, the joint rate
+// qd and the COM offset R com.  Ordered so that what a pass reads is one range (two for
+// the acceleration pass).
 enum : int {
-  W_U = 0, W_DI = 6, W_u = 8, W_R = 9, W_V = 18, W_D = 24, W_AP = 27, W_QDD = 33, W_QD = 34, W_RW = 35, NWT = 38
+  W_U = 0, W_DI = 6, W_u = 8, W_D = 9, W_S = 12, W_XY = 15, W_V = 21, W_AP = 27, W_QDD = 33, W_QD = 34, W_RW = 35,
+  NWT = 38
 };
 // Record of a free root (FR kernels; link 0 only), [field][lane]: its articulated
 // inertia, qdd, the quaternion and velocity the step started from and the rotated COM
@@ -101,8 +103,8 @@ template <class T, bool STG = false> struct WSys {
   T* stk = nullptr;  // [entry][WSW][LANES]: the stack of parent values (see the tree data flow above)
   T* root = nullptr; // [NWF][LANES]: the free root's record (FR only)
   int links = -1;    // STG: links the warp walks (its longest system's; every lane walks them together)
-  T* ring = nullptr; // STG: this warp's ring in shared memory, [ahead + 1][rows][LANES], at lane 0
-  int ahead = 2;     // STG: links a record is fetched ahead of its use, 0 .. RING_AHEAD
+  T* ring = nullptr; // STG: this warp's ring in shared memory, [rows][LANES], at lane 0
+  bool full = true;  // STG: it has three slots of the longest pass, not one
   int lane = 0;
   SD T P(int l, int f) const { return prm[(l * pstride + f) * LANES]; }
   SD int M(int l) const { return meta[l * LANES * mstride]; }
@@ -119,8 +121,11 @@ template <class T, bool STG = false> struct WSys {
 // written since); with the ring a 64-link chain tile's rollout step went from 123 to 86 us,
 // 1500 trees of 2-40 links with segment replay from 17.3 to 12.6 ms over 48 steps.  It
 // takes 3 x rows x 128 bytes a warp and a quarter of the instructions (four rows each).
-constexpr int RING_AHEAD = 2;
-// rows a warp's ring needs: the forward passes', the adjoint passes'
+// A pass that reads fewer rows has more slots in the same ring, so a short pass looks as
+// far ahead in time as a long one.  The slot filled while link i computes was read at link
+// i - 2, so one warp barrier a link orders both the reads and the writes.
+// rows of a warp's ring: three slots of its longest pass (the forward passes', the adjoint
+// passes'); a ring of one slot (staging without looking ahead) is a third of it
 constexpr int RING_FWD = 29, RING_ADJ = 36;
 // producers of the pipelined adjoint at most, each with a tape; in global memory, one stack
 // of parent values for each of its warps is beside them
@@ -132,78 +137,96 @@ __device__ __forceinline__ void stage_cp16(void* dst, const void* src) {
                : "memory");
 }
 __device__ __forceinline__ void stage_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void stage_wait(int newer) {  // all but the `newer` newest groups are in place
-  if (newer >= 2)
-    asm volatile("cp.async.wait_group 2;\n" ::: "memory");
-  else if (newer == 1)
-    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-  else
-    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+template <int NEWER> __device__ __forceinline__ void stage_wait() {  // all but the NEWER newest groups are in place
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(NEWER) : "memory");
 }
 #endif
 
-// The records of one pass over `n` links from `first` in steps of `dir`: tape fields
-// [TF, TF + TN), model constants [PF, PF + PN), adjoint fields [AF, AF + AN).  next() makes
-// the following link's records readable through t, p and a (indexed by field; at this
-// lane).  All lanes of the warp call it together when staging.
-template <class T, bool STG, int TF, int TN, int PF, int PN, int AF = 0, int AN = 0> struct Records {
-  static constexpr int ROWS = TN + PN + AN;
-  static_assert(ROWS <= RING_ADJ, "ring rows");
+// The records of one pass over `n` links from link 0 up (DIR 1) or from link n - 1 down
+// (DIR -1): tape fields [TF, TF + TN) and [SF, SF + SN), model constants [PF, PF + PN),
+// adjoint fields [AF, AF + AN).  next() makes the following link's records readable through
+// t (fields of the first range), t2 (the second), p and a, indexed by field, at this lane.
+// All lanes of the warp call it together when staging.
+template <class T, bool STG, int DIR, int RING, int TF, int TN, int PF, int PN, int AF = 0, int AN = 0, int SF = 0,
+          int SN = 0>
+struct Records {
+  static constexpr int ROWS = TN + SN + PN + AN, SLOTS = 3 * RING / ROWS, AHEAD = SLOTS - 2;
+  static_assert(ROWS <= RING, "ring rows");
   const WSys<T, STG>& s;
-  int first, dir, n, i = 0, slot = 0, fill = 0;
-  const T *t = nullptr, *p = nullptr, *a = nullptr;
-  SD Records(const WSys<T, STG>& sys, int first_, int dir_, int n_) : s(sys), first(first_), dir(dir_), n(n_) {
+  int left;              // links still to fetch (staging)
+  const T *st, *sp, *sa;  // the next record to fetch, or the current one
+  T *fill, *read;        // ring slots
+  const T *t, *t2, *p, *a;
+  SD Records(const WSys<T, STG>& sys, int n) : s(sys), left(n) {
+    const int first = DIR > 0 ? 0 : n - 1;
+    st = s.tape + first * NWT * LANES;
+    sp = s.prm + first * s.pstride * LANES;
+    sa = AN ? s.adj + first * NWA * LANES : nullptr;
     if constexpr (STG) {
 #ifdef __CUDA_ARCH__
+      constexpr int PER = 16 / sizeof(T);
+      st += TF * LANES - s.lane + s.lane * PER;  // each lane copies 16 bytes of every LANES x 16
+      sp += PF * LANES - s.lane + s.lane * PER;
+      if (AN) sa += AF * LANES - s.lane + s.lane * PER;
+      fill = read = s.ring;
       __syncwarp();  // the previous pass has read its last slot and written its records
-      for (int j = 0; j < s.ahead; ++j) fetch(j);
+      if (s.full)
+        for (int j = 0; j < AHEAD; ++j) fetch();
 #endif
+    } else {
+      st -= DIR * NWT * LANES;
+      sp -= DIR * s.pstride * LANES;
+      if (AN) sa -= DIR * NWA * LANES;
     }
   }
-  SD void fetch(int j) {
+  SD void fetch() {
 #ifdef __CUDA_ARCH__
-    if (j < n) {
-      const int l = first + dir * j;
-      constexpr int PER = 16 / sizeof(T), CH = LANES / PER;  // words per copy, copies per row
-      T* dst = s.ring + (long long)fill * ROWS * LANES;
-      copy<TN * CH>(dst, s.tape - s.lane + (l * NWT + TF) * LANES);
-      copy<PN * CH>(dst + TN * LANES, s.prm - s.lane + (l * s.pstride + PF) * LANES);
-      if (AN) copy<AN * CH>(dst + (TN + PN) * LANES, s.adj - s.lane + (l * NWA + AF) * LANES);
+    constexpr int CH = LANES * (int)sizeof(T) / 16;  // copies per row
+    if (left > 0) {
+      copy<TN * CH>(fill, st);
+      copy<SN * CH>(fill + TN * LANES, st + (SF - TF) * LANES);
+      copy<PN * CH>(fill + (TN + SN) * LANES, sp);
+      if (AN) copy<AN * CH>(fill + (TN + SN + PN) * LANES, sa);
+      st += DIR * NWT * LANES;
+      sp += DIR * s.pstride * LANES;
+      if (AN) sa += DIR * NWA * LANES;
+      --left;
     }
-    fill = fill == s.ahead ? 0 : fill + 1;
     stage_commit();
+    if (s.full) fill = fill == s.ring + (SLOTS - 1) * ROWS * LANES ? s.ring : fill + ROWS * LANES;
 #endif
   }
   template <int COPIES> SD void copy(T* dst, const T* src) {
 #ifdef __CUDA_ARCH__
     constexpr int PER = 16 / sizeof(T);
+    dst += s.lane * PER;
 #pragma unroll
-    for (int c0 = 0; c0 < COPIES; c0 += LANES) {
-      const int c = c0 + s.lane;
-      if (c0 + LANES <= COPIES || c < COPIES) stage_cp16(dst + c * PER, src + c * PER);
-    }
+    for (int c = 0; c < COPIES; c += LANES)
+      if (c + LANES <= COPIES || c + s.lane < COPIES) stage_cp16(dst + c * PER, src + c * PER);
 #endif
   }
   SD void next() {
     if constexpr (STG) {
 #ifdef __CUDA_ARCH__
-      __syncwarp();  // every lane is done with the slot that is filled next
-      fetch(i + s.ahead);
-      stage_wait(s.ahead);
+      if (!s.full) __syncwarp();  // every lane is done with the only slot
+      fetch();
+      if (s.full)
+        stage_wait<AHEAD>();
+      else
+        stage_wait<0>();
       __syncwarp();
-      const T* r = s.ring + (long long)slot * ROWS * LANES + s.lane;
+      const T* r = read + s.lane;
       t = r - TF * LANES;
-      p = r + (TN - PF) * LANES;
-      a = r + (TN + PN - AF) * LANES;
-      slot = slot == s.ahead ? 0 : slot + 1;
+      t2 = r + (TN - SF) * LANES;
+      p = r + (TN + SN - PF) * LANES;
+      a = r + (TN + SN + PN - AF) * LANES;
+      if (s.full) read = read == s.ring + (SLOTS - 1) * ROWS * LANES ? s.ring : read + ROWS * LANES;
 #endif
     } else {
-      const int l = first + dir * i;
-      t = s.tape + l * NWT * LANES;
-      p = s.prm + l * s.pstride * LANES;
-      a = s.adj + l * NWA * LANES;
+      t = t2 = st += DIR * NWT * LANES;
+      p = sp += DIR * s.pstride * LANES;
+      if (AN) a = sa += DIR * NWA * LANES;
     }
-    ++i;
   }
 };
 
@@ -261,15 +284,17 @@ template <class T> SD M3<T> fld_m3(const T* r, int f) {
   for (int i = 0; i < 9; ++i) m.a[i] = fld(r, f + i);
   return m;
 }
-// the joint axis: the third column of the record's R
-template <class T> SD V3<T> fld_axis(const T* r) { return {fld(r, W_R + 2), fld(r, W_R + 5), fld(r, W_R + 8)}; }
-// the rotated COM inertia in the first two columns of the record's R
-template <class T> SD S3<T> fld_inertia(const T* r) {
-  return {fld(r, W_R), fld(r, W_R + 1), fld(r, W_R + 3), fld(r, W_R + 4), fld(r, W_R + 6), fld(r, W_R + 7)};
+// the orientation, stored by columns with the joint axis (the third) first
+template <class T> SD M3<T> fld_rot(const T* r) {
+  const V3<T> s = fld_v3(r, W_S), x = fld_v3(r, W_XY), y = fld_v3(r, W_XY + 3);
+  return M3<T>{{x.x, y.x, s.x, x.y, y.y, s.y, x.z, y.z, s.z}};
 }
-template <class T> SD void put_inertia(T* r, const S3<T>& v) {
-  const T x[6] = {v.xx, v.yy, v.zz, v.xy, v.xz, v.yz};
-  for (int i = 0; i < 6; ++i) r[(W_R + i + i / 2) * LANES] = x[i];
+template <class T> SD void put_rot(T* r, const M3<T>& R) {
+  for (int i = 0; i < 3; ++i) {
+    r[(W_S + i) * LANES] = R.a[3 * i + 2];
+    r[(W_XY + i) * LANES] = R.a[3 * i];
+    r[(W_XY + 3 + i) * LANES] = R.a[3 * i + 1];
+  }
 }
 template <class T, class DT> SD void put_wdi(T* r, DT di) {
   const T hi = (T)di;
@@ -404,7 +429,7 @@ SD void wstep_forward(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd, Co
   // outward: orientation, joint offset, velocity (a root takes R_p = 1, v_p = 0,
   // which gives its values exactly)
   {
-    Records<T, STG, 0, 0, P_E, 12> rec(s, 0, 1, walk);
+    Records<T, STG, 1, RING_FWD, 0, 0, P_E, 12> rec(s, walk);
     Inputs<T, STG, true> in(s, q, qd, 0, 1, walk);
     M3<T> R_prev = eye3<T>();
     SV<T> v_prev = zeroSV<T>();
@@ -450,7 +475,7 @@ SD void wstep_forward(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd, Co
         wv3(w, 0, 0, W_D, d);
         if (ADJ) w[W_QD * LANES] = vl;
       }
-      wm3(w, 0, 0, W_R, R);
+      put_rot(w, R);
       wsv(w, 0, 0, W_V, v);
       if (meta_treechild(m)) {
         wm3(s.stk, WSW, sp, 0, R);
@@ -464,7 +489,7 @@ SD void wstep_forward(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd, Co
   // inward: articulated inertias and bias forces, from each link's own terms and its
   // children's contributions
   {
-    Records<T, STG, W_R, W_AP - W_R, P_M, NPRM_W - P_M> rec(s, walk - 1, -1, walk);
+    Records<T, STG, -1, RING_FWD, W_D, W_AP - W_D, P_M, NPRM_W - P_M> rec(s, walk);
     Inputs<T, STG, false> in(s, tau, qd, walk - 1, -1, walk);
     SI<T> cI = zeroSI<T>();  // link l + 1's contribution if l is its parent, else 0
     SV<T> cp = zeroSV<T>();
@@ -477,7 +502,7 @@ SD void wstep_forward(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd, Co
       const int par = meta_parent(m), vo = meta_voff(m);
       T* w = tp + l * NWT * LANES;
       const bool fr = FR && meta_jtype(m) == J_FREE;
-      const M3<T> R = fld_m3(rec.t, W_R);
+      const M3<T> R = fld_rot(rec.t);
       const SV<T> v = fld_sv(rec.t, W_V);
       const V3<T> sx = col2(R);
       const T vl = in.b;
@@ -495,7 +520,7 @@ SD void wstep_forward(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd, Co
         if (fr)
           ws3(s.root, 0, 0, WF_IC, Ic);
         else
-          put_inertia(w, Ic);
+          ws3(w, 0, 0, W_XY, Ic);
         wv3(w, 0, 0, W_RW, rw);
       }
       if (meta_treechild(m)) {
@@ -538,7 +563,7 @@ SD void wstep_forward(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd, Co
     }
   }
   // outward: accelerations (and the integrator)
-  Records<T, STG, 0, W_AP, 0, 0> rec(s, 0, 1, walk);
+  Records<T, STG, 1, RING_FWD, 0, W_XY, 0, 0, 0, 0, W_V, 6> rec(s, walk);
   Inputs<T, STG, true> in(s, q, qd, 0, 1, walk);
   const SV<T> a0{zero3<T>(), -grav};
   SV<T> a_prev = a0;
@@ -552,7 +577,7 @@ SD void wstep_forward(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd, Co
     T* w = tp + l * NWT * LANES;
     SV<T> a;
     if (FR && meta_jtype(m) == J_FREE) {
-      const M3<T> R = fld_m3(rec.t, W_R);
+      const M3<T> R = fld_rot((const T*)w);
       a = wsv(w, 0, 0, W_AP);
       const SV<T> b = a - a0;
       const V3<T> bw = mulT(R, b.w), bv = mulT(R, b.v);
@@ -573,8 +598,8 @@ SD void wstep_forward(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd, Co
         for (int i = 0; i < 7; ++i) qo[qi + i] = x[i];
       }
     } else {
-      const V3<T> sx = fld_axis(rec.t);
-      const SV<T> v = fld_sv(rec.t, W_V);
+      const V3<T> sx = fld_v3(rec.t, W_S);
+      const SV<T> v = fld_sv(rec.t2, W_V);
       const SV<T> U = fld_sv(rec.t, W_U);
       const DT Di = fld_wdi<T, DT>(rec.t);
       const T u = fld(rec.t, W_u);
@@ -647,7 +672,7 @@ SD void wstep_adjoint(const WSys<T, STG>& s, Col<T> gq, Col<T> gqd, Col<T> gtau,
   const int nl = s.nl, walk = s.walk();
   // the integrator's adjoint and the inward half of lambda = M^-1 qddb (leaves -> root)
   {
-    Records<T, STG, 0, W_AP, 0, 0> rec(s, walk - 1, -1, walk);
+    Records<T, STG, -1, RING_ADJ, 0, W_XY, 0, 0> rec(s, walk);
     SV<T> cy = zeroSV<T>();
     bool carry = false;
     int sp = 0;
@@ -670,7 +695,7 @@ SD void wstep_adjoint(const WSys<T, STG>& s, Col<T> gq, Col<T> gqd, Col<T> gtau,
           if (integ == I_SEMI_IMPLICIT) nu[i] += dt * s.root[(WF_QDD + i) * LANES];
         }
         free_integrator_adjoint(qt, nu, gq, gqd, qi, vi, dt, integ, qddb6);
-        const M3<T> R = fld_m3(rec.t, W_R);
+        const M3<T> R = fld_rot((const T*)tp + l * NWT * LANES);
         y += SV<T>{mul(R, V3<T>{qddb6[0], qddb6[1], qddb6[2]}), mul(R, V3<T>{qddb6[3], qddb6[4], qddb6[5]})};
         const SV<T> w = spd_solve<T, DT>(wsi(s.root, 0, 0, WF_IA), y);
         wsv(ad, NWA, l, WA_W, zeroSV<T>() - w);
@@ -686,7 +711,7 @@ SD void wstep_adjoint(const WSys<T, STG>& s, Col<T> gq, Col<T> gqd, Col<T> gtau,
         gqd[vi] = vt;
         qddb = dt * (integ == I_SEMI_IMPLICIT ? vt : vb);
       }
-      const V3<T> sx = fld_axis(rec.t);
+      const V3<T> sx = fld_v3(rec.t, W_S);
       const SV<T> U = fld_sv(rec.t, W_U);
       const T wb = (T)((DT)(qddb + dot(sx, y.w)) * fld_wdi<T, DT>(rec.t));
       s.tp(l, W_u) = wb;
@@ -706,7 +731,7 @@ SD void wstep_adjoint(const WSys<T, STG>& s, Col<T> gq, Col<T> gqd, Col<T> gtau,
   }
   // the outward half: lambda, W = -w (root -> leaves)
   {
-    Records<T, STG, 0, W_AP, P_DAMP, 1> rec(s, 0, 1, walk);
+    Records<T, STG, 1, RING_ADJ, 0, W_XY, P_DAMP, 1> rec(s, walk);
     SV<T> W_prev = zeroSV<T>();
     int sp = 0;
     for (int l = 0; l < walk; ++l) {
@@ -728,7 +753,7 @@ SD void wstep_adjoint(const WSys<T, STG>& s, Col<T> gq, Col<T> gqd, Col<T> gtau,
         }
         const SV<T> U = fld_sv(rec.t, W_U);
         const T lam = fld(rec.t, W_u) + (T)((DT)dot(U, W) * fld_wdi<T, DT>(rec.t));
-        W.w = W.w - lam * fld_axis(rec.t);
+        W.w = W.w - lam * fld_v3(rec.t, W_S);
         wsv(ad, NWA, l, WA_W, W);
         gtau[vi] = lam;
         gqd[vi] -= fld(rec.p, P_DAMP) * lam;
@@ -742,7 +767,7 @@ SD void wstep_adjoint(const WSys<T, STG>& s, Col<T> gq, Col<T> gqd, Col<T> gtau,
   }
   // the derivative of L (leaves -> root)
   {
-    Records<T, STG, W_R, NWT - W_R, P_M, 1, WA_W, 6> rec(s, walk - 1, -1, walk);
+    Records<T, STG, -1, RING_ADJ, W_D, NWT - W_D, P_M, 1, WA_W, 6> rec(s, walk);
     SV<T> cv = zeroSV<T>(), ca = zeroSV<T>(), cw = zeroSV<T>();
     bool carry = false;
     int sp = 0;
@@ -752,12 +777,12 @@ SD void wstep_adjoint(const WSys<T, STG>& s, Col<T> gq, Col<T> gqd, Col<T> gtau,
       const int m = s.M(l);
       const int par = meta_parent(m), qi = meta_qoff(m), vi = meta_voff(m);
       const bool fr = FR && meta_jtype(m) == J_FREE;
-      const V3<T> sx = fld_axis(rec.t);
+      const V3<T> sx = fld_v3(rec.t, W_S);
       const SV<T> v = fld_sv(rec.t, W_V), ap = fld_sv(rec.t, W_AP), W = fld_sv(rec.a, WA_W);
       const T vl = fr ? T(0) : fld(rec.t, W_QD);
       const T qdd = fr ? T(0) : fld(rec.t, W_QDD);
       const SV<T> a{ap.w + qdd * sx, ap.v};
-      const S3<T> Ic = fr ? ws3(s.root, 0, 0, WF_IC) : fld_inertia(rec.t);
+      const S3<T> Ic = fr ? ws3(s.root, 0, 0, WF_IC) : fld_s3(rec.t, W_XY);
       BodyGrad<T> g = body_grad(fld(rec.p, P_M), fld_v3(rec.t, W_RW), Ic, v, a, W);
       gm[l] += g.mb;
       if (carry) {
@@ -773,7 +798,7 @@ SD void wstep_adjoint(const WSys<T, STG>& s, Col<T> gq, Col<T> gqd, Col<T> gtau,
         g.F += wsv(s.stk, WSW, sp, 12);
       }
       if (fr) {  // v = R qd, a = R qdd + [0; -g]: only the gravity does not turn with R
-        const M3<T> R = fld_m3(rec.t, W_R);
+        const M3<T> R = fld_rot(rec.t);
         const V3<T> bw = mulT(R, g.vb.w), bv = mulT(R, g.vb.v);
         const T vv[6] = {bw.x, bw.y, bw.z, bv.x, bv.y, bv.z};
         for (int i = 0; i < 6; ++i) gqd[vi + i] += vv[i];
