@@ -291,11 +291,11 @@ int sim_set_launch(sim_handle* h, int32_t threads, int32_t schedule);
  * available on them (AUTO then takes the one-warp kernels). */
 #define SIM_TAPE_ALIGNED 5
 /* SIM_TAPE_ALIGNED_PIPELINED is SIM_TAPE_ALIGNED with the adjoint (checkpoint
- * interval 1) on two warps per 32-system tile: one recomputes step t's forward
- * intermediates (Sec. 3.2, Eq. 7) into one of two tapes while the other runs the
- * adjoint of step t + 1 from the other tape (on chip when a tile's tapes fit a
- * block, else in global memory).  AUTO uses this adjoint wherever it uses the
- * world-aligned kernels with k = 1. */
+ * interval 1, or segment replay) on two to four warps per 32-system tile: the
+ * producers recompute steps' forward intermediates (Sec. 3.2, Eq. 7) ahead, each into
+ * its own tape, while one warp runs the adjoint of step after step (tapes on chip
+ * when they fit a block, else in global memory).  AUTO uses this adjoint wherever it
+ * uses the world-aligned kernels, except for the quadratic replay. */
 #define SIM_TAPE_ALIGNED_PIPELINED 6
 int sim_set_tape_space(sim_handle* h, int32_t space);
 

@@ -1,6 +1,6 @@
 """Build the CUDA library in-tree: ``csrc/*.cu`` -> ``_lib/libabasim.so``.
 
-Twenty-two translation units (the host side of the C ABI; kernel instantiation
+Twenty-five translation units (the host side of the C ABI; kernel instantiation
 units per precision, direction and adjoint storage mode; the kernels of models
 with contact spheres per precision; the world-aligned kernels per precision and
 direction, and their pipelined adjoint per precision), compiled by nvcc for sm_103a only, in parallel, then linked; beside it
@@ -24,7 +24,8 @@ INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 SOURCES = ["abasim.cu", "inst_fp32_fwd.cu", "inst_fp32_bwd.cu", "inst_fp32_bwd_hybrid.cu",
            "inst_fp32_bwd_smem.cu", "inst_mixed_fwd.cu", "inst_mixed_bwd.cu", "inst_mixed_bwd_hybrid.cu",
            "inst_mixed_bwd_smem.cu", "inst_fp64.cu", "inst_fp32_contact.cu", "inst_mixed_contact.cu",
-           "inst_fp64_contact.cu", "inst_w_fp32_fwd.cu", "inst_w_fp32_bwd.cu", "inst_w_mixed_fwd.cu", "inst_w_mixed_bwd.cu", "inst_w_fp64_fwd.cu", "inst_w_fp64_bwd.cu", "inst_wp_fp32.cu", "inst_wp_mixed.cu", "inst_wp_fp64.cu"]
+           "inst_fp64_contact.cu", "inst_w_fp32_fwd.cu", "inst_w_fp32_bwd.cu", "inst_w_mixed_fwd.cu", "inst_w_mixed_bwd.cu", "inst_w_fp64_fwd.cu", "inst_w_fp64_bwd.cu", "inst_wp_fp32.cu", "inst_wp_mixed.cu", "inst_wp_fp64.cu",
+           "inst_wps_fp32.cu", "inst_wps_mixed.cu", "inst_wps_fp64.cu"]
 DEPS = SOURCES + ["fma_peak.cu", "aba_step.cuh", "contact.cuh", "spatial.cuh", "twofloat.cuh", "dual.cuh", "kernels.cuh", "handle.h",
                   "wstep.cuh", "wkernels.cuh", "wpipe.cuh", "tree_order.h"]
 

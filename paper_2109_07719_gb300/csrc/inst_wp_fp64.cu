@@ -5,12 +5,12 @@
 namespace abasim {
 namespace host {
 
-template <class T, class DT>
+template <class T, class DT, bool SEG>
 BackwardKernel<T> wbackward_pipe_kernel(bool onchip, bool fr) {
-  if (fr) return onchip ? k_wbackward_pipe<T, DT, true, true> : k_wbackward_pipe<T, DT, false, true>;
-  return onchip ? k_wbackward_pipe<T, DT, true, false> : k_wbackward_pipe<T, DT, false, false>;
+  if (fr) return onchip ? k_wbackward_pipe<T, DT, true, true, SEG> : k_wbackward_pipe<T, DT, false, true, SEG>;
+  return onchip ? k_wbackward_pipe<T, DT, true, false, SEG> : k_wbackward_pipe<T, DT, false, false, SEG>;
 }
-template BackwardKernel<double> wbackward_pipe_kernel<double, double>(bool, bool);
+template BackwardKernel<double> wbackward_pipe_kernel<double, double, false>(bool, bool);
 
 }  // namespace host
 }  // namespace abasim

@@ -42,6 +42,7 @@ template <class T> struct DevModel {
   int slots;     // world-aligned kernels with a global tape: slots of a warp's ring, 3 or 1 (no look-ahead)
   T* stk;        // world-aligned kernels: two stacks of parent values [2][tiles][wdepth][WSW][lane] (null: none)
   int wdepth;    // entries per stack
+  T* tapes;      // pipelined world-aligned adjoint: [WPIPE_TAPES][tile][tape words][lane]
   int sd;        // scalars of a system's stack in shared memory beside a global tape (0: in stk)
 };
 
@@ -51,7 +52,8 @@ template <class T> DevModel<T> dev_model(const sim_handle* h) {
                      (T)h->g[0], (T)h->g[1], (T)h->g[2], h->integrator, 0, 0,
                      h->replay == SIM_REPLAY_QUADRATIC, (T*)h->ctape, (T*)h->csys,
                      ContactParams<T>{(T)h->friction, (T)h->erp, h->pgs_iterations}, h->dt,
-                     h->state64 ? (double*)h->x64 : nullptr, h->prefetch > 0 ? 3 : 1, (T*)h->wstk, h->wdepth, 0};
+                     h->state64 ? (double*)h->x64 : nullptr, h->prefetch > 0 ? 3 : 1, (T*)h->wstk, h->wdepth,
+                     (T*)(h->wtapes ? h->wtapes : h->tape), 0};
 }
 
 extern __shared__ __align__(16) unsigned char g_smem[];
@@ -773,7 +775,7 @@ template <class T, class DT>
 RolloutKernel<T> wrollout_kernel(bool onchip, bool fr);
 template <class T, class DT>
 BackwardKernel<T> wbackward_kernel(bool onchip, bool fr);
-template <class T, class DT>
+template <class T, class DT, bool SEG>
 BackwardKernel<T> wbackward_pipe_kernel(bool onchip, bool fr);
 
 // One step with tangents: the state, torque and tape are dual numbers staged in
@@ -996,7 +998,7 @@ int choose_w(sim_handle* h, K k_on, K k_off, bool bwd, bool* onchip, int* thread
 // against the link-frame one-warp kernels, 1024 humanoids over 60 steps (FP32) 10.95
 // -> 4.39 ms.
 template <class T, class DT>
-bool use_aligned(const sim_handle* h, bool rollout, int k) {
+bool use_aligned(const sim_handle* h, bool rollout) {
   const bool fr = !h->all_revolute;
   if (!h->unconstrained || (rollout && h->state64)) return false;
   if (fr && h->tape_space != SIM_TAPE_AUTO) return false;
@@ -1033,12 +1035,13 @@ int launch_wrollout(sim_handle* h, const void* q0, const void* qd0, const void* 
   return e == cudaSuccess ? SIM_OK : cuda_fail(h, e, "rollout launch");
 }
 
-// The pipelined world-aligned adjoint (k = 1): one consumer warp and np producer warps per
+// The pipelined world-aligned adjoint (k = 1, or segment replay: 1500 trees of 2-40 links
+// with k = 8 went from 168 us a step, replay, recompute and adjoint in one warp, to 116): one consumer warp and np producer warps per
 // 32-system tile, their tapes on chip when they fit a block, else in global memory.
 template <class T, class DT>
-int launch_wbackward_pipe(sim_handle* h, const void* ckpt, const void* tau, int64_t T_, const void* gqT,
+int launch_wbackward_pipe(sim_handle* h, const void* ckpt, const void* tau, int64_t T_, int k, const void* gqT,
                           const void* gqdT, const void* gtraj, void* gq0, void* gqd0, void* gtau, void* gmass,
-                          void* stream) {
+                          void* work, void* stream) {
   DevModel<T> m = dev_model<T>(h);
   int limit = 0;
   cudaError_t e = cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
@@ -1066,7 +1069,8 @@ int launch_wbackward_pipe(sim_handle* h, const void* ckpt, const void* tau, int6
   const size_t shm = need(onchip, np);
   if (shm > (size_t)limit) return fail(h, SIM_EUNSUPPORTED, "the working state does not fit in shared memory");
   const int threads = (np + 1) * LANES;
-  const BackwardKernel<T> kern = wbackward_pipe_kernel<T, DT>(onchip, fr);
+  const BackwardKernel<T> kern =
+      k > 1 ? wbackward_pipe_kernel<T, DT, true>(onchip, fr) : wbackward_pipe_kernel<T, DT, false>(onchip, fr);
   e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
   if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory opt-in");
   if (!onchip) {  // shared memory for the blocks an SM holds at once, the rest of the SM's storage as L1
@@ -1078,9 +1082,9 @@ int launch_wbackward_pipe(sim_handle* h, const void* ckpt, const void* tau, int6
   int grid = 0;
   int rc = launch_shape(h, kern, &grid, &m.persistent, shm, stream, threads, LANES);
   if (rc != SIM_OK) return rc;
-  kern<<<grid, threads, shm, S(stream)>>>(m, (const T*)ckpt, (const T*)tau, (long long)T_, 1, (const T*)gqT,
+  kern<<<grid, threads, shm, S(stream)>>>(m, (const T*)ckpt, (const T*)tau, (long long)T_, k, (const T*)gqT,
                                           (const T*)gqdT, (const T*)gtraj, (T*)gq0, (T*)gqd0, (T*)gtau,
-                                          (T*)h->gm_acc, (T*)(h->wtapes ? h->wtapes : h->tape));
+                                          (T*)h->gm_acc, (T*)work);
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(h, e, "backward launch");
   if (gmass) {
@@ -1097,8 +1101,8 @@ int launch_wbackward(sim_handle* h, const void* ckpt, const void* tau, int64_t T
                      const void* gqdT, const void* gtraj, void* gq0, void* gqd0, void* gtau, void* gmass, void* work,
                      void* stream) {
   DevModel<T> m = dev_model<T>(h);
-  if (k == 1 && T_ > 0 && h->tape_space != SIM_TAPE_ALIGNED)
-    return launch_wbackward_pipe<T, DT>(h, ckpt, tau, T_, gqT, gqdT, gtraj, gq0, gqd0, gtau, gmass, stream);
+  if (T_ > 0 && h->tape_space != SIM_TAPE_ALIGNED && (k == 1 || !m.quadratic))
+    return launch_wbackward_pipe<T, DT>(h, ckpt, tau, T_, k, gqT, gqdT, gtraj, gq0, gqd0, gtau, gmass, work, stream);
   const BackwardKernel<T> k_on = wbackward_kernel<T, DT>(true, !h->all_revolute),
                           k_off = wbackward_kernel<T, DT>(false, !h->all_revolute);
   bool onchip = false;
@@ -1128,7 +1132,7 @@ int launch_wbackward(sim_handle* h, const void* ckpt, const void* tau, int64_t T
 template <class T, class DT>
 int launch_rollout(sim_handle* h, const void* q0, const void* qd0, const void* tau, int64_t T_,
                    int k, void* ckpt, void* qT, void* qdT, void* traj, void* stream) {
-  if (use_aligned<T, DT>(h, true, k)) return launch_wrollout<T, DT>(h, q0, qd0, tau, T_, k, ckpt, qT, qdT, traj, stream);
+  if (use_aligned<T, DT>(h, true)) return launch_wrollout<T, DT>(h, q0, qd0, tau, T_, k, ckpt, qT, qdT, traj, stream);
   if (h->tape_space == SIM_TAPE_ALIGNED || h->tape_space == SIM_TAPE_ALIGNED_PIPELINED)
     return fail(h, SIM_EUNSUPPORTED,
                 "the world-aligned kernels need revolute joints only, no contact spheres or limits, FP32 state sums "
@@ -1187,7 +1191,7 @@ template <class T, class DT>
 int launch_backward(sim_handle* h, const void* ckpt, const void* tau, int64_t T_, int k,
                     const void* gqT, const void* gqdT, const void* gtraj, void* gq0, void* gqd0,
                     void* gtau, void* gmass, void* work, void* stream) {
-  if (use_aligned<T, DT>(h, false, k))
+  if (use_aligned<T, DT>(h, false))
     return launch_wbackward<T, DT>(h, ckpt, tau, T_, k, gqT, gqdT, gtraj, gq0, gqd0, gtau, gmass, work, stream);
   if (h->tape_space == SIM_TAPE_ALIGNED || h->tape_space == SIM_TAPE_ALIGNED_PIPELINED)
     return fail(h, SIM_EUNSUPPORTED, "the world-aligned kernels need revolute joints only, no contact spheres or "

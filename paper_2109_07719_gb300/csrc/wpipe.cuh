@@ -1,6 +1,5 @@
 // The pipelined adjoint of the world-aligned step: a consumer warp and one or more
-// producer warps per 32-system tile, for models without contacts or limits and a
-// checkpoint every step.  With every step's initial state checkpointed, the recompute
+// producer warps per 32-system tile, for models without contacts or limits.  With every step's initial state checkpointed, the recompute
 // of step t (Sec. 3.2, Eq. 7: Z^t = G(x^t)) depends on no adjoint, so the producers
 // recompute steps ahead, in turn, into a ring of tapes while the consumer runs the
 // adjoint of step after step.  Step j (counted from the last one) lives in tape j mod NT
@@ -13,6 +12,12 @@
 // the other's matching wait: a tape's next FULL arrival follows its EMPTY wait, which
 // follows the consumer's FULL wait, and vice versa.  (A tape shared by several producers
 // would need more: one could take the EMPTY arrival meant for another.)
+//
+// SEG, a checkpoint every k > 1 steps: a segment's states are replayed once into the
+// caller's workspace by the producer of the segment's first (latest) step, with that step's
+// tape as scratch, between two barriers of the producers (all have read the previous
+// segment's states; all may read this one's); the consumer meanwhile finishes the steps of
+// the previous segment.
 //
 // Why several producers: the implicit-form adjoint takes less time than the recompute
 // (468 against 736 operations a link), so with one producer the consumer waits; how many
@@ -42,14 +47,19 @@ __host__ __device__ __forceinline__ long long wpipe_smem_per_tile(int maxL, int 
 __device__ __forceinline__ void pipe_sync(int id) { asm volatile("bar.sync %0, 64;\n" ::"r"(id) : "memory"); }
 __device__ __forceinline__ void pipe_arrive(int id) { asm volatile("bar.arrive %0, 64;\n" ::"r"(id) : "memory"); }
 
+// all producers of a block
+__device__ __forceinline__ void producers_sync(int nt, int np) {
+  asm volatile("bar.sync %0, %1;\n" ::"r"(1 + 2 * nt), "r"(np * LANES) : "memory");
+}
+
 // Registers: an on-chip block may have its SM alone; three global-tape blocks of one consumer
 // and up to three producers share one (FP64: two).
-template <class T, class DT, bool ONCHIP, bool FR>
+template <class T, class DT, bool ONCHIP, bool FR, bool SEG>
 __global__ void __launch_bounds__(LANES * (WPIPE_TAPES + 1),
                                   ONCHIP ? 1 : sizeof(T) == 4 ? 3 : 2)
 k_wbackward_pipe(DevModel<T> m, const T* __restrict__ ckpt, const T* __restrict__ tau, long long Tn, int k,
                  const T* __restrict__ gqT, const T* __restrict__ gqdT, const T* __restrict__ gtraj, T* gq0,
-                 T* gqd0, T* gtau, T* gm_acc, T* tapes) {
+                 T* gqd0, T* gtau, T* gm_acc, T* ring) {
   const int warp = threadIdx.x / LANES, lane = threadIdx.x % LANES;
   const int NP = blockDim.x / LANES - 1, NT = wpipe_tapes(NP);
   const bool consumer = warp == 0;
@@ -106,53 +116,89 @@ k_wbackward_pipe(DevModel<T> m, const T* __restrict__ ckpt, const T* __restrict_
         T* tape = s_tape + buf * TW * LANES + lane;
         return WSys<T>{s_prm + lane, meta_l, tape, s_adj + lane, nl, MS, NPRM_W, s_stk, tape + L * NWT * LANES};
       } else {
-        T* tape = tapes + (buf * units + unit) * TW * LANES + lane;
+        T* tape = m.tapes + (buf * units + unit) * TW * LANES + lane;
         return WSys<T, true>{gprm, gmeta, tape, m.adj + (long long)unit * L * NWA * LANES + lane, nl, 1, NPRM,
                              m.sd ? s_stk : w_stack(m, warp, unit, lane), tape + L * NWT * LANES, links, s_ring,
                              m.slots > 1, lane};
       }
     };
+    // x^t: the checkpoint, or (SEG) the replayed state of the segment that starts at t0
+    auto state_of = [&](long long t, long long t0) -> const T* {
+      return SEG ? ring + (t - t0) * NX * B + (act ? slot : 0) : ckpt + t * NX * B + b;
+    };
     // a producer's inputs of step t: x^t and tau^t (the system's own coordinates)
-    auto fetch = [&](long long t, int buf) {
+    auto fetch = [&](long long t, long long t0, int buf) {
       T* dst = s_in + buf * W * LANES + lane;
-      for (int d = 0; d < nq; ++d) cp_async(dst + d * LANES, ckpt + (t * NX + d) * B + b);
-      for (int d = 0; d < nv; ++d) cp_async(dst + (nqm + d) * LANES, ckpt + (t * NX + nqm + d) * B + b);
+      const T* x = state_of(t, t0);
+      for (int d = 0; d < nq; ++d) cp_async(dst + d * LANES, x + d * B);
+      for (int d = 0; d < nv; ++d) cp_async(dst + (nqm + d) * LANES, x + (nqm + d) * B);
       for (int d = 0; d < nv; ++d) cp_async(dst + (NX + d) * LANES, tau + (t * nvm + d) * B + b);
     };
-    if (!consumer) {  // producer `warp`: recompute steps j = warp - 1, warp - 1 + NP, ...
-      int in = 0;
-      if (ONCHIP) {
-        if (act && warp - 1 < Tn) fetch(Tn - warp, 0);
-        cp_commit();
-      }
-      int buf = (warp - 1) % NT;
-      for (long long j = warp - 1; j < Tn; j += NP, in ^= 1) {
-        const long long t = Tn - 1 - j;
-        if (ONCHIP) {
-          if (act && t >= NP) fetch(t - NP, in ^ 1);
-          cp_commit();
-          cp_wait_all_but_newest();
-        } else if (act && t >= NP && m.slots > 1) {
-          const T* xn = ckpt + (t - NP) * NX * B + b;
-          for (int d = 0; d < nq; ++d) pf_line(xn + d * B);
-          for (int d = 0; d < nv; ++d) pf_line(xn + (nqm + d) * B);
-          for (int d = 0; d < nv; ++d) pf_line(tau + ((t - NP) * nvm + d) * B + b);
-        }
-        __syncwarp();
-        if (j >= NT) pipe_sync(1 + NT + buf);
-        if (ONCHIP ? act : true) {
-          const WSys<T, !ONCHIP> sp = sys_of_buf(buf);
-          const T* x = ONCHIP ? s_in + in * W * LANES + lane : ckpt + t * NX * B + b;
-          const T* ta = ONCHIP ? x + NX * LANES : tau + t * nvm * B + b;
-          const long long st = ONCHIP ? (long long)LANES : B;
-          wstep_forward<T, DT, true, false, FR>(sp, Col<const T>{x, st}, Col<const T>{x + nqm * st, st},
-                                                Col<const T>{ta, st}, g, m.dt, m.integ, Col<T>{nullptr, 0},
-                                                Col<T>{nullptr, 0});
-        }
+    // the segment's states x^{t0 + 1} .. x^{t1 - 1} from its checkpoint, one step each
+    auto replay = [&](const WSys<T, !ONCHIP>& sp, long long seg, long long t0, long long t1) {
+      if constexpr (SEG) {
+        T* r = ring + (act ? slot : 0);
+        const T* xs = ckpt + seg * NX * B + b;
+        if (act)
+          for (int d = 0; d < NX; ++d) r[d * B] = xs[d * B];
+        if (ONCHIP ? act : true)
+          for (long long t = t0; t + 1 < t1; ++t, r += NX * B)
+            wstep_forward<T, DT, false, true, FR>(sp, Col<const T>{r, B}, Col<const T>{r + nqm * B, B},
+                                                  Col<const T>{tau + t * nvm * B + b, B}, g, m.dt, m.integ,
+                                                  Col<T>{r + NX * B, B}, Col<T>{r + (NX + nqm) * B, B});
         __threadfence_block();
         __syncwarp();
-        pipe_arrive(1 + buf);
-        buf = (buf + NP) % NT;
+      }
+    };
+    if (!consumer) {  // producer `warp`: recompute steps j = warp - 1, warp - 1 + NP, ...
+      long long j = warp - 1;
+      int buf = (warp - 1) % NT, in = 0;
+      // the whole rollout, or segment after segment
+      for (long long seg = SEG ? (Tn + k - 1) / k - 1 : 0; seg >= 0; --seg) {
+        const long long t0 = SEG ? seg * k : 0, t1 = SEG && t0 + k < Tn ? t0 + k : Tn;
+        bool mine = false;  // SEG: this warp replays the segment (its tape is then free)
+        if (SEG) {
+          mine = j == Tn - t1;
+          if (NP > 1) producers_sync(NT, NP);
+          if (mine) {
+            if (j >= NT) pipe_sync(1 + NT + buf);
+            replay(sys_of_buf(buf), seg, t0, t1);
+          }
+          if (NP > 1) producers_sync(NT, NP);
+        }
+        if (ONCHIP) {
+          if (act && Tn - 1 - j >= t0) fetch(Tn - 1 - j, t0, in);
+          cp_commit();
+        }
+        for (; Tn - 1 - j >= t0; j += NP, in ^= 1) {
+          const long long t = Tn - 1 - j;
+          if (ONCHIP) {
+            if (act && t - NP >= t0) fetch(t - NP, t0, in ^ 1);
+            cp_commit();
+            cp_wait_all_but_newest();
+          } else if (act && t - NP >= t0 && m.slots > 1) {
+            const T* xn = state_of(t - NP, t0);
+            for (int d = 0; d < nq; ++d) pf_line(xn + d * B);
+            for (int d = 0; d < nv; ++d) pf_line(xn + (nqm + d) * B);
+            for (int d = 0; d < nv; ++d) pf_line(tau + ((t - NP) * nvm + d) * B + b);
+          }
+          __syncwarp();
+          if (j >= NT && !mine) pipe_sync(1 + NT + buf);
+          mine = false;
+          if (ONCHIP ? act : true) {
+            const WSys<T, !ONCHIP> sp = sys_of_buf(buf);
+            const T* x = ONCHIP ? s_in + in * W * LANES + lane : state_of(t, t0);
+            const T* ta = ONCHIP ? x + NX * LANES : tau + t * nvm * B + b;
+            const long long st = ONCHIP ? (long long)LANES : B;
+            wstep_forward<T, DT, true, false, FR>(sp, Col<const T>{x, st}, Col<const T>{x + nqm * st, st},
+                                                  Col<const T>{ta, st}, g, m.dt, m.integ, Col<T>{nullptr, 0},
+                                                  Col<T>{nullptr, 0});
+          }
+          __threadfence_block();
+          __syncwarp();
+          pipe_arrive(1 + buf);
+          buf = (buf + NP) % NT;
+        }
       }
       if (ONCHIP) cp_wait_all();
     } else {  // consumer: the adjoint of step after step
