@@ -47,6 +47,7 @@ constexpr int MAXC = SIM_MAX_CONTACTS;         // contact spheres per system
 constexpr int MAXL = SIM_MAX_LIMITS;           // limited joints per system
 constexpr int NROW = 3 * MAXC + MAXL;          // impulse rows: world x, y, z per contact, then limits
 constexpr int MAXPGS = SIM_MAX_PGS_ITERATIONS;  // Gauss-Seidel sweeps
+constexpr int CT_WARPS = 4;                    // warps of a contact kernel that share a system's test passes
 
 // per-system contact record, [field][system]
 enum : int {
@@ -62,13 +63,17 @@ enum : int {
   S_AB = S_NL + 1,               // adjoint of A
   S_BB = S_AB + NROW * NROW,     // adjoint of b
   S_LB = S_BB + NROW,            // adjoint of lambda
-  NCS = S_LB + NROW
+  S_RD = S_LB + NROW,            // 1 / A_rr (a division is 10 FP64 instructions; one to four an update otherwise)
+  NCS = S_RD + NROW
 };
 
 template <class T> struct CView {
   T* ct;  // per-link contact tape of this system: [link][NCT][LANES] at its lane
   T* cs;  // per-system contact record: [NCS][LANES] at its lane
-  SD T& L(int l, int f) const { return ct[(l * NCT + f) * LANES]; }
+  // where the fields from B_U on (a test pass's scratch and the adjoint accumulators) live,
+  // when several warps run test passes of one system at once: a contact tape of this warp's
+  T* own = nullptr;
+  SD T& L(int l, int f) const { return (own && f >= B_U ? own : ct)[(l * NCT + f) * LANES]; }
   SD T& S(int f) const { return cs[f * LANES]; }
 };
 
@@ -359,7 +364,7 @@ SD void gs_update(const CView<T>& cv, int r, int nr, bool box, T hi) {
   const T lr = cv.S(S_LF + r);
   T res = cv.S(S_B + r);
   for (int k = 0; k < nr; ++k) res += cv.S(S_A + r * NROW + k) * cv.S(S_LF + k);
-  const T sv = lr - res / cv.S(S_A + r * NROW + r);
+  const T sv = lr - res * cv.S(S_RD + r);
   T ln;
   if (!box) {
     ln = sv > T(0) ? sv : T(0);
@@ -406,12 +411,38 @@ SD TPIn<T> impulse_inputs(const CView<T>& cv, int nc, int nlr, const int* link, 
   return in;
 }
 
-// Contact and limit impulses of one step; requires aba_forward to have filled the
-// tape (unconstrained qdd included).  Leaves the velocity change in C_DV of every
-// link and returns the number of active rows (0: C_DV is not written and the step
-// has no constraint term).
+// The active rows of a system, from its contact record.
+template <class T> struct Rows {
+  int nc, nlr, nr;
+  int link[MAXC], llink[MAXL];
+  V3<T> pc[MAXC];
+  T lsg[MAXL];
+};
+template <class T, class PT> SD Rows<T> active_rows(const Sys<T, PT>& s, const CView<T>& cv) {
+  Rows<T> r;
+  r.nc = (int)cv.S(S_NC);
+  r.nlr = (int)cv.S(S_NL);
+  r.nr = 3 * r.nc + r.nlr;
+  for (int c = 0; c < r.nc; ++c) {
+    r.link[c] = (int)cv.S(S_LINK + c);
+    r.pc[c] = s.pv3(r.link[c], P_CP);
+  }
+  for (int k = 0; k < r.nlr; ++k) {
+    r.llink[k] = (int)cv.S(S_LINK + MAXC + k);
+    r.lsg[k] = cv.S(S_SGN + k);
+  }
+  return r;
+}
+
+// The constraint step is in parts, so that several warps can share one system's columns
+// of A (each with a contact tape of its own for the test passes): the rows and b
+// (contact_rows), the columns in groups of three (contact_columns, group j of `parts`
+// warps' share by j mod parts), the sweeps and the velocity change (contact_solve).
+//
+// Detection, rows and b; requires aba_forward to have filled the tape (unconstrained qdd
+// included).  Returns the number of active rows.
 template <class T, class DT, class PT>
-CD int contact_forward(Sys<T, PT> s, CView<T> cv, Col<const T> q, Col<const T> qd, T dt, ContactParams<T> cp) {
+CD int contact_rows(Sys<T, PT> s, CView<T> cv, Col<const T> q, Col<const T> qd, T dt, ContactParams<T> cp) {
   const int nl = s.nl;
   world_poses(s, cv);
   int nc = 0;
@@ -490,8 +521,17 @@ CD int contact_forward(Sys<T, PT> s, CView<T> cv, Col<const T> q, Col<const T> q
     const T vstar = qd[meta_voff(s.M(l))] + dt * s.tp(l, T_QDD);
     cv.S(S_B + 3 * nc + k) = lsg[k] * vstar + kphi * cv.S(S_PHI + MAXC + k);
   }
-  // A, three columns (right-hand sides) per test pass
-  for (int j0 = 0; j0 < nr; j0 += 3) {
+  return nr;
+}
+
+// A, three columns (right-hand sides) per test pass.
+template <class T, class DT, class PT> CD void contact_columns(Sys<T, PT> s, CView<T> cv, int part, int parts) {
+  const Rows<T> rows = active_rows(s, cv);
+  const int nc = rows.nc, nlr = rows.nlr, nr = rows.nr;
+  const int *link = rows.link, *llink = rows.llink;
+  const V3<T>* pc = rows.pc;
+  const T* lsg = rows.lsg;
+  for (int j0 = 3 * part; j0 < nr; j0 += 3 * parts) {
     const TPIn<T> in = unit_inputs(cv, nc, nr, j0, link, pc, llink, lsg);
     test_pass<T, DT, PT, 3>(s, cv, in, C_TQ);
     for (int r = 0; r < 3 && j0 + r < nr; ++r) {
@@ -507,8 +547,17 @@ CD int contact_forward(Sys<T, PT> s, CView<T> cv, Col<const T> q, Col<const T> q
         cv.S(S_A + (3 * nc + k2) * NROW + j) = lsg[k2] * cv.L(llink[k2], C_TQ + 6 * r);
     }
   }
+}
+
+// The Gauss-Seidel sweeps and the velocity change, left in C_DV of every link.
+template <class T, class DT, class PT> CD void contact_solve(Sys<T, PT> s, CView<T> cv, ContactParams<T> cp) {
+  const Rows<T> rows = active_rows(s, cv);
+  const int nc = rows.nc, nlr = rows.nlr, nr = rows.nr;
   // projected Gauss-Seidel
-  for (int r = 0; r < nr; ++r) cv.S(S_LF + r) = T(0);
+  for (int r = 0; r < nr; ++r) {
+    cv.S(S_LF + r) = T(0);
+    cv.S(S_RD + r) = T(1) / cv.S(S_A + r * NROW + r);
+  }
   for (int it = 0; it < cp.iters; ++it) {
     for (int c = 0; c < nc; ++c) {
       for (int qq = 0; qq < 3; ++qq) {
@@ -524,7 +573,18 @@ CD int contact_forward(Sys<T, PT> s, CView<T> cv, Col<const T> q, Col<const T> q
     }
   }
   // velocity change M^-1 J^T lambda
-  test_pass<T, DT, PT, 1>(s, cv, impulse_inputs(cv, nc, nlr, link, pc, llink, lsg), C_DV);
+  test_pass<T, DT, PT, 1>(s, cv, impulse_inputs(cv, nc, nlr, rows.link, rows.pc, rows.llink, rows.lsg), C_DV);
+}
+
+// Contact and limit impulses of one step in one thread.  Returns the number of active
+// rows (0: C_DV is not written and the step has no constraint term).
+template <class T, class DT, class PT>
+CD int contact_forward(Sys<T, PT> s, CView<T> cv, Col<const T> q, Col<const T> qd, T dt, ContactParams<T> cp) {
+  const int nr = contact_rows<T, DT, PT>(s, cv, q, qd, dt, cp);
+  if (nr > 0) {
+    contact_columns<T, DT, PT>(s, cv, 0, 1);
+    contact_solve<T, DT, PT>(s, cv, cp);
+  }
   return nr;
 }
 
@@ -539,10 +599,10 @@ SD void gs_update_reverse(const CView<T>& cv, int it, int r, int nr, bool box, i
   const T lr = cv.S(S_LAM + it * NROW + r);
   cv.S(S_LF + r) = lr;  // the vector as the update saw it
   cv.S(S_LB + r) = T(0);
-  const T Arr = cv.S(S_A + r * NROW + r);
+  const T rd = cv.S(S_RD + r);
   T res = cv.S(S_B + r);
   for (int k = 0; k < nr; ++k) res += cv.S(S_A + r * NROW + k) * cv.S(S_LF + k);
-  const T sv = lr - res / Arr;
+  const T sv = lr - res * rd;
   T sb = T(0);
   if (!box) {
     if (sv >= T(0)) sb = lnb;
@@ -556,39 +616,36 @@ SD void gs_update_reverse(const CView<T>& cv, int it, int r, int nr, bool box, i
   }
   if (sb != T(0)) {  // sv = lambda_r - (A_r . lambda + b_r) / A_rr
     cv.S(S_LB + r) += sb;
-    const T g = sb / Arr;
+    const T g = sb * rd;
     for (int k = 0; k < nr; ++k) {
       cv.S(S_LB + k) -= g * cv.S(S_A + r * NROW + k);
       cv.S(S_AB + r * NROW + k) -= g * cv.S(S_LF + k);
     }
     cv.S(S_BB + r) -= g;
-    cv.S(S_AB + r * NROW + r) += g * res / Arr;
+    cv.S(S_AB + r * NROW + r) += g * (res * rd);
   }
 }
 
-// Requires aba_forward and contact_forward (with active rows) of the same step,
-// and the adjoint of the unconstrained-plus-constraint qdd from the integrator
-// adjoint in C_QDDB (dt times the adjoint of qd').  Fills the B_* fields.
+// The accumulators a test pass's reverse adds to, zeroed for every link (all: the whole
+// B_* range).
+template <class T, class PT> SD void zero_accumulators(const Sys<T, PT>& s, const CView<T>& cv, int end) {
+  for (int l = 0; l < s.nl; ++l)
+    for (int f = B_U; f < end; ++f) cv.L(l, f) = T(0);
+}
+
+// The constraint adjoint, in parts as the forward step.  It requires aba_forward and the
+// forward parts (with active rows) of the same step, and the adjoint of the
+// unconstrained-plus-constraint qdd from the integrator adjoint in C_QDDB (dt times the
+// adjoint of qd'), and fills the B_* fields.  First the velocity change and the sweeps:
 template <class T, class DT, class PT>
-CD void contact_adjoint(Sys<T, PT> s, CView<T> cv, T dt, ContactParams<T> cp) {
+CD void contact_adjoint_solve(Sys<T, PT> s, CView<T> cv, T dt, ContactParams<T> cp) {
   const int nl = s.nl;
-  const int nc = (int)cv.S(S_NC);
-  const int nlr = (int)cv.S(S_NL);
-  const int nr = 3 * nc + nlr;
-  for (int l = 0; l < nl; ++l)
-    for (int f = B_U; f < B_END; ++f) cv.L(l, f) = T(0);
-  int link[MAXC];
-  V3<T> pc[MAXC];
-  for (int c = 0; c < nc; ++c) {
-    link[c] = (int)cv.S(S_LINK + c);
-    pc[c] = s.pv3(link[c], P_CP);
-  }
-  int llink[MAXL];
-  T lsg[MAXL];
-  for (int k = 0; k < nlr; ++k) {
-    llink[k] = (int)cv.S(S_LINK + MAXC + k);
-    lsg[k] = cv.S(S_SGN + k);
-  }
+  const Rows<T> rows = active_rows(s, cv);
+  const int nc = rows.nc, nlr = rows.nlr, nr = rows.nr;
+  const int *link = rows.link, *llink = rows.llink;
+  const V3<T>* pc = rows.pc;
+  const T* lsg = rows.lsg;
+  zero_accumulators(s, cv, B_END);
   // 1. the velocity change dv = M^-1 J^T lambda; dv enters qd' directly
   {
     const TPIn<T> in = impulse_inputs(cv, nc, nlr, link, pc, llink, lsg);
@@ -617,8 +674,19 @@ CD void contact_adjoint(Sys<T, PT> s, CView<T> cv, T dt, ContactParams<T> cp) {
     for (int c = nc - 1; c >= 0; --c)
       for (int qq = 2; qq >= 0; --qq) gs_update_reverse(cv, it, contact_row(c, qq), nr, qq != 0, 3 * c + 2, cp.mu);
   }
-  // 3. the columns of A, three per test pass
-  for (int j0 = 0; j0 < nr; j0 += 3) {
+}
+
+// the columns of A, three per test pass (each warp's share into its own accumulators):
+template <class T, class DT, class PT>
+CD void contact_adjoint_columns(Sys<T, PT> s, CView<T> cv, int part, int parts) {
+  const int nl = s.nl;
+  const Rows<T> rows = active_rows(s, cv);
+  const int nc = rows.nc, nlr = rows.nlr, nr = rows.nr;
+  const int *link = rows.link, *llink = rows.llink;
+  const V3<T>* pc = rows.pc;
+  const T* lsg = rows.lsg;
+  // 3. the columns of A
+  for (int j0 = 3 * part; j0 < nr; j0 += 3 * parts) {
     const TPIn<T> in = unit_inputs(cv, nc, nr, j0, link, pc, llink, lsg);
     test_pass<T, DT, PT, 3>(s, cv, in, -1);
     for (int l = 0; l < nl; ++l)
@@ -655,6 +723,33 @@ CD void contact_adjoint(Sys<T, PT> s, CView<T> cv, T dt, ContactParams<T> cp) {
       caddm(cv, link[c], B_EW, outer(flb, ek));
     }
   }
+}
+
+// the other warps' accumulators (contact tapes `stride` apart) added to the system's, links
+// part, part + parts, ...:
+template <class T, class PT> CD void contact_adjoint_sum(Sys<T, PT> s, CView<T> cv, long long stride, int part, int parts) {
+  const int groups = ((int)cv.S(S_NC) * 3 + (int)cv.S(S_NL) + 2) / 3;
+  const int copies = groups < parts ? groups : parts;
+  for (int l = part; l < s.nl; l += parts) {
+    const bool rev = meta_jtype(s.M(l)) == J_REVOLUTE;
+    for (int f = B_U; f < B_OW; ++f) {
+      if (rev && f == B_IA) f = B_E;  // only a free root has an articulated-inertia adjoint
+      T* w = cv.ct + (l * NCT + f) * LANES;
+      T sum = *w;
+      for (int c = 1; c < copies; ++c) sum += w[c * stride];
+      *w = sum;
+    }
+  }
+}
+
+// and b, the link velocities and the world kinematics.
+template <class T, class DT, class PT> CD void contact_adjoint_finish(Sys<T, PT> s, CView<T> cv, T dt, ContactParams<T> cp) {
+  const int nl = s.nl;
+  const Rows<T> rows = active_rows(s, cv);
+  const int nc = rows.nc, nlr = rows.nlr;
+  const int *link = rows.link, *llink = rows.llink;
+  const V3<T>* pc = rows.pc;
+  const T* lsg = rows.lsg;
   // 4. b = E_w^T (V*_v + V*_w x p) + (erp / dt) phi e_z on contacts, s v*_j + (erp / dt) phi on limits
   for (int l = 0; l < nl; ++l) cputv(cv, l, B_VS, zeroSV<T>());
   const T kphi = cp.erp / dt;
@@ -722,6 +817,13 @@ CD void contact_adjoint(Sys<T, PT> s, CView<T> cv, T dt, ContactParams<T> cp) {
       cadd3(cv, par, B_OW, ob);
     }
   }
+}
+
+template <class T, class DT, class PT>
+CD void contact_adjoint(Sys<T, PT> s, CView<T> cv, T dt, ContactParams<T> cp) {
+  contact_adjoint_solve<T, DT, PT>(s, cv, dt, cp);
+  contact_adjoint_columns<T, DT, PT>(s, cv, 0, 1);
+  contact_adjoint_finish<T, DT, PT>(s, cv, dt, cp);
 }
 
 }  // namespace abasim

@@ -38,7 +38,7 @@ struct sim_handle {
   int* status = nullptr;     // [B] by system
   int* sys_of_slot = nullptr;  // [B]
   unsigned* counter = nullptr;  // work-unit ticket of persistent launches
-  void* ctape = nullptr;     // [maxL][NCT][B] scalar, models with contact spheres only
+  void* ctape = nullptr;     // [CT_WARPS][maxL][NCT][B] scalar, models with contact spheres or limits only
   void* csys = nullptr;      // [NCS][B] scalar, models with contact spheres only
   double friction = 0.8, erp = 0.2;
   int pgs_iterations = 20;

@@ -7,11 +7,11 @@ namespace host {
 
 template <class T, class DT>
 RolloutKernel<T> rollout_contact_kernel() {
-  return k_rollout<T, DT, ST_GLOBAL, true>;
+  return k_rollout_contact<T, DT>;
 }
 template <class T, class DT>
 BackwardKernel<T> backward_contact_kernel() {
-  return k_backward<T, DT, ST_GLOBAL, true>;
+  return k_backward_contact<T, DT>;
 }
 template RolloutKernel<float> rollout_contact_kernel<float, FF>();
 template BackwardKernel<float> backward_contact_kernel<float, FF>();

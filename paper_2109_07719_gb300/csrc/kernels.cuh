@@ -34,7 +34,7 @@ template <class T> struct DevModel {
   int persistent;
   int smem;
   int quadratic;
-  T* ctape;  // per-link contact tape [tile][maxL][NCT][lane] (null: no contact spheres or limits)
+  T* ctape;  // per-link contact tapes [CT_WARPS][tile][maxL][NCT][lane] (null: no contact spheres or limits)
   T* csys;   // per-system contact record [tile][NCS][lane]
   ContactParams<T> cp;
   double dt64;   // the time step in FP64
@@ -148,25 +148,11 @@ __device__ __forceinline__ Sys<T> sys_of(const DevModel<T>& m, int slot) {
 
 template <class T> __device__ __forceinline__ bool finite_t(T x) { return isfinite(x); }
 
-template <class T> __device__ __forceinline__ CView<T> cview_of(const DevModel<T>& m, int slot) {
-  const long long tile = slot / LANES, lane = slot % LANES;
-  return CView<T>{m.ctape + tile * m.maxL * NCT * LANES + lane, m.csys + tile * NCS * LANES + lane};
-}
-
-// One step x -> x' in place: ABA, the contact and joint-limit impulses (CT: the
-// model has contact spheres or joint limits), integration.
-template <class T, class DT, bool CT>
-__device__ __forceinline__ void forward_step(const DevModel<T>& m, const Sys<T>& s, int slot, Col<T> q,
-                                             Col<T> qd, Col<const T> tau_t, V3<T> g,
-                                             Col<double> xw = Col<double>{nullptr, 0}) {
-  aba_forward<T, DT, false>(s, Col<const T>{q.p, q.B}, Col<const T>{qd.p, qd.B}, tau_t, g);
-  const T* ct = nullptr;
-  if constexpr (CT) {
-    const CView<T> cv = cview_of(m, slot);
-    const int nc =
-        contact_forward<T, DT, T>(s, cv, Col<const T>{q.p, q.B}, Col<const T>{qd.p, qd.B}, m.dt, m.cp);
-    if (nc > 0) ct = cv.ct;
-  }
+// Integrates the step whose accelerations are on the tape (ct: plus the constraint velocity
+// change of that contact tape).
+template <class T, class DT>
+__device__ __forceinline__ void integrate_step(const DevModel<T>& m, const Sys<T>& s, Col<T> q, Col<T> qd, const T* ct,
+                                               Col<double> xw) {
   if constexpr (!std::is_same<T, DT>::value) {
     if (xw.p) {  // the running state in FP64 (xw); the dynamics read its FP32 rounding
       const Col<double> xq = xw, xqd{xw.p + (long long)m.nq_max * xw.B, xw.B};
@@ -179,31 +165,20 @@ __device__ __forceinline__ void forward_step(const DevModel<T>& m, const Sys<T>&
   integrate<T>(s, q, qd, m.dt, m.integ, ct);
 }
 
-// Recomputes the step from x^t and pulls the state adjoint (gq, gqd) back
-// through it.  With active contact or limit rows the integrator adjoint runs
-// first for every link (the constraint adjoint needs all of qdd's adjoint), then
-// the constraint adjoint, then the ABA adjoint with its terms added.
-template <class T, class DT, bool CT>
-__device__ __forceinline__ void adjoint_step(const DevModel<T>& m, const Sys<T>& s, int slot, Col<const T> q,
-                                             Col<const T> qd, Col<const T> tau_t, Col<T> gq, Col<T> gqd,
-                                             Col<T> gt, Col<T> gm, V3<T> g) {
+// One step x -> x' in place.
+template <class T, class DT>
+__device__ __forceinline__ void forward_step(const DevModel<T>& m, const Sys<T>& s, Col<T> q, Col<T> qd,
+                                             Col<const T> tau_t, V3<T> g, Col<double> xw = Col<double>{nullptr, 0}) {
+  aba_forward<T, DT, false>(s, Col<const T>{q.p, q.B}, Col<const T>{qd.p, qd.B}, tau_t, g);
+  integrate_step<T, DT>(m, s, q, qd, (const T*)nullptr, xw);
+}
+
+// Recomputes the step from x^t and pulls the state adjoint (gq, gqd) back through it.
+template <class T, class DT>
+__device__ __forceinline__ void adjoint_step(const DevModel<T>& m, const Sys<T>& s, Col<const T> q, Col<const T> qd,
+                                             Col<const T> tau_t, Col<T> gq, Col<T> gqd, Col<T> gt, Col<T> gm,
+                                             V3<T> g) {
   aba_forward<T, DT, true>(s, q, qd, tau_t, g);
-  if constexpr (CT) {
-    const CView<T> cv = cview_of(m, slot);
-    const int nc = contact_forward<T, DT, T>(s, cv, q, qd, m.dt, m.cp);
-    if (nc > 0) {
-      for (int l = 0; l < s.nl; ++l) {
-        const int mt = s.M(l);
-        T qb[6] = {0, 0, 0, 0, 0, 0};
-        integrator_adjoint(s, l, meta_jtype(mt), meta_qoff(mt), meta_voff(mt), q, qd, gq, gqd, m.dt, m.integ,
-                           qb, (const T*)cv.ct);
-        for (int i = 0; i < 6; ++i) cv.L(l, C_QDDB + i) = qb[i];
-      }
-      contact_adjoint<T, DT, T>(s, cv, m.dt, m.cp);
-      step_adjoint<T, DT>(s, q, qd, gq, gqd, gt, gm, g, m.dt, m.integ, (const T*)cv.ct);
-      return;
-    }
-  }
   step_adjoint<T, DT>(s, q, qd, gq, gqd, gt, gm, g, m.dt, m.integ);
 }
 
@@ -214,7 +189,7 @@ __device__ __forceinline__ void adjoint_step(const DevModel<T>& m, const Sys<T>&
 
 // T steps of one system.  The working state lives in (qT, qdT); checkpoints every
 // k steps; optional full trajectory.
-template <class T, class DT, int ST, bool CT>
+template <class T, class DT, int ST>
 __device__ __forceinline__ void rollout_one(const DevModel<T>& m, int slot, const T* __restrict__ q0,
                                             const T* __restrict__ qd0, const T* __restrict__ tau,
                                             long long Tn, int k, T* ckpt, T* qT, T* qdT, T* traj) {
@@ -265,7 +240,7 @@ __device__ __forceinline__ void rollout_one(const DevModel<T>& m, int slot, cons
       cp_wait_all_but_newest();
       tau_t = Col<const T>{sbuf + (t & 1) * nvm * LANES, LANES};
     }
-    forward_step<T, DT, CT>(m, s, slot, q, qd, tau_t, g, xw);
+    forward_step<T, DT>(m, s, q, qd, tau_t, g, xw);
     if (traj) {
       T* c = traj + (t + 1) * NX * B + b;
       for (int d = 0; d < nqm; ++d) c[d * B] = q[d];
@@ -285,7 +260,7 @@ __device__ __forceinline__ void rollout_one(const DevModel<T>& m, int slot, cons
 
 // Adjoint rollout of one system.  (gq0, gqd0) carry the running state adjoint
 // R^t = xbar^t.
-template <class T, class DT, int ST, bool CT>
+template <class T, class DT, int ST>
 __device__ __forceinline__ void backward_one(const DevModel<T>& m, int slot, const T* __restrict__ ckpt,
                                              const T* __restrict__ tau, long long Tn, int k,
                                              const T* __restrict__ gqT, const T* __restrict__ gqdT,
@@ -338,7 +313,7 @@ __device__ __forceinline__ void backward_one(const DevModel<T>& m, int slot, con
       const T* xb = sbuf + (t & 1) * W * LANES;
       Col<const T> q{xb, LANES}, qd{xb + nqm * LANES, LANES};
       T* gt = gtau + t * nvm * B + b;
-      adjoint_step<T, DT, CT>(m, s, slot, q, qd, Col<const T>{xb + NX * LANES, LANES}, gq, gqd, Col<T>{gt, B}, gm, g);
+      adjoint_step<T, DT>(m, s, q, qd, Col<const T>{xb + NX * LANES, LANES}, gq, gqd, Col<T>{gt, B}, gm, g);
       for (int d = nv; d < nvm; ++d) gt[d * B] = T(0);
       if (gtraj) {
         const T* gx = gtraj + t * NX * B + b;
@@ -359,7 +334,7 @@ __device__ __forceinline__ void backward_one(const DevModel<T>& m, int slot, con
           const T* prev = ring + (j - 1) * NX * B + slot;
           T* cur = ring + j * NX * B + slot;
           for (int d = 0; d < NX; ++d) cur[d * B] = prev[d * B];
-          forward_step<T, DT, CT>(m, s, slot, Col<T>{cur, B}, Col<T>{cur + nqm * B, B},
+          forward_step<T, DT>(m, s, Col<T>{cur, B}, Col<T>{cur + nqm * B, B},
                               Col<const T>{tau + (t0 + j - 1) * nvm * B + b, B}, g);
         }
       }
@@ -370,13 +345,13 @@ __device__ __forceinline__ void backward_one(const DevModel<T>& m, int slot, con
           x = cur;
           for (int d = 0; d < NX; ++d) cur[d * B] = xs[d * B];
           for (long long j = t0; j < t; ++j) {
-            forward_step<T, DT, CT>(m, s, slot, Col<T>{cur, B}, Col<T>{cur + nqm * B, B},
+            forward_step<T, DT>(m, s, Col<T>{cur, B}, Col<T>{cur + nqm * B, B},
                                 Col<const T>{tau + j * nvm * B + b, B}, g);
           }
         }
         Col<const T> q{x, B}, qd{x + nqm * B, B};
         T* gt = gtau + t * nvm * B + b;
-        adjoint_step<T, DT, CT>(m, s, slot, q, qd, Col<const T>{tau + t * nvm * B + b, B}, gq, gqd, Col<T>{gt, B},
+        adjoint_step<T, DT>(m, s, q, qd, Col<const T>{tau + t * nvm * B + b, B}, gq, gqd, Col<T>{gt, B},
                             gm, g);
         for (int d = nv; d < nvm; ++d) gt[d * B] = T(0);
         if (gtraj) {
@@ -421,27 +396,26 @@ __device__ __forceinline__ int next_unit(unsigned* counter) {
     unit = next_unit((m).counter);                                           \
   }
 
-// CT: the model has contact spheres or joint limits (a separate instantiation, so
-// the kernels of unconstrained models carry none of the constraint code).
-template <class T, class DT, int ST, bool CT = false>
+template <class T, class DT, int ST>
 __global__ void k_rollout(DevModel<T> m, const T* __restrict__ q0, const T* __restrict__ qd0,
                           const T* __restrict__ tau, long long Tn, int k, T* ckpt, T* qT, T* qdT,
                           T* traj) {
-  ABASIM_FOR_EACH_SLOT(m, rollout_one<T, DT, ST, CT>(m, slot, q0, qd0, tau, Tn, k, ckpt, qT, qdT, traj))
+  ABASIM_FOR_EACH_SLOT(m, rollout_one<T, DT, ST>(m, slot, q0, qd0, tau, Tn, k, ckpt, qT, qdT, traj))
 }
 
-template <class T, class DT, int ST, bool CT = false>
+template <class T, class DT, int ST>
 __global__ void k_backward(DevModel<T> m, const T* __restrict__ ckpt, const T* __restrict__ tau,
                            long long Tn, int k, const T* __restrict__ gqT, const T* __restrict__ gqdT,
                            const T* __restrict__ gtraj, T* gq0, T* gqd0, T* gtau, T* gm_acc,
                            T* ring) {
-  ABASIM_FOR_EACH_SLOT(m, backward_one<T, DT, ST, CT>(m, slot, ckpt, tau, Tn, k, gqT, gqdT, gtraj, gq0, gqd0,
+  ABASIM_FOR_EACH_SLOT(m, backward_one<T, DT, ST>(m, slot, ckpt, tau, Tn, k, gqT, gqdT, gtraj, gq0, gqd0,
                                               gtau, gm_acc, ring))
 }
 
 }  // namespace host
 }  // namespace abasim
 
+#include "ckernels.cuh"
 #include "wkernels.cuh"
 
 namespace abasim {
@@ -1145,6 +1119,7 @@ int launch_rollout(sim_handle* h, const void* q0, const void* qd0, const void* t
   int threads = h->block;
   if (h->ctape) {
     kern = rollout_contact_kernel<T, DT>();
+    threads = CT_WARPS * LANES;
   } else {
     bool piped = false;  // the pipelined rollout, any precision
     if (h->all_chains && h->maxL <= PIPE_MAX_LINKS && !h->state64 &&
@@ -1179,7 +1154,7 @@ int launch_rollout(sim_handle* h, const void* q0, const void* qd0, const void* t
   if (rc != SIM_OK) return rc;
   h->last_storage = st;
   int grid = 0;
-  rc = launch_shape(h, kern, &grid, &m.persistent, shm, stream, threads, st == ST_PIPE ? LANES : threads);
+  rc = launch_shape(h, kern, &grid, &m.persistent, shm, stream, threads, st == ST_PIPE || h->ctape ? LANES : threads);
   if (rc != SIM_OK) return rc;
   kern<<<grid, threads, shm, S(stream)>>>(m, (const T*)q0, (const T*)qd0, (const T*)tau, (long long)T_,
                                            k, (T*)ckpt, (T*)qT, (T*)qdT, (T*)traj);
@@ -1204,6 +1179,7 @@ int launch_backward(sim_handle* h, const void* ckpt, const void* tau, int64_t T_
   int threads = h->block;
   if (h->ctape) {
     kern = backward_contact_kernel<T, DT>();
+    threads = CT_WARPS * LANES;
   } else if constexpr (sizeof(T) == 4) {  // on-chip modes: FP32 storage only
     bool piped = false;
     if (k == 1 && T_ > 0 && h->all_chains &&
@@ -1238,7 +1214,7 @@ int launch_backward(sim_handle* h, const void* ckpt, const void* tau, int64_t T_
   if (rc != SIM_OK) return rc;
   h->last_storage_bwd = st;
   int grid = 0;
-  rc = launch_shape(h, kern, &grid, &m.persistent, shm, stream, threads, st == ST_PIPE ? LANES : threads);
+  rc = launch_shape(h, kern, &grid, &m.persistent, shm, stream, threads, st == ST_PIPE || h->ctape ? LANES : threads);
   if (rc != SIM_OK) return rc;
   kern<<<grid, threads, shm, S(stream)>>>(m, (const T*)ckpt, (const T*)tau, (long long)T_, k,
                                            (const T*)gqT, (const T*)gqdT, (const T*)gtraj, (T*)gq0,
@@ -1261,9 +1237,10 @@ int launch_step_with_tape(sim_handle* h, const void* q, const void* qd, const vo
                           void* qd_out, void* tape, void* stream) {
   DevModel<T> m = dev_model<T>(h);
   m.tape = (T*)tape;
-  const int grid = (h->B + h->block - 1) / h->block;
+  const int slots = h->ctape ? LANES : h->block, threads = h->ctape ? CT_WARPS * LANES : h->block;
+  const int grid = (h->B + slots - 1) / slots;
   const RolloutKernel<T> kern = h->ctape ? rollout_contact_kernel<T, DT>() : k_rollout<T, DT, ST_GLOBAL>;
-  kern<<<grid, h->block, 0, S(stream)>>>(m, (const T*)q, (const T*)qd, (const T*)tau, 1LL, 1, (T*)nullptr,
+  kern<<<grid, threads, 0, S(stream)>>>(m, (const T*)q, (const T*)qd, (const T*)tau, 1LL, 1, (T*)nullptr,
                                          (T*)q_out, (T*)qd_out, (T*)nullptr);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? SIM_OK : cuda_fail(h, e, "step launch");

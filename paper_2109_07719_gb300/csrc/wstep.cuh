@@ -148,7 +148,7 @@ template <int NEWER> __device__ __forceinline__ void stage_wait() {  // all but 
 // t (fields of the first range), t2 (the second), p and a, indexed by field, at this lane.
 // All lanes of the warp call it together when staging.
 template <class T, bool STG, int DIR, int RING, int TF, int TN, int PF, int PN, int AF = 0, int AN = 0, int SF = 0,
-          int SN = 0>
+          int SN = 0, int ASTRIDE = NWA>
 struct Records {
   static constexpr int ROWS = TN + SN + PN + AN, SLOTS = 3 * RING / ROWS, AHEAD = SLOTS - 2;
   static_assert(ROWS <= RING, "ring rows");
@@ -161,7 +161,7 @@ struct Records {
     const int first = DIR > 0 ? 0 : n - 1;
     st = s.tape + first * NWT * LANES;
     sp = s.prm + first * s.pstride * LANES;
-    sa = AN ? s.adj + first * NWA * LANES : nullptr;
+    sa = AN ? s.adj + first * ASTRIDE * LANES : nullptr;
     if constexpr (STG) {
 #ifdef __CUDA_ARCH__
       constexpr int PER = 16 / sizeof(T);
@@ -176,7 +176,7 @@ struct Records {
     } else {
       st -= DIR * NWT * LANES;
       sp -= DIR * s.pstride * LANES;
-      if (AN) sa -= DIR * NWA * LANES;
+      if (AN) sa -= DIR * ASTRIDE * LANES;
     }
   }
   SD void fetch() {
@@ -189,7 +189,7 @@ struct Records {
       if (AN) copy<AN * CH>(fill + (TN + SN + PN) * LANES, sa);
       st += DIR * NWT * LANES;
       sp += DIR * s.pstride * LANES;
-      if (AN) sa += DIR * NWA * LANES;
+      if (AN) sa += DIR * ASTRIDE * LANES;
       --left;
     }
     stage_commit();
@@ -225,7 +225,7 @@ struct Records {
     } else {
       t = t2 = st += DIR * NWT * LANES;
       p = sp += DIR * s.pstride * LANES;
-      if (AN) a = sa += DIR * NWA * LANES;
+      if (AN) a = sa += DIR * ASTRIDE * LANES;
     }
   }
 };
