@@ -10,6 +10,7 @@
 #include "contact.cuh"
 #include "dual.cuh"
 #include "handle.h"
+#include "wjvp.cuh"
 #include "wstep.cuh"
 
 namespace abasim {
@@ -721,6 +722,7 @@ k_rollout_pipe(DevModel<T> m, const T* __restrict__ q0, const T* __restrict__ qd
 }  // namespace abasim
 
 #include "wpipe.cuh"
+#include "wjvp_kernel.cuh"
 
 namespace abasim {
 namespace host {
@@ -1250,11 +1252,35 @@ template <class T>
 int launch_jvp(sim_handle* h, const void* q, const void* qd, const void* tau, const void* dq,
                const void* dqd, const void* dtau, void* q_out, void* qd_out, void* dq_out,
                void* dqd_out, void* work, void* stream) {
+  if constexpr (sizeof(T) == 8) {
+    // FP64: the implicit form on the world-aligned path, unless its inputs and ring exceed a
+    // block's shared memory or the caller's workspace is not aligned for its 16-byte copies.
+    // In FP32 its right-hand side loses digits in long trees (error against 64 bits 6.5e-7 for
+    // 64 links, 3.5e-8 on dual numbers), so the step on dual numbers stays there.
+    int limit = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
+    if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory limit query");
+    DevModel<T> m = dev_model<T>(h);
+    m.sd = h->wdepth * WSW;
+    auto need = [&] { return (size_t)wjvp_smem_per_tile(h->nq_max, h->nv_max, m.sd) * LANES * sizeof(T); };
+    if (!stacks_fit(h, LANES, need(), limit)) m.sd = 0;
+    const size_t shm = need();
+    if (shm <= (size_t)limit && (uintptr_t)work % 16 == 0) {
+      const auto kern = h->all_revolute ? k_wstep_jvp<T, false> : k_wstep_jvp<T, true>;
+      e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+      if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory opt-in");
+      kern<<<(h->B + LANES - 1) / LANES, LANES, shm, S(stream)>>>(
+          m, (const T*)q, (const T*)qd, (const T*)tau, (const T*)dq, (const T*)dqd, (const T*)dtau, (T*)q_out, (T*)qd_out,
+          (T*)dq_out, (T*)dqd_out, (T*)work);
+      e = cudaGetLastError();
+      return e == cudaSuccess ? SIM_OK : cuda_fail(h, e, "jvp launch");
+    }
+  }
   const int grid = (h->B + h->block - 1) / h->block;
   k_step_jvp<T, T><<<grid, h->block, 0, S(stream)>>>(
       dev_model<T>(h), (const T*)q, (const T*)qd, (const T*)tau, (const T*)dq, (const T*)dqd,
       (const T*)dtau, (T*)q_out, (T*)qd_out, (T*)dq_out, (T*)dqd_out, (Dual<T>*)work);
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? SIM_OK : cuda_fail(h, e, "jvp launch");
 }
 
