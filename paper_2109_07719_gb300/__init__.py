@@ -92,11 +92,17 @@ lib = _load()
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+# the current stream's handle without a Stream object, where torch offers it
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    if _raw_stream is not None:
+        return _raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 class Simulator:
@@ -163,9 +169,9 @@ class Simulator:
     def _arg(self, t, shape, name):
         if t is None:
             return None
-        if t.device != self.device or t.dtype != self.dtype or not t.is_contiguous():
+        if t.dtype != self.dtype or t.device != self.device or not t.is_contiguous():
             raise SimError(f"{name}: need a contiguous {self.dtype} tensor on {self.device}")
-        if tuple(t.shape) != tuple(shape):
+        if t.shape != shape:     # torch.Size is a tuple
             raise SimError(f"{name}: shape {tuple(t.shape)} != {tuple(shape)}")
         return t
 
@@ -258,10 +264,11 @@ class Simulator:
         self._arg(q, (self.nq_max, B), "q")
         self._arg(qd, (self.nv_max, B), "qd")
         self._arg(tau, (self.nv_max, B), "tau")
-        q_out = self.empty(self.nq_max, B) if q_out is None else q_out
-        qd_out = self.empty(self.nv_max, B) if qd_out is None else qd_out
-        self._check(lib.sim_step_batch(self._h, _ptr(q), _ptr(qd), _ptr(tau), _ptr(q_out),
-                                       _ptr(qd_out), _stream()), "sim_step_batch")
+        q_out = torch.empty_like(q) if q_out is None else q_out
+        qd_out = torch.empty_like(qd) if qd_out is None else qd_out
+        rc = lib.sim_step_batch(self._h, _ptr(q), _ptr(qd), _ptr(tau), _ptr(q_out), _ptr(qd_out), _stream())
+        if rc != SIM_OK:
+            self._check(rc, "sim_step_batch")
         return q_out, qd_out
 
     def step_static(self, q, qd, tau, q_out=None, qd_out=None):

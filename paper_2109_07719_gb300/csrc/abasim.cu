@@ -374,6 +374,7 @@ int sim_create(const sim_model_desc* d, sim_handle** out) {
     h->nv_max = std::max(h->nv_max, vo);
   }
   cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
+  cudaDeviceGetAttribute(&h->smem_limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
   h->all_chains = !any_contact;
   h->unconstrained = !any_contact;
   h->all_revolute = !any_contact;

@@ -48,6 +48,7 @@ struct sim_handle {
   int prefetch = 2;          // links ahead the world-aligned global-tape passes prefetch
   int last_storage = 0, last_storage_bwd = 0;
   int sms = 0;
+  int smem_limit = 0;        // shared memory a block may opt in to, bytes
   bool all_chains = false;   // every system a serial chain of revolute joints (the pipelined adjoint)
   bool all_revolute = false; // every joint revolute and no contact spheres or limits
   bool unconstrained = false; // no contact spheres or limits (the world-aligned kernels; FR ones unless all_revolute)

@@ -849,9 +849,8 @@ int choose_storage(sim_handle* h, K0 k_global, K1 k_hybrid, K2 k_smem, bool bwd,
   *st = ST_GLOBAL;
   *bytes = 0;
   if (h->tape_space == SIM_TAPE_GLOBAL || sizeof(T) != 4) return SIM_OK;
-  int limit = 0;
-  cudaError_t e = cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
-  if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory limit query");
+  const int limit = h->smem_limit;
+  cudaError_t e = cudaSuccess;
   int per_sm_g = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_g, k_global, h->block, 0);
   if (e != cudaSuccess) return cuda_fail(h, e, "occupancy query");
@@ -919,9 +918,8 @@ inline long long w_state_per_tile(const sim_handle* h, bool bwd) {
 template <class T, class K>
 int choose_w(sim_handle* h, K k_on, K k_off, bool bwd, bool* onchip, int* threads, int* slots, int* sd,
              size_t* bytes) {
-  int limit = 0;
-  cudaError_t e = cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
-  if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory limit query");
+  const int limit = h->smem_limit;
+  cudaError_t e = cudaSuccess;
   const int nx = h->nq_max + h->nv_max;
   const bool fr = !h->all_revolute;
   auto need = [&](bool on, int tiles) {
@@ -981,8 +979,7 @@ bool use_aligned(const sim_handle* h, bool rollout) {
   if (h->tape_space != SIM_TAPE_AUTO && h->tape_space != SIM_TAPE_ALIGNED &&
       h->tape_space != SIM_TAPE_ALIGNED_PIPELINED)
     return false;
-  int limit = 0;
-  if (cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device) != cudaSuccess) return false;
+  const int limit = h->smem_limit;
   const size_t streams = (size_t)(h->block / LANES) * w_state_per_tile(h, !rollout) * LANES * sizeof(T);
   if (streams > (size_t)limit) return false;
   if (h->tape_space != SIM_TAPE_AUTO || !h->all_chains || !rollout) return true;
@@ -1019,9 +1016,8 @@ int launch_wbackward_pipe(sim_handle* h, const void* ckpt, const void* tau, int6
                           const void* gqdT, const void* gtraj, void* gq0, void* gqd0, void* gtau, void* gmass,
                           void* work, void* stream) {
   DevModel<T> m = dev_model<T>(h);
-  int limit = 0;
-  cudaError_t e = cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
-  if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory limit query");
+  const int limit = h->smem_limit;
+  cudaError_t e = cudaSuccess;
   const int nx = h->nq_max + h->nv_max;
   const bool fr = !h->all_revolute;
   const int tiles = (h->B + LANES - 1) / LANES, sms = std::max(1, h->sms);
@@ -1128,9 +1124,8 @@ int launch_rollout(sim_handle* h, const void* q0, const void* qd0, const void* t
         (h->tape_space == SIM_TAPE_AUTO || h->tape_space == SIM_TAPE_PIPELINED)) {
       const size_t need =
           (size_t)pipe_fwd_smem_per_tile(h->maxL, h->nq_max + h->nv_max, h->nv_max) * LANES * sizeof(T);
-      int limit = 0;
-      cudaError_t e = cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
-      if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory limit query");
+      const int limit = h->smem_limit;
+      cudaError_t e = cudaSuccess;
       if (need <= (size_t)limit) {
         kern = k_rollout_pipe<T, DT>;
         e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
@@ -1187,9 +1182,8 @@ int launch_backward(sim_handle* h, const void* ckpt, const void* tau, int64_t T_
     if (k == 1 && T_ > 0 && h->all_chains &&
         (h->tape_space == SIM_TAPE_AUTO || h->tape_space == SIM_TAPE_PIPELINED)) {
       // the pipelined two-warp adjoint, when its shared memory fits one block
-      int limit = 0;
-      cudaError_t e = cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
-      if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory limit query");
+      const int limit = h->smem_limit;
+      cudaError_t e = cudaSuccess;
       const size_t need =
           (size_t)pipe_smem_per_tile(h->maxL, h->nq_max + h->nv_max, h->nv_max) * LANES * sizeof(T);
       if (need <= (size_t)limit) {
@@ -1257,9 +1251,8 @@ int launch_jvp(sim_handle* h, const void* q, const void* qd, const void* tau, co
     // block's shared memory or the caller's workspace is not aligned for its 16-byte copies.
     // In FP32 its right-hand side loses digits in long trees (error against 64 bits 6.5e-7 for
     // 64 links, 3.5e-8 on dual numbers), so the step on dual numbers stays there.
-    int limit = 0;
-    cudaError_t e = cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
-    if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory limit query");
+    const int limit = h->smem_limit;
+    cudaError_t e = cudaSuccess;
     DevModel<T> m = dev_model<T>(h);
     m.sd = h->wdepth * WSW;
     auto need = [&] { return (size_t)wjvp_smem_per_tile(h->nq_max, h->nv_max, m.sd) * LANES * sizeof(T); };
