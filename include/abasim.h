@@ -261,8 +261,8 @@ int sim_set_launch(sim_handle* h, int32_t threads, int32_t schedule);
  * the velocity, bias-force and acceleration passes; in the adjoint (FP32 storage,
  * checkpoint interval 1) one warp recomputes step t's forward intermediates into
  * one of two shared-memory tapes while the other differentiates step t + 1 from
- * the other tape (when the two tapes fit, about 7 links).  AUTO picks each when it
- * applies; forcing it fails with SIM_EUNSUPPORTED where it does not.
+ * the other tape (when the two tapes fit, about 7 links).  AUTO picks the rollout
+ * when it applies (FP64 chains of three links or more on a four-warp form of it); forcing it fails with SIM_EUNSUPPORTED where it does not.
  * SIM_TAPE_ONE_WARP chooses like AUTO among the one-warp-per-tile kernels only
  * (the autotuner times both, as one or two lanes per system).  Models with contact spheres or joint limits always run with the tape
  * in global memory.  Results do not depend on the choice beyond rounding. */

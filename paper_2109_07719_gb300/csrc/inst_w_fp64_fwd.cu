@@ -12,5 +12,8 @@ RolloutKernel<T> wrollout_kernel(bool onchip, bool fr) {
 }
 template RolloutKernel<double> wrollout_kernel<double, double>(bool, bool);
 
+template <class T> RolloutKernel<T> wrollout_team_kernel() { return k_wrollout_team<T>; }
+template RolloutKernel<double> wrollout_team_kernel<double>();
+
 }  // namespace host
 }  // namespace abasim

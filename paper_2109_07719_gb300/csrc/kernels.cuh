@@ -723,6 +723,7 @@ k_rollout_pipe(DevModel<T> m, const T* __restrict__ q0, const T* __restrict__ qd
 
 #include "wpipe.cuh"
 #include "wjvp_kernel.cuh"
+#include "wteam.cuh"
 
 namespace abasim {
 namespace host {
@@ -747,6 +748,7 @@ template <class T, class DT>
 BackwardKernel<T> backward_pipe_kernel();
 // The world-aligned kernels (tape on chip or in global memory), instantiated in
 // their own units.
+template <class T> RolloutKernel<T> wrollout_team_kernel();
 template <class T, class DT>
 RolloutKernel<T> wrollout_kernel(bool onchip, bool fr);
 template <class T, class DT>
@@ -1128,12 +1130,25 @@ int launch_rollout(sim_handle* h, const void* q0, const void* qd0, const void* t
       cudaError_t e = cudaSuccess;
       if (need <= (size_t)limit) {
         kern = k_rollout_pipe<T, DT>;
-        e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-        if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory opt-in");
         st = ST_PIPE;
         shm = need;
         threads = 2 * LANES;
         piped = true;
+      }
+      if constexpr (sizeof(T) == 8) {  // FP64: the team rollout (wteam.cuh) where a tile fits a block
+        const size_t team =
+            (size_t)team_smem_per_tile(h->maxL, h->nq_max + h->nv_max, h->nv_max) * LANES * sizeof(T);
+        if (h->tape_space == SIM_TAPE_AUTO && h->maxL >= TEAM_MIN_LINKS && team <= (size_t)limit) {
+          kern = wrollout_team_kernel<T>();
+          st = ST_PIPE;
+          shm = team;
+          threads = TEAM * LANES;
+          piped = true;
+        }
+      }
+      if (piped) {
+        e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+        if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory opt-in");
       }
     }
     if (!piped && h->tape_space == SIM_TAPE_PIPELINED)
