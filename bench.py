@@ -42,7 +42,7 @@ def _flop_table():
 def flops_per_system_step(model, kind):
     """kind: 'fwd' / 'adj' (link-frame step: forward, adjoint without its recompute)
     or 'wfwd' / 'wrec' / 'wadj' (world-aligned step: the rollout's step, the
-    adjoint's recompute, the adjoint step; revolute joints only)."""
+    adjoint's recompute, the adjoint step)."""
     import numpy as np
     tab = _flop_table()[kind]
     jt = np.asarray(model.joint_type)
@@ -50,21 +50,21 @@ def flops_per_system_step(model, kind):
     n_free = int((jt == 1).sum())
     n_rev_root = int(((jt == 0) & (par < 0)).sum())
     n_rev = int(((jt == 0) & (par >= 0)).sum())
-    if n_free and "free_root" not in tab:
-        raise ValueError(f"{kind}: no FLOP count for free joints")
-    return (tab["rev"] * n_rev + tab["rev_root"] * n_rev_root + tab.get("free_root", 0) * n_free) / model.n_systems
+    return (tab["rev"] * n_rev + tab["rev_root"] * n_rev_root + tab["free_root"] * n_free) / model.n_systems
 
 
-def kernel_flops(model, storage):
+def kernel_flops(model, storage, precision="fp32"):
     """(rollout kernel, its FLOPs per system-step, adjoint kernel, its FLOPs per
     system-step) for the storage modes the last launches reported."""
-    fwd_aligned = storage[0].startswith("aligned")
-    bwd_aligned = storage[1].startswith("aligned")
-    kf = "k_wrollout" if fwd_aligned else ("k_rollout_pipe" if storage[0] == "pipelined" else "k_rollout")
-    kb = ("k_wbackward_pipe" if storage[1].startswith("aligned_pipelined") else "k_wbackward") if bwd_aligned else \
+    world = ("aligned", "floating")              # the world-aligned kernels
+    fwd_world, bwd_world = storage[0].startswith(world), storage[1].startswith(world)
+    kf = "k_wrollout" if fwd_world else ("k_rollout_pipe" if storage[0] == "pipelined" else "k_rollout")
+    if storage[0] == "pipelined" and precision == "fp64" and int(model.nv_max) >= 3:
+        kf, fwd_world = "k_wrollout_team", True  # the same step, shared by four warps
+    kb = ("k_wbackward_pipe" if "_pipelined" in storage[1] else "k_wbackward") if bwd_world else \
         ("k_backward_pipe" if storage[1] == "pipelined" else "k_backward")
-    ff = flops_per_system_step(model, "wfwd" if fwd_aligned else "fwd")
-    fb = (flops_per_system_step(model, "wrec") + flops_per_system_step(model, "wadj")) if bwd_aligned else \
+    ff = flops_per_system_step(model, "wfwd" if fwd_world else "fwd")
+    fb = (flops_per_system_step(model, "wrec") + flops_per_system_step(model, "wadj")) if bwd_world else \
         (flops_per_system_step(model, "fwd") + flops_per_system_step(model, "adj"))
     return kf, ff, kb, fb
 
@@ -293,7 +293,7 @@ def run_ours(args):
                       qd0.cpu().pin_memory())
     if rank != 0:
         return None
-    kf, f_fwd, kb, f_bwd = kernel_flops(m, storage)
+    kf, f_fwd, kb, f_bwd = kernel_flops(m, storage, args.precision)
     adj_flops = B * T * f_bwd
     adj_s = float(np.mean(adj_ms)) / 1e3
     clocks = _clocks_summary(samples)

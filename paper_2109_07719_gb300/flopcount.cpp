@@ -77,47 +77,52 @@ static Counts count(int n, bool free_root) {
 
 struct WCounts { long long fwd, rec, adj; };
 
-// the world-aligned step of a revolute chain of n links
-static WCounts wcount(int n) {
+// the world-aligned step of a chain of n links, link 0 free or revolute
+template <bool FR> static WCounts wcount(int n) {
   const int B = 1;
-  static F prm[8 * NPRM * LANES], tape[8 * NWT * LANES], adj[8 * NWA * LANES];
+  static F prm[8 * NPRM * LANES], tape[8 * NWT * LANES], adj[8 * NWA * LANES], root[NWF * LANES];
   static int meta[8 * LANES];
   F q[64], qd[64], tau[64], gq[64], gqd[64], gtau[64], gm[8], q2[64], qd2[64];
+  int qo = 0, vo = 0;
   for (int l = 0; l < n; ++l) {
     auto P = [&](int f) -> F& { return prm[(l * NPRM + f) * LANES]; };
     for (int f = 0; f < NPRM; ++f) P(f) = F(0.1 * (f + 1));
     for (int f = 0; f < 9; ++f) P(P_E + f) = F(f % 4 == 0 ? 1.0 : 0.0);
     P(P_M) = 1;
-    meta[l * LANES] = make_meta(l - 1, J_REVOLUTE, false, l, l);
+    const bool fr = FR && l == 0;
+    meta[l * LANES] = make_meta(l - 1, fr ? J_FREE : J_REVOLUTE, false, qo, vo);
+    qo += fr ? 7 : 1;
+    vo += fr ? 6 : 1;
   }
   for (int i = 0; i < 64; ++i) { q[i] = F(0.1 * i); qd[i] = F(0.2); tau[i] = F(0.3); gq[i] = F(1); gqd[i] = F(1); q2[i] = q[i]; qd2[i] = qd[i]; }
   for (int i = 0; i < 8; ++i) gm[i] = F(0);
+  if (FR) { q[3] = 0; q[4] = 0; q[5] = 0; q[6] = 1; }
   WSys<F> s{prm, meta, tape, adj, n};
+  s.root = root;
   const V3<F> g{F(0), F(0), F(-9.81)};
   WCounts c;
   g_flops = 0;
-  wstep_forward<F, F, false, true>(s, Col<const F>{q, B}, Col<const F>{qd, B}, Col<const F>{tau, B}, g, F(1e-3),
+  wstep_forward<F, F, false, true, FR>(s, Col<const F>{q, B}, Col<const F>{qd, B}, Col<const F>{tau, B}, g, F(1e-3),
                                    I_SEMI_IMPLICIT, Col<F>{q2, B}, Col<F>{qd2, B});
   c.fwd = g_flops;
   g_flops = 0;
-  wstep_forward<F, F, true, false>(s, Col<const F>{q, B}, Col<const F>{qd, B}, Col<const F>{tau, B}, g, F(1e-3),
+  wstep_forward<F, F, true, false, FR>(s, Col<const F>{q, B}, Col<const F>{qd, B}, Col<const F>{tau, B}, g, F(1e-3),
                                    I_SEMI_IMPLICIT, Col<F>{q2, B}, Col<F>{qd2, B});
   c.rec = g_flops;
   g_flops = 0;
-  wstep_adjoint<F, F>(s, Col<F>{gq, B}, Col<F>{gqd, B}, Col<F>{gtau, B},
-                      Col<F>{gm, B}, F(1e-3), I_SEMI_IMPLICIT);
+  wstep_adjoint<F, F, FR>(s, Col<F>{gq, B}, Col<F>{gqd, B}, Col<F>{gtau, B}, Col<F>{gm, B}, F(1e-3), I_SEMI_IMPLICIT, g);
   c.adj = g_flops;
   return c;
 }
 
 int main() {
   Counts r1 = count(1, false), r2 = count(2, false), f1 = count(1, true);
-  WCounts w1 = wcount(1), w2 = wcount(2);
+  WCounts w1 = wcount<false>(1), w2 = wcount<false>(2), wf = wcount<true>(1);
   printf("{\n  \"convention\": \"+ - * / sqrt sin cos each count 1 FLOP (an FMA counts 2)\",\n");
   printf("  \"fwd\": {\"rev_root\": %lld, \"rev\": %lld, \"free_root\": %lld},\n", r1.fwd, r2.fwd - r1.fwd, f1.fwd);
   printf("  \"adj\": {\"rev_root\": %lld, \"rev\": %lld, \"free_root\": %lld},\n", r1.adj, r2.adj - r1.adj, f1.adj);
-  printf("  \"wfwd\": {\"rev_root\": %lld, \"rev\": %lld},\n", w1.fwd, w2.fwd - w1.fwd);
-  printf("  \"wrec\": {\"rev_root\": %lld, \"rev\": %lld},\n", w1.rec, w2.rec - w1.rec);
-  printf("  \"wadj\": {\"rev_root\": %lld, \"rev\": %lld}\n}\n", w1.adj, w2.adj - w1.adj);
+  printf("  \"wfwd\": {\"rev_root\": %lld, \"rev\": %lld, \"free_root\": %lld},\n", w1.fwd, w2.fwd - w1.fwd, wf.fwd);
+  printf("  \"wrec\": {\"rev_root\": %lld, \"rev\": %lld, \"free_root\": %lld},\n", w1.rec, w2.rec - w1.rec, wf.rec);
+  printf("  \"wadj\": {\"rev_root\": %lld, \"rev\": %lld, \"free_root\": %lld}\n}\n", w1.adj, w2.adj - w1.adj, wf.adj);
   return 0;
 }
