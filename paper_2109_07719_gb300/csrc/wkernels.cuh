@@ -29,7 +29,7 @@ __host__ __device__ __forceinline__ long long w_tape_words(int maxL, bool fr) {
 __host__ __device__ __forceinline__ long long w_smem_per_tile(int maxL, int nx, int nv, bool bwd, bool onchip,
                                                               int sd, bool fr, int slots) {
   const long long state = nx + (bwd ? maxL : 0);
-  if (!onchip) return state + sd + (long long)slots * (bwd ? RING_ADJ : RING_FWD);
+  if (!onchip) return state + sd + (long long)slots * (bwd ? RING_ADJ : RING_ROLL);
   return w_tape_words(maxL, fr) + (long long)maxL * ((bwd ? NWA : 0) + NPRM_W + 1) + sd + state +
          2LL * (nv + (bwd ? nx : 0));
 }
@@ -74,7 +74,7 @@ __device__ __forceinline__ WTile<T> w_tile(const DevModel<T>& m, int lane) {
     base += L * LANES;
   } else {
     t.ring = base - lane;
-    base += (long long)m.slots * (BWD ? RING_ADJ : RING_FWD) * LANES;
+    base += (long long)m.slots * (BWD ? RING_ADJ : RING_ROLL) * LANES;
   }
   t.stk = base;
   base += (long long)sd * LANES;
@@ -138,8 +138,13 @@ __device__ __forceinline__ void wrollout_one(const DevModel<T>& m, int slot, boo
     for (int d = 0; d < nqm; ++d) c[d * B + b] = q[d];
     for (int d = 0; d < nvm; ++d) c[(nqm + d) * B + b] = qd[d];
   };
-  if (traj) put(traj);
+  const Col<const T> cq{q.p, LANES}, cqd{qd.p, LANES};
   for (long long t = 0; t < Tn; ++t) {
+    if (t == 0)
+      wpass_pose<T, DT, false, FR>(s, cq, cqd);
+    else  // x^t from step t - 1's accelerations, and its pose
+      wpass_accel_pose<T, DT, FR>(s, q, qd, g, m.dt, m.integ);
+    if (traj) put(traj + t * NX * B);
     if (ckpt && t % k == 0) put(ckpt + (t / k) * NX * B);
     Col<const T> tau_t{tau + t * nvm * B + b, B};
     if (ONCHIP) {
@@ -153,10 +158,10 @@ __device__ __forceinline__ void wrollout_one(const DevModel<T>& m, int slot, boo
     } else if (t + 1 < Tn && m.slots > 1) {
       for (int d = 0; d < nv; ++d) pf_line(tau + ((t + 1) * nvm + d) * B + b);
     }
-    wstep_forward<T, DT, false, true, FR>(s, Col<const T>{q.p, LANES}, Col<const T>{qd.p, LANES}, tau_t, g, m.dt,
-                                          m.integ, q, qd);
-    if (traj) put(traj + (t + 1) * NX * B);
+    wpass_inward<T, DT, false, FR>(s, cqd, tau_t);
   }
+  if (Tn > 0) wpass_accel<T, DT, false, true, FR>(s, cq, cqd, g, m.dt, m.integ, q, qd);
+  if (traj) put(traj + Tn * NX * B);
   if (ONCHIP) cp_wait_all();
   if (!act) return;
   bool ok = true;

@@ -27,5 +27,5 @@ def test_free_root_matches_link_frame(rows, links):
     mine = [r for r in rows if r[0] == links]
     assert len(mine) == 2
     for r in mine:
-        assert max(r[1:6]) < 1e-11, r
-        assert r[6] == 1
+        assert max(r[1:7]) < 1e-11, r            # r[6]: the rollout's fused pass against whole steps
+        assert r[7] == 1

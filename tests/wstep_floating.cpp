@@ -4,7 +4,8 @@
 // formulations of the same step and gradient, so they agree to rounding.  The stack
 // is exactly as deep as the order says with NaN guard entries after it, and every
 // adjoint word starts as NaN.  Prints per tree: links, error of the new state, of
-// the gradients in q, qd, tau and the masses (each relative to the largest entry), and
+// the gradients in q, qd, tau and the masses, of four steps by the fused pass against whole
+// steps (each relative to the largest entry), and
 // whether the guards are intact.
 #include <algorithm>
 #include <cmath>
@@ -87,10 +88,27 @@ int main() {
     wstep_forward<D, D, true, false, true>(w, qc, qdc, tc, g, dt, integ, Col<D>{nullptr, 0}, Col<D>{nullptr, 0});
     wstep_adjoint<D, D, true>(w, Col<D>{gqb.data(), 1}, Col<D>{gqdb.data(), 1}, Col<D>{gtb.data(), 1},
                               Col<D>{gmb.data(), 1}, dt, integ, g);
+    // a rollout's fused pass (accelerations of one step, pose of the next) against whole steps
+    Vec qf = q, vf = qd, qs = q, vs = qd;
+    const Col<D> qfc{qf.data(), 1}, vfc{vf.data(), 1};
+    const Col<const D> qfr{qf.data(), 1}, vfr{vf.data(), 1};
+    const D h = 1e-2;
+    for (int t = 0; t < 4; ++t) {
+      if (t == 0)
+        wpass_pose<D, D, false, true>(w, qfr, vfr);
+      else
+        wpass_accel_pose<D, D, true>(w, qfc, vfc, g, h, integ);
+      wpass_inward<D, D, false, true>(w, vfr, tc);
+    }
+    wpass_accel<D, D, false, true, true>(w, qfr, vfr, g, h, integ, qfc, vfc);
+    for (int t = 0; t < 4; ++t)
+      wstep_forward<D, D, false, true, true>(w, Col<const D>{qs.data(), 1}, Col<const D>{vs.data(), 1}, tc, g, h, integ,
+                                             Col<D>{qs.data(), 1}, Col<D>{vs.data(), 1});
+    const D fused = std::max(err(qs, qf), err(vs, vf));
     bool guards = true;
     for (size_t i = (size_t)to.depth * WSW * LANES; i < stk.size(); ++i) guards &= std::isnan(stk[i]);
-    std::printf("%d %.3e %.3e %.3e %.3e %.3e %d\n", n, std::max(err(xa, xb), err(va, vb)), err(gqa, gqb),
-                err(gqda, gqdb), err(gta, gtb), err(gma, gmb), guards ? 1 : 0);
+    std::printf("%d %.3e %.3e %.3e %.3e %.3e %.3e %d\n", n, std::max(err(xa, xb), err(va, vb)), err(gqa, gqb),
+                err(gqda, gqdb), err(gta, gtb), err(gma, gmb), fused, guards ? 1 : 0);
   }
   return 0;
 }
