@@ -18,7 +18,9 @@
  *   tau  [T][nv_max][B]     joint forces; tau^t acts over step t -> t+1
  *   ckpt [ceil(T/k)][nq_max+nv_max][B]   x^t = (q^t, qd^t) for t = 0, k, 2k, ...
  *   traj [T+1][nq_max+nv_max][B]         x^0 .. x^T (optional)
- * Scalars are double for SIM_FP64 and float for SIM_FP32 / SIM_FP32_D64.
+ * Scalars are double for SIM_FP64 and float for SIM_FP32 / SIM_FP32_D64. The
+ * SIM_FP32_D64 mode runs the articulated-inertia solves (1/D, the rank-one update,
+ * the free root's 6x6 solve) in pairs of floats of 48 significant bits.
  * Per-link arrays (gmass, set_masses) follow the link order of the model
  * description (CSR by system).
  *
@@ -329,7 +331,7 @@ int sim_set_prefetch(sim_handle* h, int32_t links_ahead);
 int sim_set_replay(sim_handle* h, int32_t mode);
 
 /* Running-state precision of sim_rollout in SIM_FP32_D64 mode (the mixed mode's
- * FP64 D-solves leave the step-to-step state sums in FP32; the paper does not say
+ * D-solves leave the step-to-step state sums in FP32; the paper does not say
  * which).  fp64 = 1: sim_rollout keeps q and qd in FP64 (device memory the handle
  * allocates here, (nq_max + nv_max) * n_systems doubles) and accumulates the
  * integrator's sums there; every step's dynamics read the FP32 rounding of that

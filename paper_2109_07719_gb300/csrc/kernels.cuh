@@ -969,10 +969,10 @@ int choose_w(sim_handle* h, K k_on, K k_off, bool bwd, bool* onchip, int* thread
 // The world-aligned path applies to models without contact spheres or limits whose
 // state and input streams fit a block's shared memory: under SIM_TAPE_ALIGNED (all
 // joints revolute), or under SIM_TAPE_AUTO unless the link-frame two-warp rollout of
-// serial chains applies.  Floating bases take it under SIM_TAPE_AUTO: rollout +
-// adjoint of 8192 quadrupeds over 60 steps (FP32 + FP64 D-solves) 15.6 -> 11.3 ms
-// against the link-frame one-warp kernels, 1024 humanoids over 60 steps (FP32) 10.95
-// -> 4.39 ms.
+// serial chains applies.  Floating bases take it under SIM_TAPE_AUTO: when they moved here
+// from the link-frame one-warp kernels, rollout + adjoint of 8192 quadrupeds over 60 steps
+// in the mixed mode went from 15.6 to 11.3 ms (now 3.4), of 1024 humanoids over 60 steps in
+// FP32 from 10.95 to 4.4 (now 3.5).
 template <class T, class DT>
 bool use_aligned(const sim_handle* h, bool rollout) {
   const bool fr = !h->all_revolute;
@@ -1024,8 +1024,8 @@ int launch_wbackward_pipe(sim_handle* h, const void* ckpt, const void* tau, int6
   const bool fr = !h->all_revolute;
   const int tiles = (h->B + LANES - 1) / LANES, sms = std::max(1, h->sms);
   auto need = [&](bool on, int np) {
-    return (size_t)wpipe_smem_per_tile(h->maxL, nx, h->nv_max, on, on ? h->wdepth * WSW : m.sd, fr, np, m.slots) * LANES *
-           sizeof(T);
+    return (size_t)wpipe_smem_per_tile(h->maxL, nx, h->nv_max, on, on ? h->wdepth * WSW : m.sd, fr, np, m.slots, k > 1) *
+           LANES * sizeof(T);
   };
   const bool onchip = need(true, 1) <= (size_t)limit && (!fr || tiles <= sms);
   // Producers: three while every tile has an SM to itself (4096 7-link chains, on chip: 6.3

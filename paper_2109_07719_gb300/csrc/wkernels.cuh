@@ -143,7 +143,7 @@ __device__ __forceinline__ void wrollout_one(const DevModel<T>& m, int slot, boo
     if (t == 0)
       wpass_pose<T, DT, false, FR>(s, cq, cqd);
     else  // x^t from step t - 1's accelerations, and its pose
-      wpass_accel_pose<T, DT, FR>(s, q, qd, g, m.dt, m.integ);
+      wpass_accel_pose<T, DT, FR>(s, cq, cqd, g, m.dt, m.integ, q, qd);
     if (traj) put(traj + t * NX * B);
     if (ckpt && t % k == 0) put(ckpt + (t / k) * NX * B);
     Col<const T> tau_t{tau + t * nvm * B + b, B};
@@ -255,8 +255,9 @@ __device__ __forceinline__ void wbackward_one(const DevModel<T>& m, int slot, bo
         T* r0 = ring + rs;
         if (act)
           for (int d = 0; d < NX; ++d) r0[d * B] = xs[d * B];
-        for (long long j = 1; j < t1 - t0; ++j)
-          replay(ring + (j - 1) * NX * B + rs, ring + j * NX * B + rs, t0 + j - 1);
+        wstep_replay<T, DT, FR>(s, r0, NX * B, B, nqm, t1 - t0 - 1,
+                                [&](long long j) { return Col<const T>{tau + (t0 + j) * nvm * B + b, B}; }, g, m.dt,
+                                m.integ);
       }
       for (long long t = t1 - 1; t >= t0; --t) {
         const T* x = ring + (t - t0) * NX * B + rs;

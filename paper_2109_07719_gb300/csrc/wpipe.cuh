@@ -37,9 +37,9 @@ __host__ __device__ __forceinline__ int wpipe_tapes(int np) { return np > 1 ? np
 // double-buffered inputs (x^t, tau^t); without ONCHIP the warps' rings of `slots`
 // slots, and their stacks if the launch has room (sd > 0).
 __host__ __device__ __forceinline__ long long wpipe_smem_per_tile(int maxL, int nx, int nv, bool onchip, int sd,
-                                                                  bool fr, int np, int slots) {
+                                                                  bool fr, int np, int slots, bool seg) {
   const long long state = nx + maxL;
-  if (!onchip) return state + (np + 1LL) * sd + (long long)slots * (RING_ADJ + np * RING_FWD);
+  if (!onchip) return state + (np + 1LL) * sd + (long long)slots * (RING_ADJ + np * (seg ? RING_ROLL : RING_FWD));
   return wpipe_tapes(np) * w_tape_words(maxL, fr) + (np + 1LL) * sd + (long long)maxL * (NWA + NPRM_W + 1) + state +
          2LL * np * (nx + nv);
 }
@@ -70,6 +70,7 @@ k_wbackward_pipe(DevModel<T> m, const T* __restrict__ ckpt, const T* __restrict_
   const long long units = (B + LANES - 1) / LANES;
   const V3<T> g{m.g0, m.g1, m.g2};
   constexpr int MS = (int)(sizeof(T) / sizeof(int));
+  constexpr int RING_PROD = SEG ? RING_ROLL : RING_FWD;  // a replay's fused pass reads more rows
   T* base = reinterpret_cast<T*>(g_smem);
   T *s_tape = nullptr, *s_adj = nullptr, *s_prm = nullptr, *s_meta = nullptr, *s_in = nullptr;
   T* s_ring = nullptr;
@@ -84,8 +85,8 @@ k_wbackward_pipe(DevModel<T> m, const T* __restrict__ ckpt, const T* __restrict_
     s_meta = base;
     base += L * LANES;
   } else {
-    s_ring = base + (long long)m.slots * LANES * (consumer ? 0 : RING_ADJ + (warp - 1) * RING_FWD);
-    base += (long long)m.slots * LANES * (RING_ADJ + NP * RING_FWD);
+    s_ring = base + (long long)m.slots * LANES * (consumer ? 0 : RING_ADJ + (warp - 1) * RING_PROD);
+    base += (long long)m.slots * LANES * (RING_ADJ + NP * RING_PROD);
   }
   T* s_stk = base + warp * sdw * LANES + lane;  // [NP + 1][sdw][LANES]: one per warp
   base += (NP + 1) * sdw * LANES;
@@ -142,10 +143,9 @@ k_wbackward_pipe(DevModel<T> m, const T* __restrict__ ckpt, const T* __restrict_
         if (act)
           for (int d = 0; d < NX; ++d) r[d * B] = xs[d * B];
         if (ONCHIP ? act : true)
-          for (long long t = t0; t + 1 < t1; ++t, r += NX * B)
-            wstep_forward<T, DT, false, true, FR>(sp, Col<const T>{r, B}, Col<const T>{r + nqm * B, B},
-                                                  Col<const T>{tau + t * nvm * B + b, B}, g, m.dt, m.integ,
-                                                  Col<T>{r + NX * B, B}, Col<T>{r + (NX + nqm) * B, B});
+          wstep_replay<T, DT, FR>(sp, r, NX * B, B, nqm, t1 - t0 - 1,
+                                  [&](long long j) { return Col<const T>{tau + (t0 + j) * nvm * B + b, B}; }, g, m.dt,
+                                  m.integ);
         __threadfence_block();
         __syncwarp();
       }

@@ -649,16 +649,17 @@ SD void wpass_accel(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd, V3<T
   }
 }
 
-// The acceleration pass of one step, integrated in place, and the pose pass of the next in
-// one walk: a rollout's two outward passes without the second round of record loads, and
+// The acceleration pass of one step from (q, qd), integrated into (qo, qdo), which may alias
+// them, and the pose pass of the next in one walk: a rollout's two outward passes without the second round of record loads, and
 // two independent chains (accelerations; orientations and velocities) in one instruction
 // stream (rollout of 16384 trees of 2-64 links 119 -> 98 us a step).
 template <class T, class DT, bool FR, bool STG>
-SD void wpass_accel_pose(const WSys<T, STG>& s, Col<T> q, Col<T> qd, V3<T> grav, T dt, int integ) {
+SD void wpass_accel_pose(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd, V3<T> grav, T dt, int integ,
+                         Col<T> qo, Col<T> qdo) {
   T* tp = s.tape;
   const int nl = s.nl, walk = s.walk();
   Records<T, STG, 1, RING_ROLL, 0, W_XY, P_E, 12, 0, 0, W_V, 6> rec(s, walk);
-  Inputs<T, STG, true> in(s, Col<const T>{q.p, q.B}, Col<const T>{qd.p, qd.B}, 0, 1, walk);
+  Inputs<T, STG, true> in(s, q, qd, 0, 1, walk);
   const SV<T> a0{zero3<T>(), -grav};
   SV<T> a_prev = a0, v_prev = zeroSV<T>();
   M3<T> R_prev = eye3<T>();
@@ -682,12 +683,12 @@ SD void wpass_accel_pose(const WSys<T, STG>& s, Col<T> q, Col<T> qd, V3<T> grav,
       for (int i = 0; i < 6; ++i) {
         const T v0 = qd[vi + i];
         v1[i] = v0 + dt * qdd[i];
-        qd[vi + i] = v1[i];
+        qdo[vi + i] = v1[i];
         nu[i] = integ == I_SEMI_IMPLICIT ? v1[i] : v0;
       }
       for (int i = 0; i < 7; ++i) x[i] = q[qi + i];
       free_advance(x, nu, dt);
-      for (int i = 0; i < 7; ++i) q[qi + i] = x[i];
+      for (int i = 0; i < 7; ++i) qo[qi + i] = x[i];
       R = mTm(fld_m3(rec.p, P_E), quat_R(x[3], x[4], x[5], x[6]));
       v = SV<T>{mul(R, V3<T>{v1[0], v1[1], v1[2]}), mul(R, V3<T>{v1[3], v1[4], v1[5]})};
     } else {
@@ -714,8 +715,8 @@ SD void wpass_accel_pose(const WSys<T, STG>& s, Col<T> q, Col<T> qd, V3<T> grav,
       a = SV<T>{ap.w + qdd * sx, ap.v};
       const T v1 = v0 + dt * qdd;
       const T q1 = in.a + dt * (integ == I_SEMI_IMPLICIT ? v1 : v0);
-      qd[vi] = v1;
-      q[qi] = q1;
+      qdo[vi] = v1;
+      qo[qi] = q1;
       T sn, cs;
       sincos_t(q1, &sn, &cs);
       const V3<T> d = mul(Rp, fld_v3(rec.p, P_R));
@@ -735,6 +736,24 @@ SD void wpass_accel_pose(const WSys<T, STG>& s, Col<T> q, Col<T> qd, V3<T> grav,
     R_prev = R;
     v_prev = v;
     a_prev = a;
+  }
+}
+
+// n steps from the state at x0, each state `stride` after the one before (a replayed segment;
+// columns of B systems), q first, qd after nq coordinates.
+template <class T, class DT, bool FR, bool STG, class TAU>
+SD void wstep_replay(const WSys<T, STG>& s, T* x0, long long stride, long long B, int nq, long long n, TAU&& tau_of, V3<T> grav,
+                     T dt, int integ) {
+  T* x = x0;
+  for (long long t = 0; t < n; ++t, x += stride) {
+    const Col<const T> q{x, B}, qd{x + nq * B, B};
+    const Col<T> qo{x + stride, B}, qdo{x + stride + nq * B, B};
+    if (t == 0) wpass_pose<T, DT, false, FR>(s, q, qd);
+    wpass_inward<T, DT, false, FR>(s, qd, tau_of(t));
+    if (t + 1 < n)
+      wpass_accel_pose<T, DT, FR>(s, q, qd, grav, dt, integ, qo, qdo);
+    else
+      wpass_accel<T, DT, false, true, FR>(s, q, qd, grav, dt, integ, qo, qdo);
   }
 }
 

@@ -97,7 +97,7 @@ int main() {
       if (t == 0)
         wpass_pose<D, D, false, true>(w, qfr, vfr);
       else
-        wpass_accel_pose<D, D, true>(w, qfc, vfc, g, h, integ);
+        wpass_accel_pose<D, D, true>(w, qfr, vfr, g, h, integ, qfc, vfc);
       wpass_inward<D, D, false, true>(w, vfr, tc);
     }
     wpass_accel<D, D, false, true, true>(w, qfr, vfr, g, h, integ, qfc, vfc);
