@@ -3,9 +3,9 @@
 // the step; the warps share the columns of A = J M^-1 J^T, three to a test pass, and their
 // reverse in the adjoint, each with a contact tape of its own.
 //
-// Why: with feet on the ground the test passes were about 85 % of a step, on one warp of an
-// SM's four schedulers (in FP64 each scheduler has its own half-lane-per-cycle unit, so
-// one warp reached a quarter of the SM's rate).  A quadruped's four feet are four groups.
+// Why: with feet on the ground the test passes were about half of a step (what the split
+// below took away says so), on one warp of an SM's four schedulers (in FP64 each scheduler
+// has its own half-lane-per-cycle unit, so one warp reached a quarter of the SM's rate).  A quadruped's four feet are four groups.
 // Rollout + adjoint over 12 steps with four feet down: 512 quadrupeds in FP64 46.4 -> 30.6
 // ms, 256 in FP32 8.0 -> 6.4, 8192 in the mixed mode 20.2 -> 14.4.  What is left is the first
 // warp's: the ABA, the 20 sweeps of 12 dependent updates and their adjoints.
