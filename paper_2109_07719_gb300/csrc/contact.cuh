@@ -434,6 +434,13 @@ template <class T, class PT> SD Rows<T> active_rows(const Sys<T, PT>& s, const C
   return r;
 }
 
+// Where stored link l belongs among the n links listed so far, in the model's order.
+template <class T, class PT> SD int row_place(const Sys<T, PT>& s, const int* links, int n, int l) {
+  const int vo = meta_voff(s.M(l));
+  while (n > 0 && meta_voff(s.M(links[n - 1])) > vo) --n;
+  return n;
+}
+
 // The constraint step is in parts, so that several warps can share one system's columns
 // of A (each with a contact tape of its own for the test passes): the rows and b
 // (contact_rows), the columns in groups of three (contact_columns, group j of `parts`
@@ -445,26 +452,37 @@ template <class T, class DT, class PT>
 CD int contact_rows(Sys<T, PT> s, CView<T> cv, Col<const T> q, Col<const T> qd, T dt, ContactParams<T> cp) {
   const int nl = s.nl;
   world_poses(s, cv);
+  // The sweeps visit the rows in the model's link order, whatever order the links are stored
+  // in: a fixed number of sweeps has not converged, so the order is part of the result.  The
+  // velocity offsets grow with the model's numbering.
   int nc = 0;
   int link[MAXC];
-  V3<T> pc[MAXC];
+  T cphi[MAXC];
   for (int l = 0; l < nl && nc < MAXC; ++l) {
     const T r = s.P(l, P_CR);
     if (!(r >= T(0))) continue;
-    const V3<T> p = s.pv3(l, P_CP);
-    const V3<T> y = cget3(cv, l, C_OW) + mulT(cgetm(cv, l, C_EW), p);
+    const V3<T> y = cget3(cv, l, C_OW) + mulT(cgetm(cv, l, C_EW), s.pv3(l, P_CP));
     const T phi = y.z - r;
     if (phi < T(0)) {
-      link[nc] = l;
-      pc[nc] = p;
-      cv.S(S_LINK + nc) = (T)l;
-      cv.S(S_PHI + nc) = phi;
+      const int at = row_place(s, link, nc, l);
+      for (int c = nc; c > at; --c) {
+        link[c] = link[c - 1];
+        cphi[c] = cphi[c - 1];
+      }
+      link[at] = l;
+      cphi[at] = phi;
       ++nc;
     }
   }
+  V3<T> pc[MAXC];
+  for (int c = 0; c < nc; ++c) {
+    pc[c] = s.pv3(link[c], P_CP);
+    cv.S(S_LINK + c) = (T)link[c];
+    cv.S(S_PHI + c) = cphi[c];
+  }
   int nlr = 0;
   int llink[MAXL];
-  T lsg[MAXL];
+  T lsg[MAXL], lphi[MAXL];
   for (int l = 0; l < nl && nlr < MAXL; ++l) {
     const int m = s.M(l);
     if (meta_jtype(m) != J_REVOLUTE) continue;
@@ -480,12 +498,21 @@ CD int contact_rows(Sys<T, PT> s, CView<T> cv, Col<const T> q, Col<const T> qd, 
     } else {
       continue;
     }
-    llink[nlr] = l;
-    lsg[nlr] = sg;
-    cv.S(S_LINK + MAXC + nlr) = (T)l;
-    cv.S(S_PHI + MAXC + nlr) = phi;
-    cv.S(S_SGN + nlr) = sg;
+    const int at = row_place(s, llink, nlr, l);
+    for (int k = nlr; k > at; --k) {
+      llink[k] = llink[k - 1];
+      lsg[k] = lsg[k - 1];
+      lphi[k] = lphi[k - 1];
+    }
+    llink[at] = l;
+    lsg[at] = sg;
+    lphi[at] = phi;
     ++nlr;
+  }
+  for (int k = 0; k < nlr; ++k) {
+    cv.S(S_LINK + MAXC + k) = (T)llink[k];
+    cv.S(S_PHI + MAXC + k) = lphi[k];
+    cv.S(S_SGN + k) = lsg[k];
   }
   cv.S(S_NC) = (T)nc;
   cv.S(S_NL) = (T)nlr;
