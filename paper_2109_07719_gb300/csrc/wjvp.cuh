@@ -40,9 +40,8 @@ SD void wstep_jvp(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd, Col<co
       const SV<T> v = fld_sv(rec.t, W_V), ap = fld_sv(rec.t, W_AP);
       SV<T> a = ap, dv = zeroSV<T>(), da = zeroSV<T>();
       S3<T> Ic;
-      if (fr) {  // v = R qd, a = R qdd + [0; -g]: the gravity turns against R
-        const M3<T> R = fld_rot(rec.t);
-        dv = SV<T>{mul(R, V3<T>{dqd[vi], dqd[vi + 1], dqd[vi + 2]}), mul(R, V3<T>{dqd[vi + 3], dqd[vi + 4], dqd[vi + 5]})};
+      if (fr) {  // v = qd, a = qdd + [0; -E g]
+        dv = SV<T>{{dqd[vi], dqd[vi + 1], dqd[vi + 2]}, {dqd[vi + 3], dqd[vi + 4], dqd[vi + 5]}};
         Dual<T> x[4];
         for (int i = 0; i < 4; ++i) x[i] = Dual<T>(q[qi + 3 + i], dq[qi + 3 + i]);
         const M3<Dual<T>> Rq = quat_R(x[0], x[1], x[2], x[3]);
@@ -51,7 +50,7 @@ SD void wstep_jvp(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd, Col<co
           dEJ.a[i] = Rq.a[3 * (i % 3) + i / 3].d;
           Et.a[i] = s.P(l, P_E + i);
         }
-        da.v = mul(R, mul(dEJ, mul(Et, zero3<T>() - grav)));
+        da.v = mul(dEJ, mul(Et, zero3<T>() - grav));
         Ic = ws3(s.root, 0, 0, WF_IC);
       } else {
         const T vl = fld(rec.t, W_QD), x = dq[qi], xd = dqd[vi];
@@ -109,10 +108,8 @@ SD void wstep_jvp(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd, Col<co
         df += wsv(s.stk, WSW, sp, 6);
         y += wsv(s.stk, WSW, sp, 12);
       }
-      if (FR && meta_jtype(m) == J_FREE) {  // dqdd of the root: R^T (I^A)^-1 (R dtau - df + y)
-        const M3<T> R = fld_rot((const T*)tp + l * NWT * LANES);
-        const SV<T> t{mul(R, V3<T>{dtau[vi], dtau[vi + 1], dtau[vi + 2]}),
-                      mul(R, V3<T>{dtau[vi + 3], dtau[vi + 4], dtau[vi + 5]})};
+      if (FR && meta_jtype(m) == J_FREE) {  // dqdd of the root: (I^A)^-1 (dtau - df + y)
+        const SV<T> t{{dtau[vi], dtau[vi + 1], dtau[vi + 2]}, {dtau[vi + 3], dtau[vi + 4], dtau[vi + 5]}};
         wsv(s.adj, NWJ, l, WJ_DF, spd_solve<T, DT>(wsi(s.root, 0, 0, WF_IA), t - df + y));
         continue;
       }
@@ -152,9 +149,7 @@ SD void wstep_jvp(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd, Col<co
     SV<T> w = zeroSV<T>();
     if (FR && meta_jtype(m) == J_FREE) {
       w = wsv(s.adj, NWJ, l, WJ_DF);
-      const M3<T> R = fld_rot((const T*)tp + l * NWT * LANES);
-      const V3<T> bw = mulT(R, w.w), bv = mulT(R, w.v);
-      const T x[6] = {bw.x, bw.y, bw.z, bv.x, bv.y, bv.z};
+      const T x[6] = {w.w.x, w.w.y, w.w.z, w.v.x, w.v.y, w.v.z};
       Dual<T> nu[6], p[7];
       for (int i = 0; i < 6; ++i) {
         const Dual<T> v0(qd[vi + i], dqd[vi + i]);

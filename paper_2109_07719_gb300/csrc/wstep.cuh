@@ -31,6 +31,15 @@
 //            qdd = (u - U.a') / D,  a = a' + [s qdd; 0]
 // shift(I, d) = X^T I X with X = (1, d): the congruence by a pure translation.
 //
+// A tree with a free root (FR) is written in the axes of its base instead of the world's:
+// R = 1 and v = qd at the root, and only the gravity turns, E g with E = R(quat)^T E_tree.
+// The axes need not be the world's, only the same for the whole tree; in the base's own, the
+// base's orientation rounds nothing else, and a quaternion that is not of unit length acts as
+// in the link-frame step, through the gravity and the position alone.  (In world axes an
+// FP32 step's own part of the new state had 3 times the link-frame step's error, of the
+// gradient in q 6 times; in the base's axes 2 and 0.9, over random bases of 13 and 23 links.
+// A quaternion rounded to float was 1e-7 off in FP64, now 1e-16.)
+//
 // Adjoint step.  The joint accelerations solve M qdd = tau - b qd - C(q, qd), i.e.
 // RNEA(q, qd, qdd) + b qd = tau, so with qddb the adjoint of qdd
 //   lambda = M^-1 qddb,  taub = lambda,  (q, qd, m)b = -d(lambda . (RNEA + b qd)) at fixed qdd
@@ -74,12 +83,14 @@ namespace abasim {
 // the acceleration pass).
 enum : int {
   W_U = 0, W_DI = 6, W_u = 8, W_D = 9, W_S = 12, W_XY = 15, W_V = 21, W_AP = 27, W_QDD = 33, W_QD = 34, W_RW = 35,
-  NWT = 38
+  NWT = 38,
+  W_E = 0  // a free root's E, in the words of U, 1/D and u, which it does not have
 };
 // Record of a free root (FR kernels; link 0 only), [field][lane]: its articulated
-// inertia, qdd, the quaternion and velocity the step started from and the rotated COM
-// inertia.  Its link's tape words hold R whole and its acceleration in W_AP.
-enum : int { WF_IA = 0, WF_QDD = 21, WF_Q = 27, WF_QD = 31, WF_IC = 37, NWF = 43 };
+// inertia, qdd (its linear part then gives way to that of qddb), the quaternion and velocity
+// the step started from and its COM inertia.  Its link's tape words hold E, R = 1 whole and
+// its acceleration in W_AP.
+enum : int { WF_IA = 0, WF_QDD = 21, WF_QDDB = WF_QDD + 3, WF_Q = 27, WF_QD = 31, WF_IC = 37, NWF = 43 };
 // Per-link adjoint record, [link][field][lane]: W = -w.
 enum : int { WA_W = 0, NWA = 6 };
 // One entry of the stack of parent values, [entry][field][lane]: (R, v), a or W in
@@ -416,9 +427,13 @@ template <class T> SD void add_body(T m, V3<T> rw, const S3<T>& Ic, SV<T> v, SI<
   pA += SV<T>{cross(v.w, mul(Ic, v.w)) + cross(rw, f), f};
 }
 
+// A free root's rotation from the parent's axes to its own, from the quaternion as it is given.
+template <class T> SD M3<T> free_rotation(const T* qt, const M3<T>& Et) {
+  return mTm(quat_R(qt[0], qt[1], qt[2], qt[3]), Et);
+}
+
 // The passes of a step.  ADJ: also store what the adjoint reads.  FR: link 0 may be a free
-// joint (R = E_tree^T R(quat), S = R on both halves, so D = I^A in world axes: one Cholesky
-// solve).
+// joint (its tree's axes: R = 1, S = 1 on both halves, D = I^A, one Cholesky solve).
 template <class T, class DT, bool ADJ, bool FR, bool STG>
 SD void wpass_pose(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd) {
   T* tp = s.tape;
@@ -444,8 +459,9 @@ SD void wpass_pose(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd) {
         const T qt[4] = {q[qi + 3], q[qi + 4], q[qi + 5], q[qi + 6]};
         T x[6];
         for (int i = 0; i < 6; ++i) x[i] = qd[vi + i];
-        R = mTm(fld_m3(rec.p, P_E), quat_R(qt[0], qt[1], qt[2], qt[3]));
-        v = SV<T>{mul(R, V3<T>{x[0], x[1], x[2]}), mul(R, V3<T>{x[3], x[4], x[5]})};
+        R = eye3<T>();
+        v = SV<T>{{x[0], x[1], x[2]}, {x[3], x[4], x[5]}};
+        wm3(w, 0, 0, W_E, free_rotation(qt, fld_m3(rec.p, P_E)));
         if (ADJ) {
           for (int i = 0; i < 4; ++i) s.root[(WF_Q + i) * LANES] = qt[i];
           for (int i = 0; i < 6; ++i) s.root[(WF_QD + i) * LANES] = x[i];
@@ -531,9 +547,8 @@ SD void wpass_inward(const WSys<T, STG>& s, Col<const T> qd, Col<const T> tau) {
         IA += wsi(s.stk, WSW, sp, 0);
         pA += wsv(s.stk, WSW, sp, 21);
       }
-      if (fr) {  // D = I^A, u = R tau - p^A
-        const SV<T> f{mul(R, V3<T>{tau[vo], tau[vo + 1], tau[vo + 2]}),
-                      mul(R, V3<T>{tau[vo + 3], tau[vo + 4], tau[vo + 5]})};
+      if (fr) {  // D = I^A, u = tau - p^A
+        const SV<T> f{{tau[vo], tau[vo + 1], tau[vo + 2]}, {tau[vo + 3], tau[vo + 4], tau[vo + 5]}};
         if (ADJ) wsi(s.root, 0, 0, WF_IA, IA);
         wsv(w, 0, 0, W_AP, spd_solve<T, DT>(IA, f - pA));
         continue;
@@ -589,11 +604,9 @@ SD void wpass_accel(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd, V3<T
     T* w = tp + l * NWT * LANES;
     SV<T> a;
     if (FR && meta_jtype(m) == J_FREE) {
-      const M3<T> R = fld_rot((const T*)w);
       a = wsv(w, 0, 0, W_AP);
-      const SV<T> b = a - a0;
-      const V3<T> bw = mulT(R, b.w), bv = mulT(R, b.v);
-      const T qdd[6] = {bw.x, bw.y, bw.z, bv.x, bv.y, bv.z};
+      const V3<T> bv = a.v + mul(fld_m3(rec.t, W_E), grav);
+      const T qdd[6] = {a.w.x, a.w.y, a.w.z, bv.x, bv.y, bv.z};
       if (ADJ)
         for (int i = 0; i < 6; ++i) s.root[(WF_QDD + i) * LANES] = qdd[i];
       if (INTEG) {
@@ -674,11 +687,10 @@ SD void wpass_accel_pose(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd,
     SV<T> a, v;
     M3<T> R;
     if (FR && meta_jtype(m) == J_FREE) {
-      R = fld_rot((const T*)w);
+      R = eye3<T>();
       a = wsv(w, 0, 0, W_AP);
-      const SV<T> b = a - a0;
-      const V3<T> bw = mulT(R, b.w), bv = mulT(R, b.v);
-      const T qdd[6] = {bw.x, bw.y, bw.z, bv.x, bv.y, bv.z};
+      const V3<T> bv = a.v + mul(fld_m3(rec.t, W_E), grav);
+      const T qdd[6] = {a.w.x, a.w.y, a.w.z, bv.x, bv.y, bv.z};
       T v1[6], nu[6], x[7];
       for (int i = 0; i < 6; ++i) {
         const T v0 = qd[vi + i];
@@ -689,8 +701,8 @@ SD void wpass_accel_pose(const WSys<T, STG>& s, Col<const T> q, Col<const T> qd,
       for (int i = 0; i < 7; ++i) x[i] = q[qi + i];
       free_advance(x, nu, dt);
       for (int i = 0; i < 7; ++i) qo[qi + i] = x[i];
-      R = mTm(fld_m3(rec.p, P_E), quat_R(x[3], x[4], x[5], x[6]));
-      v = SV<T>{mul(R, V3<T>{v1[0], v1[1], v1[2]}), mul(R, V3<T>{v1[3], v1[4], v1[5]})};
+      v = SV<T>{{v1[0], v1[1], v1[2]}, {v1[3], v1[4], v1[5]}};
+      wm3(w, 0, 0, W_E, free_rotation(x + 3, fld_m3(rec.p, P_E)));
     } else {
       SV<T> apar = a_prev, vp = v_prev;
       M3<T> Rp = R_prev;
@@ -792,7 +804,7 @@ template <class T> SD BodyGrad<T> body_grad(T m, V3<T> rw, const S3<T>& Ic, SV<T
 // Requires wstep_forward<ADJ = true>(q, qd, tau) to have filled the tape.  On entry
 // (gq, gqd) hold the adjoint of x^{k+1}; on exit that of x^k.  Writes the adjoint
 // of tau into gtau and adds dPhi/dm of every link into gm.  FR (link 0 may be a free
-// joint) needs the gravity: the only motion a free root's orientation turns against.
+// joint) needs the gravity, all that depends on a free root's orientation.
 template <class T, class DT, bool FR = false, bool STG = false>
 SD void wstep_adjoint(const WSys<T, STG>& s, Col<T> gq, Col<T> gqd, Col<T> gtau, Col<T> gm, T dt, int integ,
                       V3<T> grav = zero3<T>()) {
@@ -816,7 +828,7 @@ SD void wstep_adjoint(const WSys<T, STG>& s, Col<T> gq, Col<T> gqd, Col<T> gtau,
         --sp;
         y += wsv(s.stk, WSW, sp, 0);
       }
-      if (FR && meta_jtype(m) == J_FREE) {  // lambda_root = (I^A)^-1 (R qddb + y)
+      if (FR && meta_jtype(m) == J_FREE) {  // lambda_root = (I^A)^-1 (qddb + y)
         T qt[4], nu[6], qddb6[6];
         for (int i = 0; i < 4; ++i) qt[i] = s.root[(WF_Q + i) * LANES];
         for (int i = 0; i < 6; ++i) {
@@ -824,12 +836,11 @@ SD void wstep_adjoint(const WSys<T, STG>& s, Col<T> gq, Col<T> gqd, Col<T> gtau,
           if (integ == I_SEMI_IMPLICIT) nu[i] += dt * s.root[(WF_QDD + i) * LANES];
         }
         free_integrator_adjoint(qt, nu, gq, gqd, qi, vi, dt, integ, qddb6);
-        const M3<T> R = fld_rot((const T*)tp + l * NWT * LANES);
-        y += SV<T>{mul(R, V3<T>{qddb6[0], qddb6[1], qddb6[2]}), mul(R, V3<T>{qddb6[3], qddb6[4], qddb6[5]})};
+        y += SV<T>{{qddb6[0], qddb6[1], qddb6[2]}, {qddb6[3], qddb6[4], qddb6[5]}};
+        for (int i = 0; i < 3; ++i) s.root[(WF_QDDB + i) * LANES] = qddb6[3 + i];
         const SV<T> w = spd_solve<T, DT>(wsi(s.root, 0, 0, WF_IA), y);
         wsv(ad, NWA, l, WA_W, zeroSV<T>() - w);
-        const V3<T> lw = mulT(R, w.w), lv = mulT(R, w.v);
-        const T lam[6] = {lw.x, lw.y, lw.z, lv.x, lv.y, lv.z};
+        const T lam[6] = {w.w.x, w.w.y, w.w.z, w.v.x, w.v.y, w.v.z};
         for (int i = 0; i < 6; ++i) gtau[vi + i] = lam[i];
         continue;
       }
@@ -926,14 +937,14 @@ SD void wstep_adjoint(const WSys<T, STG>& s, Col<T> gq, Col<T> gqd, Col<T> gtau,
         g.ab += wsv(s.stk, WSW, sp, 6);
         g.F += wsv(s.stk, WSW, sp, 12);
       }
-      if (fr) {  // v = R qd, a = R qdd + [0; -g]: only the gravity does not turn with R
-        const M3<T> R = fld_rot(rec.t);
-        const V3<T> bw = mulT(R, g.vb.w), bv = mulT(R, g.vb.v);
-        const T vv[6] = {bw.x, bw.y, bw.z, bv.x, bv.y, bv.z};
+      if (fr) {  // v = qd, a = qdd + [0; -E g]: only the gravity depends on the orientation
+        const T vv[6] = {g.vb.w.x, g.vb.w.y, g.vb.w.z, g.vb.v.x, g.vb.v.y, g.vb.v.z};
         for (int i = 0; i < 6; ++i) gqd[vi + i] += vv[i];
         M3<T> Et;
         for (int i = 0; i < 9; ++i) Et.a[i] = s.P(l, P_E + i);
-        const M3<T> EJb = mmT(outer(mulT(R, g.ab.v), zero3<T>() - grav), Et);  // E = E_J E_t
+        // dL/da of the whole tree is -M lambda = -qddb, which the sum over the links only approaches
+        const V3<T> qddb{s.root[WF_QDDB * LANES], s.root[(WF_QDDB + 1) * LANES], s.root[(WF_QDDB + 2) * LANES]};
+        const M3<T> EJb = mmT(outer(qddb, grav), Et);  // E = E_J E_t
         T qb[4] = {T(0), T(0), T(0), T(0)};
         quat_R_adj(s.root[WF_Q * LANES], s.root[(WF_Q + 1) * LANES], s.root[(WF_Q + 2) * LANES],
                    s.root[(WF_Q + 3) * LANES], transpose(EJb), qb);
