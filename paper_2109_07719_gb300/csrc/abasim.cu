@@ -375,6 +375,7 @@ int sim_create(const sim_model_desc* d, sim_handle** out) {
   }
   cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
   cudaDeviceGetAttribute(&h->smem_limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
+  h->smem_limit = std::max(0, h->smem_limit - kStaticSmem);
   h->all_chains = !any_contact;
   h->unconstrained = !any_contact;
   h->all_revolute = !any_contact;

@@ -14,6 +14,9 @@
 namespace abasim {
 namespace host {
 constexpr int kDefaultBlock = 32;
+// Of the shared memory a block may opt in to, left to the kernels' static variables (a work
+// ticket); a launch that asks for all of it is refused.
+constexpr int kStaticSmem = 128;
 }  // namespace host
 }  // namespace abasim
 
@@ -48,7 +51,7 @@ struct sim_handle {
   int prefetch = 2;          // links ahead the world-aligned global-tape passes prefetch
   int last_storage = 0, last_storage_bwd = 0;
   int sms = 0;
-  int smem_limit = 0;        // shared memory a block may opt in to, bytes
+  int smem_limit = 0;        // dynamic shared memory a launch may ask for, bytes
   bool all_chains = false;   // every system a serial chain of revolute joints (the pipelined adjoint)
   bool all_revolute = false; // every joint revolute and no contact spheres or limits
   bool unconstrained = false; // no contact spheres or limits (the world-aligned kernels; FR ones unless all_revolute)

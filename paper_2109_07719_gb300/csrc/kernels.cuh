@@ -904,7 +904,7 @@ inline int l1_carveout(const sim_handle* h, int slots_per_block, size_t bytes) {
 inline bool stacks_fit(const sim_handle* h, int slots_per_block, size_t bytes, int limit) {
   const long long units = (h->B + slots_per_block - 1) / slots_per_block, sms = std::max(1, h->sms);
   const long long blocks = std::min(2LL, (units + sms - 1) / sms);
-  return blocks * ((long long)bytes + 1024) <= (long long)limit + 1024;
+  return blocks * ((long long)bytes + kStaticSmem + 1024) <= (long long)limit + kStaticSmem + 1024;  // the SM's
 }
 
 // Scalars per tile of a world-aligned kernel's working state (w_smem_per_tile's, without
