@@ -916,7 +916,8 @@ inline long long w_state_per_tile(const sim_handle* h, bool bwd) {
 // Storage of a world-aligned one-warp launch: the tape on chip when a block's tiles fit the
 // per-block opt-in limit and that adds no wave of blocks over the global-tape kernel.  The
 // latter's rings take shared memory too: where a block of h->block threads with them would
-// not fit, it runs fewer tiles per block (*threads), then stages without looking ahead.
+// not fit, or needs more registers than an SM has, it runs fewer tiles per block (*threads),
+// then stages without looking ahead.
 template <class T, class K>
 int choose_w(sim_handle* h, K k_on, K k_off, bool bwd, bool* onchip, int* threads, int* slots, int* sd,
              size_t* bytes) {
@@ -931,6 +932,12 @@ int choose_w(sim_handle* h, K k_on, K k_off, bool bwd, bool* onchip, int* thread
   int tiles = h->block / LANES;
   *sd = 0;
   while (tiles > 1 && need(false, tiles) > (size_t)limit) --tiles;
+  if (tiles > 8) {  // any kernel runs 256 threads; more only if its registers allow them
+    cudaFuncAttributes a;
+    e = cudaFuncGetAttributes(&a, (const void*)k_off);
+    if (e != cudaSuccess) return cuda_fail(h, e, "kernel attributes");
+    tiles = std::max(1, std::min(tiles, a.maxThreadsPerBlock / LANES));
+  }
   if (need(false, tiles) > (size_t)limit) *slots = 1;
   *sd = h->wdepth * WSW;
   if (!stacks_fit(h, tiles * LANES, need(false, tiles), limit)) *sd = 0;

@@ -49,3 +49,15 @@ def test_whole_shared_memory(n, free, precision, threads, k):
     b = _run(w, precision, 0, "global", k)
     for name in a:
         check(name, a[name], b[name], 1e-3 if precision == "fp32" else 1e-9)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp32_d64"])
+@pytest.mark.parametrize("threads", [288, 416, 512])
+def test_large_blocks_of_floating_bases(precision, threads):
+    """Block sizes that the kernel's registers or shared memory do not allow run as smaller
+    blocks: the same arithmetic, so the same results up to the look-ahead's storage."""
+    w = wl.quadruped(B=600, T=3, precision=precision)
+    a = _run(w, precision, threads, "auto", 1)
+    b = _run(w, precision, 32, "auto", 1)
+    for name in a:
+        check(name, a[name], b[name], 1e-6)
