@@ -843,6 +843,14 @@ int launch_shape(sim_handle* h, K kernel, int* grid, int* persistent, size_t shm
   return e == cudaSuccess ? SIM_OK : cuda_fail(h, e, "work ticket reset");
 }
 
+// Lets a kernel's launches ask for dynamic shared memory up to the limit.  The attribute is the
+// kernel's, shared by every handle and thread, so all of them set the same value: with each
+// launch's own size, a smaller simulator's call could lower it between another thread's set
+// and launch, which then failed.
+inline cudaError_t allow_smem(const sim_handle* h, const void* kern) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, h->smem_limit);
+}
+
 // Storage mode and dynamic shared memory of a launch: the most on-chip mode that
 // fits the per-block opt-in limit and (in auto mode) adds no wave of blocks over
 // the all-global kernel.
@@ -865,7 +873,7 @@ int choose_storage(sim_handle* h, K0 k_global, K1 k_hybrid, K2 k_smem, bool bwd,
                         smem_per_tile(h->maxL, h->nq_max + h->nv_max, h->nv_max, bwd, mode) * LANES * sizeof(T);
     if (need > (size_t)limit) continue;
     const void* kern = mode == ST_SMEM ? (const void*)k_smem : (const void*)k_hybrid;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
+    e = allow_smem(h, (const void*)kern);
     if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory opt-in");
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, h->block, need);
@@ -943,7 +951,7 @@ int choose_w(sim_handle* h, K k_on, K k_off, bool bwd, bool* onchip, int* thread
   if (!stacks_fit(h, tiles * LANES, need(false, tiles), limit)) *sd = 0;
   const size_t need_on = need(true, h->block / LANES), need_off = need(false, tiles);
   if (need_off > (size_t)limit) return fail(h, SIM_EUNSUPPORTED, "the working state does not fit in shared memory");
-  e = cudaFuncSetAttribute((const void*)k_off, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need_off);
+  e = allow_smem(h, (const void*)k_off);
   if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory opt-in");
   // the global-tape kernel: shared memory for the blocks an SM holds at once, the rest of the SM's
   // unified L1 / shared storage as L1 for the stacks
@@ -954,7 +962,7 @@ int choose_w(sim_handle* h, K k_on, K k_off, bool bwd, bool* onchip, int* thread
   *threads = tiles * LANES;
   *bytes = need_off;
   if (need_on > (size_t)limit) return SIM_OK;
-  e = cudaFuncSetAttribute((const void*)k_on, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need_on);
+  e = allow_smem(h, (const void*)k_on);
   if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory opt-in");
   int per_on = 0, per_off = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_on, k_on, h->block, need_on);
@@ -1052,7 +1060,7 @@ int launch_wbackward_pipe(sim_handle* h, const void* ckpt, const void* tau, int6
   const int threads = (np + 1) * LANES;
   const BackwardKernel<T> kern =
       k > 1 ? wbackward_pipe_kernel<T, DT, true>(onchip, fr) : wbackward_pipe_kernel<T, DT, false>(onchip, fr);
-  e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+  e = allow_smem(h, (const void*)kern);
   if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory opt-in");
   if (!onchip) {  // shared memory for the blocks an SM holds at once, the rest of the SM's storage as L1
     e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -1154,7 +1162,7 @@ int launch_rollout(sim_handle* h, const void* q0, const void* qd0, const void* t
         }
       }
       if (piped) {
-        e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+        e = allow_smem(h, (const void*)kern);
         if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory opt-in");
       }
     }
@@ -1210,7 +1218,7 @@ int launch_backward(sim_handle* h, const void* ckpt, const void* tau, int64_t T_
           (size_t)pipe_smem_per_tile(h->maxL, h->nq_max + h->nv_max, h->nv_max) * LANES * sizeof(T);
       if (need <= (size_t)limit) {
         kern = backward_pipe_kernel<T, DT>();
-        e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
+        e = allow_smem(h, (const void*)kern);
         if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory opt-in");
         st = ST_PIPE;
         shm = need;
@@ -1282,7 +1290,7 @@ int launch_jvp(sim_handle* h, const void* q, const void* qd, const void* tau, co
     const size_t shm = need();
     if (shm <= (size_t)limit && (uintptr_t)work % 16 == 0) {
       const auto kern = h->all_revolute ? k_wstep_jvp<T, false> : k_wstep_jvp<T, true>;
-      e = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+      e = allow_smem(h, (const void*)kern);
       if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory opt-in");
       kern<<<(h->B + LANES - 1) / LANES, LANES, shm, S(stream)>>>(
           m, (const T*)q, (const T*)qd, (const T*)tau, (const T*)dq, (const T*)dqd, (const T*)dtau, (T*)q_out, (T*)qd_out,
