@@ -902,7 +902,7 @@ SD void step_adjoint(const Sys<T, PT, TL, AL>& s, Col<const T> q, Col<const T> q
           IAb += Iab;
           const SV<T> IbU = mul(Iab, U);
           Ub -= (T)(DT(2) * Di) * IbU;
-          Db += (T)(Di * Di * (DT)dot(U, IbU));
+          Db += (T)(Di * (Di * (DT)dot(U, IbU)));  // 1/D^2 alone may leave float's range
         }
         // u = tau - b qd - S^T pA,  D = S^T U,  U = IA S with S = [e_z; 0]:
         // IAb += sym_outer(Ub.w, e_z) and outer(e_z, Ub.v) / 2 (third column / row)
