@@ -406,13 +406,14 @@ int sim_create(const sim_model_desc* d, sim_handle** out) {
   if (rc == SIM_OK) rc = put(h->nqv, nqv.data(), B * sizeof(int));
   if (rc == SIM_OK) rc = alloc((void**)&h->link_slot, slot.size() * sizeof(int), "link map");
   if (rc == SIM_OK) rc = put(h->link_slot, slot.data(), slot.size() * sizeof(int));
-  if (rc == SIM_OK) rc = alloc(&h->tape, (size_t)maxL * NTAPE * Bpad * h->scalar, "tape");
+  // one buffer for the link-frame tape, the world-aligned one and the pipelined adjoint's
+  // tapes: a launch uses one of them
+  size_t tape_words = (size_t)maxL * NTAPE;
+  if (h->unconstrained)
+    tape_words = std::max(tape_words, (size_t)WPIPE_TAPES * (maxL * NWT + (h->all_revolute ? 0 : NWF)));
+  if (rc == SIM_OK) rc = alloc(&h->tape, tape_words * Bpad * h->scalar, "tape");
   if (rc == SIM_OK) rc = alloc(&h->adj, (size_t)maxL * NADJ * Bpad * h->scalar, "adjoint tape");
   if (rc == SIM_OK) rc = alloc(&h->gm_acc, (size_t)maxL * B * h->scalar, "mass-gradient buffer");
-  // the pipelined adjoint's tapes share the link-frame tape's buffer where they fit in it
-  const size_t ring_words = (size_t)WPIPE_TAPES * (maxL * NWT + (h->all_revolute ? 0 : NWF));
-  if (rc == SIM_OK && h->unconstrained && ring_words > (size_t)maxL * NTAPE)
-    rc = alloc(&h->wtapes, ring_words * Bpad * h->scalar, "world-aligned tapes");
   if (rc == SIM_OK && h->unconstrained && h->wdepth > 0)
     rc = alloc(&h->wstk, (size_t)(WPIPE_TAPES + 1) * h->wdepth * WSW * Bpad * h->scalar, "world-aligned stacks");
   if (rc == SIM_OK) rc = alloc((void**)&h->status, B * sizeof(int), "status");
@@ -442,7 +443,7 @@ int sim_create(const sim_model_desc* d, sim_handle** out) {
 void sim_destroy(sim_handle* h) {
   if (!h) return;
   void* ptrs[] = {h->prm, h->meta, h->nl, h->nqv, h->tape, h->adj, h->gm_acc, h->link_slot,
-                  h->status, h->sys_of_slot, h->counter, h->ctape, h->csys, h->x64, h->wtapes, h->wstk};
+                  h->status, h->sys_of_slot, h->counter, h->ctape, h->csys, h->x64, h->wstk};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   delete h;

@@ -31,9 +31,9 @@ struct sim_handle {
   int* meta = nullptr;       // [maxL][B]
   int* nl = nullptr;         // [B]
   int* nqv = nullptr;        // [B]  nq | nv << 16
-  void* tape = nullptr;      // [maxL][NTAPE][B] scalar
+  void* tape = nullptr;      // scalars of one launch's tape: [tile][maxL][NTAPE][lane] link-frame, [tile][maxL * NWT + NWF][lane]
+                             // world-aligned, or [WPIPE_TAPES] of those for the pipelined world-aligned adjoint
   void* adj = nullptr;       // [maxL][NADJ][B] scalar
-  void* wtapes = nullptr;    // [WPIPE_TAPES][maxL * NWT + NWF][B] scalar: the pipelined adjoint's tapes (null: in tape)
   void* wstk = nullptr;      // [WPIPE_TAPES + 1][wdepth][WSW][B] scalar: the warps' stacks of parent values
   int wdepth = 0;            // entries a system's stack holds at most (depth-first nesting of its branchings)
   void* gm_acc = nullptr;    // [maxL][B] scalar

@@ -43,7 +43,6 @@ template <class T> struct DevModel {
   int slots;     // world-aligned kernels with a global tape: slots of a warp's ring, 3 or 1 (no look-ahead)
   T* stk;        // world-aligned kernels: two stacks of parent values [2][tiles][wdepth][WSW][lane] (null: none)
   int wdepth;    // entries per stack
-  T* tapes;      // pipelined world-aligned adjoint: [WPIPE_TAPES][tile][tape words][lane]
   int sd;        // scalars of a system's stack in shared memory beside a global tape (0: in stk)
 };
 
@@ -53,8 +52,7 @@ template <class T> DevModel<T> dev_model(const sim_handle* h) {
                      (T)h->g[0], (T)h->g[1], (T)h->g[2], h->integrator, 0, 0,
                      h->replay == SIM_REPLAY_QUADRATIC, (T*)h->ctape, (T*)h->csys,
                      ContactParams<T>{(T)h->friction, (T)h->erp, h->pgs_iterations}, h->dt,
-                     h->state64 ? (double*)h->x64 : nullptr, h->prefetch > 0 ? 3 : 1, (T*)h->wstk, h->wdepth,
-                     (T*)(h->wtapes ? h->wtapes : h->tape), 0};
+                     h->state64 ? (double*)h->x64 : nullptr, h->prefetch > 0 ? 3 : 1, (T*)h->wstk, h->wdepth, 0};
 }
 
 extern __shared__ __align__(16) unsigned char g_smem[];

@@ -117,7 +117,7 @@ k_wbackward_pipe(DevModel<T> m, const T* __restrict__ ckpt, const T* __restrict_
         T* tape = s_tape + buf * TW * LANES + lane;
         return WSys<T>{s_prm + lane, meta_l, tape, s_adj + lane, nl, MS, NPRM_W, s_stk, tape + L * NWT * LANES};
       } else {
-        T* tape = m.tapes + (buf * units + unit) * TW * LANES + lane;
+        T* tape = m.tape + (buf * units + unit) * TW * LANES + lane;
         return WSys<T, true>{gprm, gmeta, tape, m.adj + (long long)unit * L * NWA * LANES + lane, nl, 1, NPRM,
                              m.sd ? s_stk : w_stack(m, warp, unit, lane), tape + L * NWT * LANES, links, s_ring,
                              m.slots > 1, lane};
