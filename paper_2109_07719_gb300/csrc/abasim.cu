@@ -424,7 +424,8 @@ int sim_create(const sim_model_desc* d, sim_handle** out) {
     h->friction = d->friction;
     h->erp = d->erp;
     h->pgs_iterations = d->pgs_iterations;
-    if (rc == SIM_OK) rc = alloc(&h->ctape, (size_t)CT_WARPS * maxL * NCT * Bpad * h->scalar, "contact tapes");
+    h->cwarps = contact_warps((long long)(Bpad / LANES), h->sms, h->precision == SIM_FP64);
+    if (rc == SIM_OK) rc = alloc(&h->ctape, (size_t)h->cwarps * maxL * NCT * Bpad * h->scalar, "contact tapes");
     if (rc == SIM_OK) rc = alloc(&h->csys, (size_t)NCS * Bpad * h->scalar, "contact record");
   }
   if (rc == SIM_OK) {

@@ -1,5 +1,5 @@
 // Rollout and adjoint kernels of models with contact spheres or joint limits (link-frame
-// step, tapes in global memory): CT_WARPS warps per 32-system tile.  The first warp runs
+// step, tapes in global memory): one to four warps per 32-system tile (contact_warps).  The first warp runs
 // the step; the warps share the columns of A = J M^-1 J^T, three to a test pass, and their
 // reverse in the adjoint, each with a contact tape of its own.
 //
@@ -29,6 +29,7 @@ template <class T> __device__ __forceinline__ CView<T> cview_of(const DevModel<T
 template <class T, class DT, bool ADJ>
 __device__ __forceinline__ int contact_step(const DevModel<T>& m, const Sys<T>& s, const CView<T>& cv, int warp, bool act,
                                             Col<const T> q, Col<const T> qd, Col<const T> tau_t, V3<T> g, bool* any) {
+  const int parts = blockDim.x / LANES;
   int nr = 0;
   if (warp == 0 && act) {
     aba_forward<T, DT, ADJ>(s, q, qd, tau_t, g);
@@ -36,7 +37,7 @@ __device__ __forceinline__ int contact_step(const DevModel<T>& m, const Sys<T>& 
   }
   *any = __syncthreads_or(nr > 0);
   if (*any) {
-    if (act) contact_columns<T, DT, T>(s, cv, warp, CT_WARPS);
+    if (act) contact_columns<T, DT, T>(s, cv, warp, parts);
     __syncthreads();
     if (nr > 0) contact_solve<T, DT, T>(s, cv, m.cp);
   }
@@ -61,6 +62,7 @@ template <class T, class DT>
 __device__ __forceinline__ void contact_adjoint_step(const DevModel<T>& m, const Sys<T>& s, const CView<T>& cv, int warp,
                                                      bool act, Col<const T> q, Col<const T> qd, Col<const T> tau_t,
                                                      Col<T> gq, Col<T> gqd, Col<T> gt, Col<T> gm, V3<T> g) {
+  const int parts = blockDim.x / LANES;
   bool any;
   const int nr = contact_step<T, DT, true>(m, s, cv, warp, act, q, qd, tau_t, g, &any);
   if (any) {
@@ -77,10 +79,12 @@ __device__ __forceinline__ void contact_adjoint_step(const DevModel<T>& m, const
       zero_accumulators(s, cv, B_OW);
     }
     __syncthreads();
-    if (act) contact_adjoint_columns<T, DT, T>(s, cv, warp, CT_WARPS);
+    if (act) contact_adjoint_columns<T, DT, T>(s, cv, warp, parts);
     __syncthreads();
-    if (act) contact_adjoint_sum(s, cv, contact_stride(m), warp, CT_WARPS);
-    __syncthreads();
+    if (parts > 1) {
+      if (act) contact_adjoint_sum(s, cv, contact_stride(m), warp, parts);
+      __syncthreads();
+    }
     if (nr > 0) contact_adjoint_finish<T, DT, T>(s, cv, m.dt, m.cp);
   }
   if (warp == 0 && act) {

@@ -47,7 +47,19 @@ constexpr int MAXC = SIM_MAX_CONTACTS;         // contact spheres per system
 constexpr int MAXL = SIM_MAX_LIMITS;           // limited joints per system
 constexpr int NROW = 3 * MAXC + MAXL;          // impulse rows: world x, y, z per contact, then limits
 constexpr int MAXPGS = SIM_MAX_PGS_ITERATIONS;  // Gauss-Seidel sweeps
-constexpr int CT_WARPS = 4;                    // warps of a contact kernel that share a system's test passes
+constexpr int CT_WARPS = 4;                    // warps of a contact kernel that share a system's test passes, at most
+
+// Warps per tile of a batch of `tiles` tiles.  An SM's registers hold eight of these warps:
+// four a tile as long as all tiles then run at once, in FP64 two as long as that holds, else
+// one.  Rollout + adjoint of 12 steps in ms with one, two and four warps a tile: quadrupeds
+// with feet down, 9728 (304 tiles on 152 SMs) in FP64 65.3, -, 50.6, in FP32 16.0, -, 14.7;
+// 12288 in FP64 65.5, 55.2, 69.4, in FP32 16.5, 15.6, 19.0; 20000 in FP64 70.0, -, 100.3, in
+// FP32 20.0, -, 27.4; 16384 chains past their limits in FP32 11.7, 12.9, 15.6; 12288
+// quadrupeds in the air in FP64 16.2, 16.3, 30.4.
+inline int contact_warps(long long tiles, int sms, bool fp64) {
+  const long long room = 8LL * sms;
+  return CT_WARPS * tiles <= room ? CT_WARPS : fp64 && 2 * tiles <= room ? 2 : 1;
+}
 
 // per-system contact record, [field][system]
 enum : int {

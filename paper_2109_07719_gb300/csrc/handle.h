@@ -41,7 +41,8 @@ struct sim_handle {
   int* status = nullptr;     // [B] by system
   int* sys_of_slot = nullptr;  // [B]
   unsigned* counter = nullptr;  // work-unit ticket of persistent launches
-  void* ctape = nullptr;     // [CT_WARPS][maxL][NCT][B] scalar, models with contact spheres or limits only
+  void* ctape = nullptr;     // [cwarps][maxL][NCT][B] scalar, models with contact spheres or limits only
+  int cwarps = 1;            // warps per tile of the contact kernels (contact_warps)
   void* csys = nullptr;      // [NCS][B] scalar, models with contact spheres only
   double friction = 0.8, erp = 0.2;
   int pgs_iterations = 20;

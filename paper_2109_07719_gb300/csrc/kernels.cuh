@@ -35,7 +35,7 @@ template <class T> struct DevModel {
   int persistent;
   int smem;
   int quadratic;
-  T* ctape;  // per-link contact tapes [CT_WARPS][tile][maxL][NCT][lane] (null: no contact spheres or limits)
+  T* ctape;  // per-link contact tapes [cwarps][tile][maxL][NCT][lane] (null: no contact spheres or limits)
   T* csys;   // per-system contact record [tile][NCS][lane]
   ContactParams<T> cp;
   double dt64;   // the time step in FP64
@@ -1132,7 +1132,7 @@ int launch_rollout(sim_handle* h, const void* q0, const void* qd0, const void* t
   int threads = h->block;
   if (h->ctape) {
     kern = rollout_contact_kernel<T, DT>();
-    threads = CT_WARPS * LANES;
+    threads = h->cwarps * LANES;
   } else {
     bool piped = false;  // the pipelined rollout, any precision
     if (h->all_chains && h->maxL <= PIPE_MAX_LINKS && !h->state64 &&
@@ -1204,7 +1204,7 @@ int launch_backward(sim_handle* h, const void* ckpt, const void* tau, int64_t T_
   int threads = h->block;
   if (h->ctape) {
     kern = backward_contact_kernel<T, DT>();
-    threads = CT_WARPS * LANES;
+    threads = h->cwarps * LANES;
   } else if constexpr (sizeof(T) == 4) {  // on-chip modes: FP32 storage only
     bool piped = false;
     if (k == 1 && T_ > 0 && h->all_chains &&
@@ -1261,7 +1261,7 @@ int launch_step_with_tape(sim_handle* h, const void* q, const void* qd, const vo
                           void* qd_out, void* tape, void* stream) {
   DevModel<T> m = dev_model<T>(h);
   m.tape = (T*)tape;
-  const int slots = h->ctape ? LANES : h->block, threads = h->ctape ? CT_WARPS * LANES : h->block;
+  const int slots = h->ctape ? LANES : h->block, threads = h->ctape ? h->cwarps * LANES : h->block;
   const int grid = (h->B + slots - 1) / slots;
   const RolloutKernel<T> kern = h->ctape ? rollout_contact_kernel<T, DT>() : k_rollout<T, DT, ST_GLOBAL>;
   kern<<<grid, threads, 0, S(stream)>>>(m, (const T*)q, (const T*)qd, (const T*)tau, 1LL, 1, (T*)nullptr,
