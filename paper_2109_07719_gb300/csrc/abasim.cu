@@ -376,6 +376,8 @@ int sim_create(const sim_model_desc* d, sim_handle** out) {
   cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
   cudaDeviceGetAttribute(&h->smem_limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
   h->smem_limit = std::max(0, h->smem_limit - kStaticSmem);
+  for (int t = 0; t < B; t += LANES)
+    h->load += (double)*std::max_element(nl.begin() + t, nl.begin() + std::min(B, t + LANES)) / maxL / std::max(1, h->sms);
   h->all_chains = !any_contact;
   h->unconstrained = !any_contact;
   h->all_revolute = !any_contact;

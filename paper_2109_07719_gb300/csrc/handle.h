@@ -52,6 +52,7 @@ struct sim_handle {
   int prefetch = 2;          // links ahead the world-aligned global-tape passes prefetch
   int last_storage = 0, last_storage_bwd = 0;
   int sms = 0;
+  double load = 0;           // the batch's tiles per SM, each by its links relative to the longest
   int smem_limit = 0;        // dynamic shared memory a launch may ask for, bytes
   bool all_chains = false;   // every system a serial chain of revolute joints (the pipelined adjoint)
   bool all_revolute = false; // every joint revolute and no contact spheres or limits

@@ -5,6 +5,7 @@
 #pragma once
 
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "contact.cuh"
@@ -902,15 +903,27 @@ inline int l1_carveout(const sim_handle* h, int slots_per_block, size_t bytes) {
   return (int)std::min(100LL, std::max(1LL, (100 * want + sm_smem - 1) / sm_smem));
 }
 
-// Whether a global-tape block of `bytes` with its warps' stacks in shared memory fits, with
-// as many blocks an SM as the batch has, up to two: blocks are sorted by length, so those
-// that wait for room run beside the end of the long ones (adjoint of 16384 trees of 2-64
-// links 257 us a step with the stacks in global memory and three blocks an SM, 168 with them
-// here and two).
-inline bool stacks_fit(const sim_handle* h, int slots_per_block, size_t bytes, int limit) {
+// Whether `blocks` blocks of `bytes` dynamic shared memory fit an SM.
+inline bool blocks_fit(const sim_handle* h, long long blocks, size_t bytes) {
+  return blocks * ((long long)bytes + kStaticSmem + 1024) <= (long long)h->smem_limit + kStaticSmem + 1024;
+}
+
+// How many global-tape blocks an SM should hold before the warps' stacks share its memory
+// with them.  As many as the batch has, up to two: blocks are sorted by length, so those that
+// wait for room run beside the end of the long ones (FP32 adjoint of 16384 trees of 2-64 links
+// 257 us a step with the stacks in global memory and three blocks an SM, 168 with them in
+// shared memory and two).  In FP64, whose arithmetic only the four schedulers' warps of an
+// SM keep busy together, up to four where the batch's links fill them (1.1: the short tiles
+// at the end cost less than the stacks): rollouts of 40000 such trees over 8 steps 20.4 ms
+// with two blocks, 12.4 with five.
+inline long long blocks_wanted(const sim_handle* h, int slots_per_block) {
   const long long units = (h->B + slots_per_block - 1) / slots_per_block, sms = std::max(1, h->sms);
-  const long long blocks = std::min(2LL, (units + sms - 1) / sms);
-  return blocks * ((long long)bytes + kStaticSmem + 1024) <= (long long)limit + kStaticSmem + 1024;  // the SM's
+  const long long few = std::min(2LL, (units + sms - 1) / sms);
+  if (h->precision != SIM_FP64) return few;
+  return std::max(few, std::min(4LL, (long long)std::ceil(h->load * LANES / slots_per_block / 1.1)));
+}
+inline bool stacks_fit(const sim_handle* h, int slots_per_block, size_t bytes) {
+  return blocks_fit(h, blocks_wanted(h, slots_per_block), bytes);
 }
 
 // Scalars per tile of a world-aligned kernel's working state (w_smem_per_tile's, without
@@ -946,7 +959,11 @@ int choose_w(sim_handle* h, K k_on, K k_off, bool bwd, bool* onchip, int* thread
   }
   if (need(false, tiles) > (size_t)limit) *slots = 1;
   *sd = h->wdepth * WSW;
-  if (!stacks_fit(h, tiles * LANES, need(false, tiles), limit)) *sd = 0;
+  if (!stacks_fit(h, tiles * LANES, need(false, tiles))) *sd = 0;
+  // a batch that wants more than two blocks an SM (FP64) rather stages without looking ahead
+  // than run fewer (rollouts of 40000 FP64 trees 15.7 ms with three blocks, 12.4 with five)
+  const long long wanted = blocks_wanted(h, tiles * LANES);
+  if (wanted > 2 && *sd == 0 && !blocks_fit(h, wanted, need(false, tiles))) *slots = 1;
   const size_t need_on = need(true, h->block / LANES), need_off = need(false, tiles);
   if (need_off > (size_t)limit) return fail(h, SIM_EUNSUPPORTED, "the working state does not fit in shared memory");
   e = allow_smem(h, (const void*)k_off);
@@ -1040,7 +1057,14 @@ int launch_wbackward_pipe(sim_handle* h, const void* ckpt, const void* tau, int6
     return (size_t)wpipe_smem_per_tile(h->maxL, nx, h->nv_max, on, on ? h->wdepth * WSW : m.sd, fr, np, m.slots, k > 1) *
            LANES * sizeof(T);
   };
-  const bool onchip = need(true, 1) <= (size_t)limit && (!fr || tiles <= sms);
+  // On chip where one tile's memory fits; a free base while every tile has an SM to itself,
+  // FP64 (whose on-chip blocks leave room for one or two an SM) while all tiles run at once:
+  // adjoint of 20000 7-link chains over 8 steps 4.1 ms on chip, 2.6 with global tapes, with
+  // segments of four 7.5 and 3.7; 10000 3-link chains 0.74 and 0.58, 6000 (one round) 0.39 and
+  // 0.47.
+  bool onchip = need(true, 1) <= (size_t)limit && (!fr || tiles <= sms);
+  if (onchip && sizeof(T) == 8 && tiles > sms)
+    onchip = blocks_fit(h, (long long)std::ceil(h->load / 1.1), need(true, 2));
   // Producers: three while every tile has an SM to itself (4096 7-link chains, on chip: 6.3
   // us a step with one, 5.4, 5.0 with three; 1024 humanoids, global tapes: 32.8, 30.1, 29.9;
   // 1000 FP64 trees of 2-20 links 379, 325, 277).  With more tiles than that the SMs are
@@ -1052,7 +1076,7 @@ int launch_wbackward_pipe(sim_handle* h, const void* ckpt, const void* tau, int6
   while (np > 1 && need(onchip, np) > (size_t)limit) --np;
   if (need(onchip, np) > (size_t)limit) m.slots = 1;
   m.sd = h->wdepth * WSW;
-  if (!stacks_fit(h, LANES, need(onchip, np), limit)) m.sd = 0;
+  if (!stacks_fit(h, LANES, need(onchip, np))) m.sd = 0;
   const size_t shm = need(onchip, np);
   if (shm > (size_t)limit) return fail(h, SIM_EUNSUPPORTED, "the working state does not fit in shared memory");
   const int threads = (np + 1) * LANES;
@@ -1151,7 +1175,12 @@ int launch_rollout(sim_handle* h, const void* q0, const void* qd0, const void* t
       if constexpr (sizeof(T) == 8) {  // FP64: the team rollout (wteam.cuh) where a tile fits a block
         const size_t team =
             (size_t)team_smem_per_tile(h->maxL, h->nq_max + h->nv_max, h->nv_max) * LANES * sizeof(T);
-        if (h->tape_space == SIM_TAPE_AUTO && h->maxL >= TEAM_MIN_LINKS && team <= (size_t)limit) {
+        // three links: while all tiles run at once (10000 systems 0.51 ms for 8 steps, pipelined
+        // 0.39; 9728, two blocks an SM, 0.28 and 0.32); longer chains at any batch size (20000
+        // 4-link ones 1.04 and 1.29)
+        const long long sms = std::max(1, h->sms), each = ((h->B + LANES - 1) / LANES + sms - 1) / sms;
+        if (h->tape_space == SIM_TAPE_AUTO && h->maxL >= TEAM_MIN_LINKS && team <= (size_t)limit &&
+            (h->maxL > TEAM_MIN_LINKS || blocks_fit(h, each, team))) {
           kern = wrollout_team_kernel<T>();
           st = ST_PIPE;
           shm = team;
@@ -1284,9 +1313,12 @@ int launch_jvp(sim_handle* h, const void* q, const void* qd, const void* tau, co
     DevModel<T> m = dev_model<T>(h);
     m.sd = h->wdepth * WSW;
     auto need = [&] { return (size_t)wjvp_smem_per_tile(h->nq_max, h->nv_max, m.sd) * LANES * sizeof(T); };
-    if (!stacks_fit(h, LANES, need(), limit)) m.sd = 0;
+    if (!stacks_fit(h, LANES, need())) m.sd = 0;
     const size_t shm = need();
-    if (shm <= (size_t)limit && (uintptr_t)work % 16 == 0) {
+    // with one block an SM and several rounds of them the dual numbers' eight blocks are faster
+    // (40000 trees of 2-64 links 8.75 ms against 7.66, 16384 of them 3.8 against 5.3)
+    const bool rounds = h->load > 3 && !blocks_fit(h, 2, shm);
+    if (shm <= (size_t)limit && !rounds && (uintptr_t)work % 16 == 0) {
       const auto kern = h->all_revolute ? k_wstep_jvp<T, false> : k_wstep_jvp<T, true>;
       e = allow_smem(h, (const void*)kern);
       if (e != cudaSuccess) return cuda_fail(h, e, "shared-memory opt-in");

@@ -68,18 +68,39 @@ def test_free_bases_replay(family, k):
     assert _agree(w, k, T=7)[1] == "floating_pipelined_global"
 
 
-@pytest.mark.parametrize("family,storage", [("chains", "aligned_pipelined_shared"), ("quadruped", "floating_pipelined_global")])
+@pytest.mark.parametrize("links,storage", [(3, "aligned_pipelined_shared"), (5, "aligned_pipelined_global"),
+                                           (0, "floating_pipelined_global")])
 @pytest.mark.parametrize("k", [1, 2])
-def test_more_tiles_than_sms(family, storage, k):
-    """Two producers (on chip) and one (global tapes)."""
-    w = wl.serial_chains(B=6000, n=5, T=1) if family == "chains" else wl.quadruped(B=6000, T=1)
+def test_more_tiles_than_sms(links, storage, k):
+    """Two producers (on chip while all tiles run at once) and one (global tapes)."""
+    w = wl.serial_chains(B=6000, n=links, T=1) if links else wl.quadruped(B=6000, T=1)
     assert _agree(w, k)[1] == storage
+
+
+@pytest.mark.parametrize("B", [10000, 26000])
+def test_many_fp64_trees(B):
+    """Stacks in global memory and (26000) no look-ahead, so that four blocks fit an SM."""
+    w = _trees([[(i - 1) // 2 for i in range(63)]] * 8)
+    w.model = w.model.subset(np.arange(B) % 8)
+    w.q0, w.qd0, w.tau_mask = [np.ascontiguousarray(x[:, np.arange(B) % 8]) for x in (w.q0, w.qd0, w.tau_mask)]
+    w.tau_sigma = 0.0
+    big, _ = _run(w, T=2)
+    w8 = _trees([[(i - 1) // 2 for i in range(63)]] * 8)
+    w8.tau_sigma = 0.0
+    small, _ = _run(w8, T=2)
+    check("qT", big[0][:, -8:], small[0][:, (np.arange(B) % 8)[-8:]], 1e-12)
+    check("qdT", big[1][:, -8:], small[1][:, (np.arange(B) % 8)[-8:]], 1e-12)
 
 
 @pytest.mark.parametrize("n", [3, 9, 10, 14])    # 9: the longest whose tile fits a block; 14: the pipelined rollout's last
 @pytest.mark.parametrize("T", [0, 1, 2, 5])
 def test_fp64_chain_rollouts(n, T):
     _agree(wl.serial_chains(B=37, n=n, T=1, precision="fp64"), T=T)
+
+
+def test_three_link_chains_of_many_tiles():
+    """The pipelined rollout where the team's blocks would run in turns."""
+    _agree(wl.serial_chains(B=10000, n=3, T=1, precision="fp64"), T=2)
 
 
 @pytest.mark.parametrize("persistent", [False, True])
