@@ -53,19 +53,22 @@ def flops_per_system_step(model, kind):
     return (tab["rev"] * n_rev + tab["rev_root"] * n_rev_root + tab["free_root"] * n_free) / model.n_systems
 
 
-def kernel_flops(model, storage, precision="fp32"):
+def kernel_flops(model, storage):
     """(rollout kernel, its FLOPs per system-step, adjoint kernel, its FLOPs per
     system-step) for the storage modes the last launches reported."""
     world = ("aligned", "floating")              # the world-aligned kernels
     fwd_world, bwd_world = storage[0].startswith(world), storage[1].startswith(world)
     kf = "k_wrollout" if fwd_world else ("k_rollout_pipe" if storage[0] == "pipelined" else "k_rollout")
-    if storage[0] == "pipelined" and precision == "fp64" and int(model.nv_max) >= 3:
+    if storage[0] == "pipelined_team":
         kf, fwd_world = "k_wrollout_team", True  # the same step, shared by four warps
     kb = ("k_wbackward_pipe" if "_pipelined" in storage[1] else "k_wbackward") if bwd_world else \
         ("k_backward_pipe" if storage[1] == "pipelined" else "k_backward")
     ff = flops_per_system_step(model, "wfwd" if fwd_world else "fwd")
     fb = (flops_per_system_step(model, "wrec") + flops_per_system_step(model, "wadj")) if bwd_world else \
         (flops_per_system_step(model, "fwd") + flops_per_system_step(model, "adj"))
+    constrained = getattr(model, "contact", None) is not None or getattr(model, "limits", None) is not None
+    if constrained:                              # the count covers the ABA and its adjoint alone
+        kf, kb = "k_rollout_contact", "k_backward_contact"
     return kf, ff, kb, fb
 
 
@@ -293,7 +296,7 @@ def run_ours(args):
                       qd0.cpu().pin_memory())
     if rank != 0:
         return None
-    kf, f_fwd, kb, f_bwd = kernel_flops(m, storage, args.precision)
+    kf, f_fwd, kb, f_bwd = kernel_flops(m, storage)
     adj_flops = B * T * f_bwd
     adj_s = float(np.mean(adj_ms)) / 1e3
     clocks = _clocks_summary(samples)

@@ -309,7 +309,8 @@ int sim_set_tape_space(sim_handle* h, int32_t space);
  * kernels, 4 the world-aligned kernels with the tape on chip, 5 the world-aligned
  * kernels with the tape in global memory, 6 / 7 the pipelined world-aligned adjoint
  * with its tapes on chip / in global memory, 8 - 11 the modes 4 - 7 for a model with
- * a free joint (AUTO only).  Either pointer may be NULL.  No device work. */
+ * a free joint (AUTO only), 12 the FP64 rollout of serial chains by four warps (AUTO
+ * only).  Either pointer may be NULL.  No device work. */
 int sim_last_storage(const sim_handle* h, int32_t* rollout_mode, int32_t* backward_mode);
 
 /* Look-ahead of the world-aligned kernels when their tape is in global memory: each

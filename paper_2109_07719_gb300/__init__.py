@@ -218,11 +218,12 @@ class Simulator:
 
     STORAGE = ("global", "hybrid", "shared", "pipelined", "aligned_shared", "aligned_global",
                "aligned_pipelined_shared", "aligned_pipelined_global", "floating_shared", "floating_global",
-               "floating_pipelined_shared", "floating_pipelined_global")
+               "floating_pipelined_shared", "floating_pipelined_global", "pipelined_team")
 
     def last_storage(self):
         """(rollout, backward) storage modes of the last launches: 'global', 'hybrid',
-        'shared', 'pipelined', the world-aligned kernels' 'aligned_shared' /
+        'shared', 'pipelined', 'pipelined_team' (FP64 rollouts of serial chains by four
+        warps), the world-aligned kernels' 'aligned_shared' /
         'aligned_global' and 'aligned_pipelined_shared' / 'aligned_pipelined_global',
         or 'floating_...' where they run a model with a floating base."""
         f, b = ctypes.c_int32(), ctypes.c_int32()

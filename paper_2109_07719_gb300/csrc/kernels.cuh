@@ -1153,6 +1153,7 @@ int launch_rollout(sim_handle* h, const void* q0, const void* qd0, const void* t
   int st = ST_GLOBAL;
   int rc = SIM_OK;
   RolloutKernel<T> kern = k_rollout<T, DT, ST_GLOBAL>;
+  bool team_ran = false;
   int threads = h->block;
   if (h->ctape) {
     kern = rollout_contact_kernel<T, DT>();
@@ -1185,7 +1186,7 @@ int launch_rollout(sim_handle* h, const void* q0, const void* qd0, const void* t
           st = ST_PIPE;
           shm = team;
           threads = TEAM * LANES;
-          piped = true;
+          piped = team_ran = true;
         }
       }
       if (piped) {
@@ -1206,7 +1207,7 @@ int launch_rollout(sim_handle* h, const void* q0, const void* qd0, const void* t
     }
   }
   if (rc != SIM_OK) return rc;
-  h->last_storage = st;
+  h->last_storage = team_ran ? 12 : st;
   int grid = 0;
   rc = launch_shape(h, kern, &grid, &m.persistent, shm, stream, threads, st == ST_PIPE || h->ctape ? LANES : threads);
   if (rc != SIM_OK) return rc;

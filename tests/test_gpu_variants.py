@@ -92,15 +92,16 @@ def test_many_fp64_trees(B):
     check("qdT", big[1][:, -8:], small[1][:, (np.arange(B) % 8)[-8:]], 1e-12)
 
 
-@pytest.mark.parametrize("n", [3, 9, 10, 14])    # 9: the longest whose tile fits a block; 14: the pipelined rollout's last
+@pytest.mark.parametrize("n", [3, 9, 10, 14])    # 9: the longest whose tile fits a block
 @pytest.mark.parametrize("T", [0, 1, 2, 5])
 def test_fp64_chain_rollouts(n, T):
-    _agree(wl.serial_chains(B=37, n=n, T=1, precision="fp64"), T=T)
+    storage = _agree(wl.serial_chains(B=37, n=n, T=1, precision="fp64"), T=T)
+    assert storage[0] == ("pipelined_team" if n <= 9 else "global")
 
 
 def test_three_link_chains_of_many_tiles():
     """The pipelined rollout where the team's blocks would run in turns."""
-    _agree(wl.serial_chains(B=10000, n=3, T=1, precision="fp64"), T=2)
+    assert _agree(wl.serial_chains(B=10000, n=3, T=1, precision="fp64"), T=2)[0] == "pipelined"
 
 
 @pytest.mark.parametrize("persistent", [False, True])
@@ -108,7 +109,7 @@ def test_three_link_chains_of_many_tiles():
 def test_fp64_chains_of_mixed_lengths(persistent, integrator):
     w = _trees([list(range(-1, 2 + i % 7)) for i in range(5000)])   # 3 to 9 links
     w.model = w.model.with_damping(3)
-    assert _agree(w, 2, 3, persistent, integrator)[0] == "pipelined"
+    assert _agree(w, 2, 3, persistent, integrator)[0] == "pipelined_team"
 
 
 @pytest.mark.parametrize("k", [1, 2])
