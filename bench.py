@@ -304,7 +304,7 @@ def run_ours(args):
     line = {
         "metric": METRIC, "value": value, "unit": "env-steps/s", "n_gpus": ws, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": step_ms, "higher_is_better": True, "scaling": "weak",
-        "vs_baseline": None, "dtype": {"fp64": "f64", "fp32": "f32", "fp32_d64": "f32+f64"}[args.precision],
+        "vs_baseline": None, "dtype": {"fp64": "f64", "fp32": "f32", "fp32_d64": "f32+f32x2"}[args.precision],
         "data": "synthetic",
         "config": {"workload": m.name, "n_systems": B, "horizon": T, "dt": m.dt, "checkpoint_interval": k,
                    "precision": args.precision, "l2": "flushed between steps (256 MB write)",

@@ -20,7 +20,8 @@
  *   traj [T+1][nq_max+nv_max][B]         x^0 .. x^T (optional)
  * Scalars are double for SIM_FP64 and float for SIM_FP32 / SIM_FP32_D64. The
  * SIM_FP32_D64 mode runs the articulated-inertia solves (1/D, the rank-one update,
- * the free root's 6x6 solve) in pairs of floats of 48 significant bits.
+ * the free root's 6x6 solve) in pairs of floats of 48 significant bits, as exact as
+ * double there (every result is rounded to float) over float's range.
  * Per-link arrays (gmass, set_masses) follow the link order of the model
  * description (CSR by system).
  *
@@ -268,7 +269,7 @@ int sim_set_launch(sim_handle* h, int32_t threads, int32_t schedule);
  * forcing either fails with SIM_EUNSUPPORTED where it does not apply.
  * SIM_TAPE_ONE_WARP chooses like AUTO among the one-warp-per-tile kernels only (the
  * autotuner times both, as one or two lanes per system).  Models with contact spheres
- * or joint limits always run with the tape in global memory, four warps per tile.
+ * or joint limits always run with the tape in global memory, one to four warps per tile.
  * Results do not depend on the choice beyond rounding. */
 #define SIM_TAPE_AUTO 0
 #define SIM_TAPE_GLOBAL 1

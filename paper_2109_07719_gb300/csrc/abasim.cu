@@ -621,7 +621,7 @@ int sim_set_state_accumulation(sim_handle* h, int32_t fp64) {
   if (!h) return SIM_EINVAL;
   if (fp64 != 0 && fp64 != 1) return fail(h, SIM_EINVAL, "state accumulation flag must be 0 or 1");
   if (fp64 && h->precision != SIM_FP32_D64)
-    return fail(h, SIM_EUNSUPPORTED, "FP64 state accumulation applies to the FP32 + FP64 D-solve mode");
+    return fail(h, SIM_EUNSUPPORTED, "FP64 state accumulation applies to the mixed mode (FP32 with 48-bit D-solves)");
   if (fp64 && !h->x64) {
     cudaError_t e = cudaMalloc(&h->x64, (size_t)(h->nq_max + h->nv_max) * h->B * sizeof(double));
     if (e != cudaSuccess) {

@@ -49,7 +49,7 @@ struct sim_handle {
   int schedule = SIM_SCHED_GRID;
   int tape_space = SIM_TAPE_AUTO;
   int replay = SIM_REPLAY_SEGMENT;
-  int prefetch = 2;          // links ahead the world-aligned global-tape passes prefetch
+  int prefetch = 2;          // 0: the world-aligned global-tape passes stage records without looking ahead
   int last_storage = 0, last_storage_bwd = 0;
   int sms = 0;
   double load = 0;           // the batch's tiles per SM, each by its links relative to the longest

@@ -40,9 +40,9 @@ template <class T> struct DevModel {
   T* csys;   // per-system contact record [tile][NCS][lane]
   ContactParams<T> cp;
   double dt64;   // the time step in FP64
-  double* x64;   // FP64 running state [nq_max + nv_max][B] of the rollout (null: off; FP32 + FP64 D only)
+  double* x64;   // FP64 running state [nq_max + nv_max][B] of the rollout (null: off; the mixed mode only)
   int slots;     // world-aligned kernels with a global tape: slots of a warp's ring, 3 or 1 (no look-ahead)
-  T* stk;        // world-aligned kernels: two stacks of parent values [2][tiles][wdepth][WSW][lane] (null: none)
+  T* stk;        // world-aligned kernels: a warp's stack of parent values [WPIPE_TAPES + 1][tiles][wdepth][WSW][lane] (null: none)
   int wdepth;    // entries per stack
   int sd;        // scalars of a system's stack in shared memory beside a global tape (0: in stk)
 };
@@ -999,10 +999,9 @@ int choose_w(sim_handle* h, K k_on, K k_off, bool bwd, bool* onchip, int* thread
 // The world-aligned path applies to models without contact spheres or limits whose
 // state and input streams fit a block's shared memory: under SIM_TAPE_ALIGNED (all
 // joints revolute), or under SIM_TAPE_AUTO unless the link-frame two-warp rollout of
-// serial chains applies.  Floating bases take it under SIM_TAPE_AUTO: when they moved here
-// from the link-frame one-warp kernels, rollout + adjoint of 8192 quadrupeds over 60 steps
-// in the mixed mode went from 15.6 to 11.3 ms (now 3.4), of 1024 humanoids over 60 steps in
-// FP32 from 10.95 to 4.4 (now 3.5).
+// serial chains applies.  Floating bases take it under SIM_TAPE_AUTO: on the link-frame
+// one-warp kernels rollout + adjoint of 8192 quadrupeds over 60 steps in the mixed mode took
+// 15.5 ms, here 3.4; of 1024 humanoids over 60 steps in FP32 10.9 and 3.5.
 template <class T, class DT>
 bool use_aligned(const sim_handle* h, bool rollout) {
   const bool fr = !h->all_revolute;
@@ -1041,8 +1040,9 @@ int launch_wrollout(sim_handle* h, const void* q0, const void* qd0, const void* 
 }
 
 // The pipelined world-aligned adjoint (k = 1, or segment replay: 1500 trees of 2-40 links
-// with k = 8 went from 168 us a step, replay, recompute and adjoint in one warp, to 116): one consumer warp and np producer warps per
-// 32-system tile, their tapes on chip when they fit a block, else in global memory.
+// with k = 8 took 168 us a step with replay, recompute and adjoint in one warp, 116 so): one
+// consumer warp and np producer warps per 32-system tile, their tapes on chip or in global
+// memory.
 template <class T, class DT>
 int launch_wbackward_pipe(sim_handle* h, const void* ckpt, const void* tau, int64_t T_, int k, const void* gqT,
                           const void* gqdT, const void* gtraj, void* gq0, void* gqd0, void* gtau, void* gmass,

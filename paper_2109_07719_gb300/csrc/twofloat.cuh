@@ -1,14 +1,19 @@
 // A number held as the unevaluated sum of two floats, h + l with |l| <= ulp(h) / 2: 48
 // significant bits out of FP32 instructions, by the error-free transformations of Dekker
 // (1971) and Knuth (The Art of Computer Programming 2, 4.2.2).  The mixed mode's D-solves
-// run in it.  They ran in double, whose instructions cost a warp 64 cycles each on this
-// chip's half-lane-per-cycle FP64 units: 140 of them (the rank-one update of the
-// articulated inertia with its 42 conversions, 1/D and the products with it) were nearly
-// all of a link's step.  Rollout + adjoint of 8192 quadrupeds over 60 steps 9.2 -> 4.7 ms,
-// of 4096 7-link chains over 100 steps 6.5 -> 1.1 ms (with the implicit-form adjoint); the
-// errors against 64 bits are 0.66e-6, 0.63e-6 and, for 333 16-link chains, 0.81e-6 (in
-// double 0.68e-6, 0.63e-6, 0.85e-6).  Every use rounds its result to float from at least
-// 44 bits of its largest term.
+// run in it.  In double, an instruction costs a warp 64 cycles on this chip's
+// half-lane-per-cycle FP64 units, and the 140 of them a link (the rank-one update of the
+// articulated inertia with its 42 conversions, 1/D and the products with it) were nearly all
+// of its step: rollout + adjoint of 8192 quadrupeds over 60 steps 9.2 ms in double, 4.7 in
+// pairs; of 4096 7-link chains over 100 steps 6.5 and 1.1 (with the implicit-form adjoint).
+//
+// Precision: every use rounds its result to float from at least 44 bits of its largest term,
+// so it differs from double's in about one rounding of 2^20, and the errors against 64 bits
+// are double's (0.66e-6, 0.63e-6 and, for 333 16-link chains, 0.81e-6; in double 0.68e-6,
+// 0.63e-6, 0.85e-6).  Range: a pair has float's exponents.  Its low half is lost below 2^-101
+// of the largest term, where float's own rounding is all that is left of double's advantage;
+// products of several factors are formed one at a time so that none leaves float's range.
+// Masses scaled by 1e-33 to 1e32 give double's errors throughout (tests/mixed_scale.cpp).
 #pragma once
 
 #include "spatial.cuh"

@@ -34,7 +34,7 @@ __host__ __device__ __forceinline__ long long w_smem_per_tile(int maxL, int nx, 
          2LL * (nv + (bwd ? nx : 0));
 }
 
-// Stack `which` (0, or 1 for the second warp of the pipelined adjoint) of a tile's
+// Stack `which` (the warp's number in the pipelined adjoint, else 0) of a tile's
 // system at `lane` in the handle's global scratch (null when no system branches).
 template <class T>
 __device__ __forceinline__ T* w_stack(const DevModel<T>& m, int which, long long tile, long long lane) {

@@ -20,7 +20,7 @@
 // the previous segment.
 //
 // Why several producers: the implicit-form adjoint takes less time than the recompute
-// (468 against 736 operations a link), so with one producer the consumer waits; how many
+// (468 against 670 operations a link), so with one producer the consumer waits; how many
 // is the launch's choice (launch_wbackward_pipe).  The tapes, the adjoint record, the
 // model constants and the inputs live on chip when the block's shared memory holds them
 // (ONCHIP), else in global memory (the tapes in the handle's ring), staged by each warp.
